@@ -367,6 +367,19 @@ __device__ void block_sort_asc(uint64_t* s, int n) {
     }
 }
 
+// 64-bit integer to FP32, rounded to nearest even, without the conversion
+// instruction: 64-bit conversions run on the FP64 pipe, at 2 lanes per clock
+// and SM on this GPU (a window's table of 24k sums took 12k clocks to
+// convert).  The leading 32 bits, with every lower bit folded into the last
+// one, round as the whole does.
+__device__ __forceinline__ float u64_to_float(unsigned long long x) {
+    const unsigned hi = (unsigned)(x >> 32), lo = (unsigned)x;
+    if (hi == 0u) return __uint2float_rn(lo);
+    const int z = __clz((int)hi);
+    const unsigned lead = __funnelshift_l(lo, hi, z) | ((lo << z) != 0u ? 1u : 0u);
+    return __fmul_rn(__uint2float_rn(lead), __int_as_float((32 - z + 127) << 23));
+}
+
 // Fixed-point scale of a column: q = trunc(v * 2^f) with 2^f = sc1 * sc2
 // (two exact power-of-two factors, each representable in FP32).
 struct FixScale {
@@ -385,13 +398,23 @@ struct FixScale {
     }
     __device__ __forceinline__ unsigned long long q(float aik, float akj) const {
         const float v = __fmul_rn(aik, akj);  // the FP32 product
-        return __float2ull_rz(__fmul_rn(__fmul_rn(v, sc1), sc2));
+        return qv(v);
     }
-    __device__ __forceinline__ unsigned long long qv(float v) const {  // v: an FP32 product
-        return __float2ull_rz(__fmul_rn(__fmul_rn(v, sc1), sc2));
+    // v: an FP32 product, 0 <= v < 2^(62 - f).  The significand is shifted
+    // into place with 32-bit shifts; the scaled conversion is the same number
+    // but runs on the FP64 pipe (see u64_to_float).  Products below 2^-126
+    // are 0 for f <= 100 and take the conversion otherwise.
+    __device__ __forceinline__ unsigned long long qv(float v) const {
+        if (f > 100) return __float2ull_rz(__fmul_rn(__fmul_rn(v, sc1), sc2));
+        const unsigned bits = __float_as_uint(v);
+        const unsigned lead = (bits << 8) | 0x80000000u;               // 24 significant bits on top
+        const int r = 190 - f - (int)((bits << 1) >> 24);              // (lead : 0) >> r, r >= 2
+        const unsigned hi = __funnelshift_rc(lead, 0u, r);
+        const unsigned lo = __funnelshift_rc(__funnelshift_rc(0u, lead, r), 0u, max(r - 32, 0));
+        return ((unsigned long long)hi << 32) | lo;
     }
     __device__ __forceinline__ float value(unsigned long long x) const {
-        return __fmul_rn(__fmul_rn(__ull2float_rn(x), is1), is2);
+        return __fmul_rn(__fmul_rn(u64_to_float(x), is1), is2);
     }
 };
 
