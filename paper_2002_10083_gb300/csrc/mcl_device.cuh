@@ -390,7 +390,8 @@ struct FixScale {
         int e = 0;
         frexp(s > 0.0 ? s * (1.0 + 1.0 / 1048576.0) : 1.0, &e);  // s (with margin) < 2^e
         f = 62 - e;
-        const int f1 = max(-126, min(127, f)), f2 = max(-126, min(127, f - f1));
+        // both factors and their inverses are normal numbers
+        const int f1 = max(-126, min(126, f)), f2 = max(-126, min(126, f - f1));
         sc1 = pow2(f1);
         sc2 = pow2(f2);
         is1 = pow2(-f1);
