@@ -220,7 +220,8 @@ mcl_status mcl_symbolic(mcl_ctx* ctx, const mcl_csc* A, int64_t* flops, int64_t*
  *                        symbolic pass, 1 the flops bound min(flops_j, span_j),
  *                        3 Cohen's estimate (mcl_cohen_estimate)
  *   2 MCL_OPT_CONF_MASK  bit mask of numeric-pass configurations (bit 0:
- *                        small CTA and window, bit 1: large; not 0)
+ *                        small CTA and window, bit 1: large, and a sum per
+ *                        row for columns dense in their span; not 0)
  *   3 MCL_OPT_VALIDATE   1 (default) validate inputs
  *   4 MCL_OPT_EST_SCALE  multiply every size estimate by value/1000 (1000 =
  *                        unchanged); a deliberate mis-estimate exercises the

@@ -29,7 +29,7 @@ struct mcl_ctx {
     void* user = nullptr;
     char err[512] = {0};
     // scratch
-    Buf flops, colsum, rlo, rhi, cap, off, est, bucket, work, kept, chaos, bnnz, tmp_row, tmp_val,
+    Buf flops, colsum, bsum, rlo, rhi, cap, off, est, bucket, work, kept, chaos, bnnz, tmp_row, tmp_val,
         cursors, scan, ctr, active, bucket_row, woff, comp_off, comp_of_col, comp_bits,
         comp_active;
     size_t bucket_budget = (size_t)32 << 30;  // bytes of product buckets (large config)
@@ -63,7 +63,8 @@ struct mcl_ctx {
     uint64_t cohen_seed = 2002;
     Buf cohen_m, cohen_e;
     // inner-dimension split
-    Buf split_bsum, split_cnt, split_scratch;
+    Buf split_cnt, split_scratch;
+    Buf spill;  // candidates of the direct configuration
 };
 
 namespace {
@@ -174,6 +175,8 @@ ExpandBuffers buffers(mcl_ctx* c) {
     ExpandBuffers b{};
     b.flops = (int64_t*)c->flops.p;
     b.colsum = (double*)c->colsum.p;
+    b.bsum = (double*)c->bsum.p;
+    b.spill = (uint64_t*)c->spill.p;
     b.rlo = (int32_t*)c->rlo.p;
     b.rhi = (int32_t*)c->rhi.p;
     b.cap = (int64_t*)c->cap.p;
@@ -201,6 +204,7 @@ ExpandBuffers buffers(mcl_ctx* c) {
 mcl_status ensure_columns(mcl_ctx* c, int64_t n, cudaStream_t s) {
     const size_t n1 = (size_t)n + 1;
     bool ok = ensure(c, c->flops, n1 * 8, s) && ensure(c, c->colsum, n1 * 8, s) &&
+              ensure(c, c->bsum, n1 * 8, s) &&
               ensure(c, c->rlo, n1 * 4, s) &&
               ensure(c, c->rhi, n1 * 4, s) && ensure(c, c->cap, n1 * 8, s) &&
               ensure(c, c->off, n1 * 8, s) && ensure(c, c->est, n1 * 8, s) &&
@@ -235,6 +239,24 @@ int max_numeric_grid(mcl_ctx* c, const PruneParams& pp) {
     }
     int gs = symbolic_grid(c->num_sms);
     return g > gs ? g : gs;
+}
+
+// Bit 0 of the mask allows the small configuration, bit 1 the other two.
+bool conf_on(const mcl_ctx* c, int q) { return (c->conf_mask >> (q == 0 ? 0 : 1)) & 1; }
+
+// b with the product buckets of configuration q: bytes of them shared by g CTAs.
+ExpandBuffers with_buckets(mcl_ctx* c, const ExpandBuffers& b, int q, int g, size_t bytes) {
+    ExpandBuffers bq = b;
+    bq.bucket_row = nullptr;
+    bq.woff = nullptr;
+    bq.bucket_cap = 0;
+    if (q != 0 && bytes > 0) {
+        bq.bucket_row = (int32_t*)c->bucket_row.p;
+        bq.woff = (int32_t*)c->woff.p;
+        bq.bucket_cap = (int64_t)(bytes / ((size_t)g * 8));
+        if (bq.bucket_cap > (int64_t)1 << 30) bq.bucket_cap = (int64_t)1 << 30;  // int32 positions
+    }
+    return bq;
 }
 
 }  // namespace
@@ -299,7 +321,7 @@ void mcl_destroy(mcl_ctx* c) {
                   &c->bucket, &c->work,   &c->kept,    &c->chaos,   &c->bnnz, &c->tmp_row,
                   &c->tmp_val, &c->cursors, &c->scan,  &c->ctr,     &c->active, &c->mlp_w,
                   &c->mlp_norm, &c->colmax, &c->feats, &c->prev_logcf, &c->cohen_m, &c->cohen_e,
-                  &c->split_bsum, &c->split_cnt, &c->split_scratch,
+                  &c->bsum, &c->spill, &c->split_cnt, &c->split_scratch,
                   &c->iter_dev};
     for (Buf* b : all) dev_free(c, b->p, 0);
     cudaDeviceSynchronize();
@@ -407,9 +429,12 @@ static mcl_status expand_impl(mcl_ctx* c, const mcl_csc* A, const mcl_params* pr
     b.cur_stride = (max_deg + 31) & ~31;
     if (b.cur_stride < 32) b.cur_stride = 32;
     const int grid_max = max_numeric_grid(c, pp);
-    if (!ensure(c, c->cursors, (size_t)grid_max * 6 * b.cur_stride * 4, s))
+    if (!ensure(c, c->cursors, (size_t)grid_max * 6 * b.cur_stride * 4, s) ||
+        !ensure(c, c->spill, direct_spill_bytes(direct_grid(pp.ksel, c->num_sms)), s))
         return fail(c, MCL_ERR_OOM, "cursor scratch allocation failed");
     b.cursors = (int32_t*)c->cursors.p;
+    b.spill = (uint64_t*)c->spill.p;
+    launch_bsum(Av, b.colsum, b.bsum, s);
     // ---- size estimate ----
     const int sizing =
         c->sizing >= 0 ? c->sizing : (prm->use_estimator && !c->run_exact ? 2 : 0);
@@ -451,28 +476,23 @@ static mcl_status expand_impl(mcl_ctx* c, const mcl_csc* A, const mcl_params* pr
     int used = 0;
     auto run_numeric = [&](const ExpandBuffers& bb) -> mcl_status {
         launch_binning(Av, pp, bb, c->conf_mask, s);
+        // product buckets for multi-window columns (optional: without them the windows
+        // walk per-source cursors); the two configurations run one after the other and
+        // share them
+        size_t bkt_bytes = 0;
+        if (conf_on(c, CONF_LARGE)) {
+            const int64_t g = numeric_grid(CONF_LARGE, pp, c->num_sms);
+            const int64_t gw = g > grid_max ? g : grid_max;
+            int64_t capb = (int64_t)(c->bucket_budget / ((size_t)g * 8));
+            if (capb > (int64_t)c->hctr->max_flops) capb = (int64_t)c->hctr->max_flops;
+            if (capb >= 1024 && ensure(c, c->bucket_row, (size_t)(g * capb * 8), s) &&
+                ensure(c, c->woff, (size_t)gw * 2 * (WINDOW_MAX + 1) * 4, s))
+                bkt_bytes = (size_t)(g * capb * 8);
+        }
         for (int q = NCONF - 1; q >= 0; --q) {
-            if (!((c->conf_mask >> q) & 1)) continue;
+            if (!conf_on(c, q)) continue;
             const int g = numeric_grid(q, pp, c->num_sms);
-            ExpandBuffers bq = bb;
-            bq.bucket_row = nullptr;
-            bq.woff = nullptr;
-            bq.bucket_cap = 0;
-            if (q == NCONF - 1) {
-                // product buckets for multi-window columns of the large configuration
-                // (optional: without them the windows walk per-source cursors)
-                const int64_t maxf = (int64_t)c->hctr->max_flops;
-                int64_t capb = (int64_t)(c->bucket_budget / ((size_t)g * 8));
-                if (capb > maxf) capb = maxf;
-                if (capb > (int64_t)1 << 30) capb = (int64_t)1 << 30;  // int32 bucket positions
-                if (capb >= 1024 && ensure(c, c->bucket_row, (size_t)g * capb * 8, s) &&
-                    ensure(c, c->woff, (size_t)g * 2 * (WINDOW_MAX + 1) * 4, s)) {
-                    bq.bucket_row = (int32_t*)c->bucket_row.p;
-                    bq.woff = (int32_t*)c->woff.p;
-                    bq.bucket_cap = capb;
-                }
-            }
-            launch_numeric(q, Av, pp, bq, g, s);
+            launch_numeric(q, Av, pp, with_buckets(c, bb, q, g, bkt_bytes), g, s);
             ++used;
         }
         return check_launch(c, "numeric");
@@ -688,10 +708,10 @@ mcl_status mcl_expand_split(mcl_ctx* c, const mcl_csc* A, const mcl_params* prm,
     stride = (stride + 31) & ~31ll;
     const int grid_cap = 4 * c->num_sms;
     const size_t n1 = (size_t)n + 1;
-    if (!ensure(c, c->split_bsum, n1 * 8, s) || !ensure(c, c->split_cnt, n1 * 8, s) ||
+    if (!ensure(c, c->split_cnt, n1 * 8, s) ||
         !ensure(c, c->split_scratch, (size_t)grid_cap * 6 * stride * 8, s))
         return fail(c, MCL_ERR_OOM, "split scratch allocation failed");
-    double* bsum = (double*)c->split_bsum.p;
+    double* bsum = b.bsum;
     int64_t* cnt = (int64_t*)c->split_cnt.p;
     launch_bsum(Av, b.colsum, bsum, s);
     mcl_merge_stats ms{};
@@ -1153,6 +1173,7 @@ static void static_iteration(mcl_ctx* c, const mcl_params* prm, const PruneParam
     launch_active_from_comp(n, (const int32_t*)c->comp_of_col.p, (const uint8_t*)c->comp_active.p,
                             (uint8_t*)c->active.p, s);
     launch_colstats(Av, pp, b, c->num_sms, s);
+    launch_bsum(Av, b.colsum, b.bsum, s);
     const int grid_max = max_numeric_grid(c, pp);
     if (sizing == 1) {
         launch_est_from_flops(Av, b, s);
@@ -1174,16 +1195,9 @@ static void static_iteration(mcl_ctx* c, const mcl_params* prm, const PruneParam
     launch_staging_guard(b.ctr, cap, s);
     launch_binning(Av, pp, b, c->conf_mask, s);
     for (int q = NCONF - 1; q >= 0; --q) {
-        if (!((c->conf_mask >> q) & 1)) continue;
+        if (!conf_on(c, q)) continue;
         const int g = numeric_grid(q, pp, c->num_sms);
-        ExpandBuffers bq = b;
-        if (q == NCONF - 1 && c->bucket_row.p) {
-            bq.bucket_row = (int32_t*)c->bucket_row.p;
-            bq.woff = (int32_t*)c->woff.p;
-            bq.bucket_cap = (int64_t)(c->bucket_row.bytes / ((size_t)g * 8));
-            if (bq.bucket_cap > (int64_t)1 << 30) bq.bucket_cap = (int64_t)1 << 30;
-        }
-        launch_numeric(q, Av, pp, bq, g, s);
+        launch_numeric(q, Av, pp, with_buckets(c, b, q, g, c->bucket_row.p ? c->bucket_row.bytes : 0), g, s);
     }
     launch_finalize_stats(n, b, s);
     launch_fill_inactive(Av, b.active, b.kept, s);
@@ -1218,13 +1232,14 @@ static mcl_status graph_prepare(mcl_ctx* c, const mcl_params* prm, const PrunePa
     int64_t stride = ((int64_t)pp.Krec + 31) & ~31ll;
     if (stride < 32) stride = 32;
     const int grid_max = max_numeric_grid(c, pp);
-    const int g1 = numeric_grid(NCONF - 1, pp, c->num_sms);
+    const int g1 = numeric_grid(CONF_LARGE, pp, c->num_sms);
     int64_t capb = (int64_t)pp.Krec * pp.Krec;
     const int64_t capb_max = (int64_t)(c->bucket_budget / ((size_t)g1 * 8));
     if (capb > capb_max) capb = capb_max;
     const size_t n1 = (size_t)n + 1;
     if (!ensure(c, c->tmp_row, (size_t)cap * 4 + 4, s) || !ensure(c, c->tmp_val, (size_t)cap * 4 + 4, s) ||
         !ensure(c, c->cursors, (size_t)grid_max * 6 * stride * 4, s) ||
+        !ensure(c, c->spill, direct_spill_bytes(direct_grid(pp.ksel, c->num_sms)), s) ||
         !ensure(c, c->comp_bits, (size_t)ncomp * 8, s))
         return fail(c, MCL_ERR_OOM, "graph replay scratch allocation failed");
     if (sizing == 2) {
@@ -1240,7 +1255,7 @@ static mcl_status graph_prepare(mcl_ctx* c, const mcl_params* prm, const PrunePa
             return fail(c, MCL_ERR_OOM, "estimator scratch allocation failed");
     }
     if (capb >= 1024 && ensure(c, c->bucket_row, (size_t)g1 * capb * 8, s) &&
-        ensure(c, c->woff, (size_t)g1 * 2 * (WINDOW_MAX + 1) * 4, s)) {
+        ensure(c, c->woff, (size_t)grid_max * 2 * (WINDOW_MAX + 1) * 4, s)) {
         // exact per-CTA capacity recorded in the buffer sizes
         c->bucket_row.bytes = (size_t)g1 * capb * 8;
     } else {

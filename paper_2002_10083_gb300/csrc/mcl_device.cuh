@@ -380,42 +380,49 @@ __device__ __forceinline__ float u64_to_float(unsigned long long x) {
     return __fmul_rn(__uint2float_rn(lead), __int_as_float((32 - z + 127) << 23));
 }
 
-// Fixed-point scale of a column: q = trunc(v * 2^f) with 2^f = sc1 * sc2
-// (two exact power-of-two factors, each representable in FP32).
+// Fixed-point scale of a column: q = trunc(v * 2^f), x = q * is1 * is2 (two
+// exact power-of-two factors, each a normal FP32 number).
 struct FixScale {
-    float sc1, sc2, is1, is2;
+    float is1, is2;
     int f;
     __device__ static float pow2(int e) { return __int_as_float((e + 127) << 23); }
     __device__ void init(double s) {
         int e = 0;
         frexp(s > 0.0 ? s * (1.0 + 1.0 / 1048576.0) : 1.0, &e);  // s (with margin) < 2^e
         f = 62 - e;
-        // both factors and their inverses are normal numbers
+        // both factors are normal numbers
         const int f1 = max(-126, min(126, f)), f2 = max(-126, min(126, f - f1));
-        sc1 = pow2(f1);
-        sc2 = pow2(f2);
         is1 = pow2(-f1);
         is2 = pow2(-f2);
     }
     __device__ __forceinline__ unsigned long long q(float aik, float akj) const {
-        const float v = __fmul_rn(aik, akj);  // the FP32 product
-        return qv(v);
+        return qv(__fmul_rn(aik, akj));  // the FP32 product
     }
-    // v: an FP32 product, 0 <= v < 2^(62 - f).  The significand is shifted
-    // into place with 32-bit shifts; the scaled conversion is the same number
-    // but runs on the FP64 pipe (see u64_to_float).  Products below 2^-126
-    // are 0 for f <= 100 and take the conversion otherwise.
+    // v: an FP32 product, 0 <= v < 2^(62 - f).  Scales outside the shifts'
+    // range take the conversion: f > 100 (products below 2^-126 may count) and
+    // f < -64 (a product may have overflowed to infinity, and saturates).
+    __device__ __forceinline__ bool plain() const { return f <= 100 && f >= -64; }
     __device__ __forceinline__ unsigned long long qv(float v) const {
-        if (f > 100) return __float2ull_rz(__fmul_rn(__fmul_rn(v, sc1), sc2));
+        return plain() ? qplain(v) : __float2ull_rz(ldexpf(v, f));
+    }
+    // The significand is shifted into place with 32-bit shifts; the scaled
+    // conversion is the same number but runs on the FP64 pipe (see
+    // u64_to_float).  Products below 2^-126 are 0: the shift is >= 90.
+    __device__ __forceinline__ unsigned long long qplain(float v) const {
         const unsigned bits = __float_as_uint(v);
-        const unsigned lead = (bits << 8) | 0x80000000u;               // 24 significant bits on top
-        const int r = 190 - f - (int)((bits << 1) >> 24);              // (lead : 0) >> r, r >= 2
+        const unsigned lead = (bits << 8) | 0x80000000u;  // 24 significant bits on top
+        const int r = 190 - f - (int)((bits << 1) >> 24);  // (lead : 0) >> r, r >= 2
         const unsigned hi = __funnelshift_rc(lead, 0u, r);
         const unsigned lo = __funnelshift_rc(__funnelshift_rc(0u, lead, r), 0u, max(r - 32, 0));
         return ((unsigned long long)hi << 32) | lo;
     }
     __device__ __forceinline__ float value(unsigned long long x) const {
         return __fmul_rn(__fmul_rn(u64_to_float(x), is1), is2);
+    }
+    // a lower bound of every sum whose value is >= v
+    __device__ __forceinline__ unsigned long long lower(float v) const {
+        const double x = ldexp((double)v * (1.0 - 1.0 / 1048576.0), f);
+        return x < 9.0e18 ? (unsigned long long)x : 9000000000000000000ull;
     }
 };
 

@@ -7,9 +7,11 @@
 
 namespace mcl {
 
-// Configurations of the fused numeric pass (mcl_numeric.cu): 0 = small CTA
-// and window for small columns, 1 = large CTA and window for the rest.
-constexpr int NCONF = 2;
+// Configurations of the fused numeric pass: 0 = small CTA and window for small
+// columns, 1 = large CTA and window (mcl_numeric.cu), CONF_DIRECT = a sum per
+// row for columns that are dense in their span (mcl_direct.cu).
+constexpr int NCONF = 3;
+constexpr int CONF_LARGE = 1, CONF_DIRECT = 2;
 constexpr int NZ = 8;                    // size classes per configuration
 constexpr int NBUCKET = NCONF * NZ;
 // device-side counters (one small block of memory per context)
@@ -32,7 +34,6 @@ struct DevCounters {
     int conf_ctr[NCONF];
     int work_ctr;
     int n_active;                    // components still iterating (graph replay)
-    int pad2;
 };
 
 enum : unsigned {
@@ -73,6 +74,7 @@ struct PruneParams {
 struct ExpandBuffers {
     int64_t* flops;     // [n]
     double* colsum;     // [n]   column sums of A (FP64)
+    double* bsum;       // [n]   column sums of A A (FP64)
     int32_t* rlo;       // [n]
     int32_t* rhi;       // [n]
     int64_t* cap;       // [n]   output capacity min(Krec, flops, span)
@@ -91,6 +93,7 @@ struct ExpandBuffers {
     int32_t* bucket_row;   // per CTA: bucket_cap (row, bits(a_ik * a_kj)) pairs (int2)
     int32_t* woff;         // per CTA: window offsets into the bucket (WINDOW_MAX + 1)
     int64_t bucket_cap;
+    uint64_t* spill;    // CONF_DIRECT, per CTA: candidates beyond the shared buffer
     int64_t* scan_tmp;  // tile sums
     int64_t scan_tmp_len;
     DevCounters* ctr;
@@ -119,8 +122,11 @@ void launch_est_from_flops(const CscView& A, const ExpandBuffers& b, cudaStream_
 void launch_binning(const CscView& A, const PruneParams& pp, const ExpandBuffers& b, int mask,
                     cudaStream_t s);
 int numeric_grid(int conf, const PruneParams& pp, int num_sms);
-size_t numeric_smem(int conf, const PruneParams& pp);
 constexpr int WINDOW_MAX = 4096;  // windows per column in bucket mode
+int direct_grid(int ksel, int num_sms);
+size_t direct_spill_bytes(int grid);
+void launch_direct(const CscView& A, const PruneParams& pp, const ExpandBuffers& b, int grid,
+                   cudaStream_t s);
 void launch_numeric(int conf, const CscView& A, const PruneParams& pp, const ExpandBuffers& b,
                     int grid, cudaStream_t s);
 void launch_compact(const CscView& A, const ExpandBuffers& b, const int64_t* colptr_out,

@@ -441,14 +441,23 @@ void launch_est_from_flops(const CscView& A, const ExpandBuffers& b, cudaStream_
 // binning: configuration by estimated size, size classes for LPT order
 // ---------------------------------------------------------------------------
 
+// Columns with a product for every DIRECT_SPARSE rows of their span take the
+// kernel with a sum per row; a span of one small window does not need it.
+// Clocks of an SM per column, hashed and direct: 1M-row spans 912k and 977k at
+// 200k products, 1.51M and 1.16M at 390k; 20k-row spans 51k and 55k at 6k
+// products, 65k and 60k at 12k.
+constexpr int DIRECT_MIN_SPAN = 2048, DIRECT_SPARSE = 4;
+
 // Configuration 0 (small CTA) takes columns whose estimate fits one small
-// window's value capacity and whose span needs few windows; configuration 1
-// takes the rest.  The size class orders work longest-first by flops_j.
+// window's value capacity and whose span needs few windows; CONF_DIRECT takes
+// the ones dense in their span (mcl_direct.cu), CONF_LARGE the rest.  The size
+// class orders work longest-first by flops_j.
 __device__ __forceinline__ int bucket_of(int64_t est, int64_t flops, int span, int mask,
                                          int small_max) {
-    int c = 1;
+    int c = CONF_LARGE;
     if ((mask & 1) && est <= small_max && span <= 8 * 16384) c = 0;
     if (!(mask & 2)) c = 0;
+    if ((mask & 2) && span > DIRECT_MIN_SPAN && flops * DIRECT_SPARSE >= span) c = CONF_DIRECT;
     int64_t f = flops >> 12;
     const int lg = f > 0 ? 63 - __clzll((long long)f) : 0;
     const int z = NZ - 1 - (lg < NZ - 1 ? lg : NZ - 1);

@@ -36,3 +36,44 @@ def test_scaled_input_gives_the_same_iteration(ctx, k):
     out, ch = ctx.expand(_dev(synth.CSC(A.n, A.colptr, A.rowidx, A.val * 2.0 ** k)), prm)
     assert torch.equal(out.colptr, ref.colptr) and torch.equal(out.rowidx, ref.rowidx)
     assert torch.equal(out.val.view(torch.int32), ref.val.view(torch.int32)) and ch == ch_ref
+
+
+def _random(n, d, seed, zeros=False):
+    """About d entries per column at random rows; with zeros, a third of the values are 0 or
+    so small that their products are truncated to 0 (they still are entries of A A)."""
+    g = torch.Generator().manual_seed(seed)
+    key = torch.unique(torch.randint(n * n, (n * d,), generator=g))
+    col, row = key // n, key % n
+    val = torch.exp(torch.randn(key.numel(), generator=g))
+    if zeros:
+        u = torch.rand(key.numel(), generator=g)
+        val = torch.where(u < 0.2, torch.zeros(()), torch.where(u < 0.35, torch.tensor(1e-30), val))
+    colptr = torch.zeros(n + 1, dtype=torch.int64)
+    colptr[1:] = torch.cumsum(torch.bincount(col, minlength=n), 0)
+    from paper_2002_10083_gb300 import mcl
+    return mcl.DeviceCSC(n, colptr.cuda(), row.int().cuda(), val.cuda())
+
+
+# rows of a direct window: 10,240; one window, its edges, several; products per source and
+# window on both sides of the bucket rule; a candidate buffer smaller and larger than a column
+@pytest.mark.parametrize("n,d,K,theta,zeros,budget", [
+    (2049, 40, 50, 1e-3, False, 32 << 30), (10240, 60, 300, 1e-4, False, 32 << 30),
+    (10241, 60, 1100, 1e-4, True, 32 << 30), (20481, 80, 4096, 0.0, True, 32 << 30),
+    (31000, 100, 1100, 1e-4, False, 0), (4500, 700, 1100, 1e-5, True, 32 << 30),
+    (12000, 500, 64, 0.0, False, 32 << 30)])
+def test_direct_windows_equal_hashed_ones(ctx, n, d, K, theta, zeros, budget):
+    from paper_2002_10083_gb300 import mcl
+    A = _random(n, d, seed=n + d, zeros=zeros)
+    prm = mcl.Params(threshold=theta, select_k=K, recover_pct=0.9, inflation=2.0)
+    try:
+        ctx.set_option(mcl.OPT_BUCKET_BUDGET, budget)
+        out, ch = ctx.expand(A, prm)
+        nnz_b = ctx.stats()["nnz_b"]
+        ctx.set_option(mcl.OPT_CONF_MASK, 1)
+        ref, ch_ref = ctx.expand(A, prm)
+    finally:
+        ctx.set_option(mcl.OPT_CONF_MASK, 3)
+        ctx.set_option(mcl.OPT_BUCKET_BUDGET, 32 << 30)
+    assert nnz_b == ctx.stats()["nnz_b"] and ch == ch_ref
+    assert torch.equal(out.colptr, ref.colptr) and torch.equal(out.rowidx, ref.rowidx)
+    assert torch.equal(out.val.view(torch.int32), ref.val.view(torch.int32))
