@@ -744,7 +744,6 @@ mcl_status mcl_expand_split(mcl_ctx* c, const mcl_csc* A, const mcl_params* prm,
         P.val = (unsigned long long*)dev_alloc(c, (size_t)P.nnz * 8 + 8, s);
         if (!P.rowidx || !P.val) return MCL_ERR_OOM;
         if (P.nnz > 0) {
-            CUDA_TRY(c, cudaMemsetAsync(P.val, 0, (size_t)P.nnz * 8, s));
             ra.colptr_out = P.colptr;
             ra.row_out = P.rowidx;
             ra.val_out = P.val;

@@ -178,7 +178,7 @@ struct RankArgs {
     int64_t* nnz_out;       // count mode: entries per output column
     const int64_t* colptr_out;  // fill mode
     int32_t* row_out;
-    unsigned long long* val_out;  // fill mode: zeroed before the launch
+    unsigned long long* val_out;  // fill mode
     DevCounters* ctr;
 };
 void launch_bsum(const CscView& A, const double* colsum, double* bsum, cudaStream_t s);

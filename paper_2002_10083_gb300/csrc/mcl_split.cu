@@ -13,12 +13,17 @@
 //
 // One kernel does both jobs on row-sorted inputs: for each output column a
 // CTA walks its sources (the columns of A of one stage, scaled by a_kj, or
-// the columns of the partial products being merged) in windows of RA_WB
-// rows; a shared bitmap marks the rows present (count mode: their number),
-// a prefix count of the bitmap gives each row its position in the output
-// column, and the values are added there with 64-bit integer atomics (fill
-// mode), so the output comes out sorted and its sums do not depend on the
-// order of the additions.
+// the columns of the partial products being merged) in windows of rows; a
+// shared bitmap marks the rows present (count mode: their number) and a prefix
+// count of the bitmap gives each row its position in the output column.  Fill
+// mode adds the values at their positions in a shared array of 64-bit sums
+// (several passes over the sources where the window has more entries than the
+// array) and writes the window's entries out in order, so the output comes out
+// sorted and its sums do not depend on the order of the additions.
+//
+// The sources are cut into units of 128 entries that the warps take in turn:
+// a merge has 2 to 5 sources and a stage of a sparse column a handful, which
+// would leave most of the 16 warps idle with a source per warp.
 #include <climits>
 #include <cstdint>
 
@@ -53,17 +58,25 @@ void launch_bsum(const CscView& A, const double* colsum, double* bsum, cudaStrea
 }
 
 constexpr int RA_T = 512;
-constexpr int RA_WORDS = 16384;          // 64 KB bitmap
-constexpr int RA_WB = RA_WORDS * 32;     // rows per window
+constexpr int RA_UNIT = 128;   // entries a warp takes at once
+constexpr int RA_BATCH = 512;  // sources whose units are listed at once
+// Shapes by the rows of the output: bitmap words (32 rows each) and sums.  Up
+// to 131k rows are one window and two CTAs share an SM.
+template <int WORDS_, int CAP_, int MINB_>
+struct RankShape {
+    static constexpr int WORDS = WORDS_, CAP = CAP_, MINB = MINB_;
+};
+using RankSmall = RankShape<4096, 8192, 2>;
+using RankLarge = RankShape<16384, 8192, 1>;
+// More passes than this over a window's sources: add in global memory instead.
+constexpr int RA_PASSES = 4;
 
 struct RankShared {
     BlockScratch bs;
     int wsm[34];
     int item;
-    int next;
-    int ns;
-    int lo, hi;  // row span of the column's sources
-    long long base;
+    int lo, hi;               // row span of the column's sources
+    int upre[RA_BATCH + 1];   // first unit of each source of a batch
 };
 
 // Sources of one output column, per CTA in global scratch (stride entries):
@@ -78,35 +91,48 @@ struct RankScratch {
     int32_t* nxt;
 };
 
-
-
-template <int T>
-__device__ __forceinline__ int block_min_max(int x, bool is_max, BlockScratch* bs) {
+// Exclusive block scan of x; the total to all threads.  Ends with a barrier.
+__device__ __forceinline__ int ra_scan(int x, int* total, int* wsm) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    x = is_max ? warp_max(x) : warp_min(x);
-    if (lane == 0) bs->q[2][warp] = x;
+    int incl = x;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_up_sync(FULL, incl, o);
+        if (lane >= o) incl += y;
+    }
+    if (lane == 31) wsm[warp] = incl;
     __syncthreads();
     if (warp == 0) {
-        long long y = lane < T / 32 ? bs->q[2][lane] : (is_max ? INT_MIN : INT_MAX);
-        int yi = (int)y;
-        yi = is_max ? warp_max(yi) : warp_min(yi);
-        if (lane == 0) bs->q[2][32] = yi;
+        const int w0 = lane < RA_T / 32 ? wsm[lane] : 0;
+        int wi = w0;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int y = __shfl_up_sync(FULL, wi, o);
+            if (lane >= o) wi += y;
+        }
+        if (lane < RA_T / 32) wsm[lane] = wi - w0;
+        if (lane == 31) wsm[32] = wi;
     }
     __syncthreads();
-    const int r = (int)bs->q[2][32];
+    const int res = wsm[warp] + incl - x;
+    *total = wsm[32];
     __syncthreads();
-    return r;
+    return res;
 }
 
 // STAGE: sources are the columns k of A in [k0, k1) referenced by column j;
 // otherwise the columns j of the partial products.  FILL: write the output
 // (else count it).
-template <bool STAGE, bool FILL>
-__global__ void __launch_bounds__(RA_T) k_rank_acc(RankArgs a) {
+template <bool STAGE, bool FILL, class SH>
+__global__ void __launch_bounds__(RA_T, SH::MINB) k_rank_acc(RankArgs a) {
     extern __shared__ __align__(16) unsigned char smem[];
+    constexpr int WORDS = SH::WORDS, CAP = SH::CAP, WB = WORDS * 32;
     uint32_t* bm = reinterpret_cast<uint32_t*>(smem);
-    int32_t* wpre = reinterpret_cast<int32_t*>(bm + RA_WORDS);  // FILL only
-    RankShared* sh = reinterpret_cast<RankShared*>(smem + (size_t)RA_WORDS * 4 * (FILL ? 2 : 1));
+    int32_t* wpre = reinterpret_cast<int32_t*>(bm + WORDS);  // from here FILL only, up to sh
+    unsigned* lo32 = reinterpret_cast<unsigned*>(wpre + WORDS);
+    unsigned* hi32 = lo32 + CAP;
+    RankShared* sh = reinterpret_cast<RankShared*>(FILL ? reinterpret_cast<unsigned char*>(hi32 + CAP)
+                                                        : reinterpret_cast<unsigned char*>(bm + WORDS));
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     constexpr int NWP = RA_T / 32;
     unsigned long long* sb = reinterpret_cast<unsigned long long*>(a.scratch) +
@@ -117,34 +143,31 @@ __global__ void __launch_bounds__(RA_T) k_rank_acc(RankArgs a) {
                    reinterpret_cast<float*>(sb + 3 * a.stride),
                    reinterpret_cast<int32_t*>(sb + 4 * a.stride),
                    reinterpret_cast<int32_t*>(sb + 5 * a.stride)};
+    if (FILL)
+        for (int i = tid; i < 2 * CAP; i += RA_T) lo32[i] = 0u;
     for (;;) {
-        if (tid == 0) sh->item = atomicAdd(&a.ctr->work_ctr, 1);
+        if (tid == 0) {
+            sh->item = atomicAdd(&a.ctr->work_ctr, 1);
+            sh->lo = INT_MAX;
+            sh->hi = -1;
+        }
         __syncthreads();
         const int64_t j = sh->item;
-        __syncthreads();
         if (j >= a.n) break;
         // ---- the column's sources ----
         int ns = 0;
         int64_t i0 = 0;
         if (STAGE) {
+            // rows are sorted: those below k0, and below k1, lead the column
             const int64_t cb = a.A.colptr[j], ce = a.A.colptr[j + 1];
-            if (tid == 0) {
-                int64_t lo = cb, hi = ce;  // first entry with row >= k0
-                while (lo < hi) {
-                    const int64_t m = (lo + hi) >> 1;
-                    if (a.A.rowidx[m] < a.k0) lo = m + 1; else hi = m;
-                }
-                int64_t lo2 = lo, hi2 = ce;  // first entry with row >= k1
-                while (lo2 < hi2) {
-                    const int64_t m = (lo2 + hi2) >> 1;
-                    if (a.A.rowidx[m] < a.k1) lo2 = m + 1; else hi2 = m;
-                }
-                sh->ns = (int)(lo2 - lo);
-                sh->base = lo;
+            int below = 0, within = 0;
+            for (int64_t base = cb; base < ce; base += RA_T) {
+                const int k = base + tid < ce ? a.A.rowidx[base + tid] : INT_MAX;
+                below += __syncthreads_count(k < a.k0);
+                within += __syncthreads_count(k < a.k1);
             }
-            __syncthreads();
-            ns = sh->ns;
-            i0 = sh->base;
+            ns = within - below;
+            i0 = cb + below;
         } else {
             ns = a.nparts;
         }
@@ -156,7 +179,7 @@ __global__ void __launch_bounds__(RA_T) k_rank_acc(RankArgs a) {
             __syncthreads();
             continue;
         }
-        int mn = INT_MAX, mx = INT_MIN;
+        int mn = INT_MAX, mx = -1;
         for (int s = tid; s < ns; s += RA_T) {
             const int32_t* rows;
             const void* vals;
@@ -179,125 +202,154 @@ __global__ void __launch_bounds__(RA_T) k_rank_acc(RankArgs a) {
             rs.vals[s] = vals;
             rs.len[s] = len;
             rs.akj[s] = f;
-            rs.cur[s] = 0;
+            rs.nxt[s] = 0;
             if (len > 0) {
                 mn = min(mn, rows[0]);
                 mx = max(mx, rows[len - 1]);
             }
         }
-        const int lo = block_min_max<RA_T>(mn, false, &sh->bs);
-        const int hiE = block_min_max<RA_T>(mx, true, &sh->bs) + 1;
+        if (mx >= 0) {
+            atomicMin(&sh->lo, mn);
+            atomicMax(&sh->hi, mx);
+        }
+        __syncthreads();
+        const int lo = sh->lo;
+        const int hiE = sh->hi + 1;
         FixScale fx;
         fx.init(STAGE ? a.bsum[j] : 1.0);
         long long cnt = 0;
         int64_t obase = FILL ? a.colptr_out[j] : 0;
-        int32_t* cur = rs.cur;
-        int32_t* nxt = rs.nxt;
         for (int r0 = lo; r0 < hiE && hiE > lo;) {
-            const int r1 = (int)min((int64_t)r0 + RA_WB, (int64_t)hiE);
+            const int r1 = (int)min((int64_t)r0 + WB, (int64_t)hiE);
             const int nwords = (r1 - r0 + 31) >> 5;
+            const bool last = r1 == hiE;
             for (int i = tid; i < nwords; i += RA_T) bm[i] = 0u;
-            if (tid == 0) sh->next = 0;
-            __syncthreads();
-            // ---- mark the rows of the window ----
-            for (;;) {
-                int s = 0;
-                if (lane == 0) s = atomicAdd(&sh->next, 1);
-                s = __shfl_sync(FULL, s, 0);
-                if (s >= ns) break;
-                const int32_t* rows = rs.rows[s];
-                const int len = rs.len[s];
-                int pos = cur[s];
-                while (pos < len) {
-                    const int p = pos + lane;
-                    const int row = p < len ? __ldg(rows + p) : INT_MAX;
-                    const bool in = row < r1;
-                    if (in) {
-                        const int off = row - r0;
-                        atomicOr(bm + (off >> 5), 1u << (off & 31));
+            // each source's entries of the window: [cur, nxt)
+            for (int s = tid; s < ns; s += RA_T) {
+                const int c0 = rs.nxt[s], len = rs.len[s];
+                int x = len;
+                if (!last) {
+                    int h = len;  // first entry at or beyond r1
+                    x = c0;
+                    const int32_t* rows = rs.rows[s];
+                    while (x < h) {
+                        const int m = (x + h) >> 1;
+                        if (rows[m] < r1) x = m + 1; else h = m;
                     }
-                    const int nin = __popc(__ballot_sync(FULL, in));
-                    pos += nin;
-                    if (nin < 32) break;
                 }
-                if (lane == 0) nxt[s] = pos;
+                rs.cur[s] = c0;
+                rs.nxt[s] = x;
             }
             __syncthreads();
+            // f(s, p0, end) for every unit [p0, p0 + RA_UNIT) of the sources' entries
+            auto each_unit = [&](auto f) {
+                for (int b0 = 0; b0 < ns; b0 += RA_BATCH) {
+                    const int m = min(RA_BATCH, ns - b0);
+                    if (RA_T >= RA_BATCH) {
+                        const int u = tid < m ? (rs.nxt[b0 + tid] - rs.cur[b0 + tid] + RA_UNIT - 1) / RA_UNIT : 0;
+                        int tot;
+                        const int at = ra_scan(u, &tot, sh->wsm);
+                        if (tid < m) sh->upre[tid] = at;
+                        if (tid == 0) sh->upre[m] = tot;
+                    }
+                    __syncthreads();
+                    const int units = sh->upre[m];
+                    int s = 0;
+                    for (int u = warp; u < units; u += NWP) {
+                        while (sh->upre[s + 1] <= u) ++s;
+                        f(b0 + s, rs.cur[b0 + s] + (u - sh->upre[s]) * RA_UNIT, rs.nxt[b0 + s]);
+                    }
+                    __syncthreads();
+                }
+            };
+            // ---- mark the rows of the window ----
+            each_unit([&](int s, int p0, int end) {
+                const int32_t* rows = rs.rows[s] + lane;
+                int rr[RA_UNIT / 32];
+#pragma unroll
+                for (int c = 0; c < RA_UNIT / 32; ++c)
+                    rr[c] = p0 + 32 * c + lane < end ? __ldg(rows + p0 + 32 * c) : -1;
+#pragma unroll
+                for (int c = 0; c < RA_UNIT / 32; ++c)
+                    if (rr[c] >= 0) {
+                        const int off = rr[c] - r0;
+                        atomicOr(bm + (off >> 5), 1u << (off & 31));
+                    }
+            });
             if (!FILL) {
                 for (int i = tid; i < nwords; i += RA_T) cnt += __popc(bm[i]);
                 __syncthreads();
             } else {
                 // ---- positions: exclusive prefix counts of the bitmap words ----
-                constexpr int PER = RA_WORDS / RA_T;
-                int loc[PER];
-                int tsum = 0;
-#pragma unroll
-                for (int q = 0; q < PER; ++q) {
-                    const int w = tid * PER + q;
-                    loc[q] = tsum;
-                    tsum += w < nwords ? __popc(bm[w]) : 0;
-                }
-                // block exclusive scan of tsum
-                int incl = tsum;
-#pragma unroll
-                for (int o = 1; o < 32; o <<= 1) {
-                    const int y = __shfl_up_sync(FULL, incl, o);
-                    if (lane >= o) incl += y;
-                }
-                if (lane == 31) sh->wsm[warp] = incl;
-                __syncthreads();
-                if (warp == 0) {
-                    const int w0 = lane < NWP ? sh->wsm[lane] : 0;
-                    int wi = w0;
-#pragma unroll
-                    for (int o = 1; o < 32; o <<= 1) {
-                        const int y = __shfl_up_sync(FULL, wi, o);
-                        if (lane >= o) wi += y;
-                    }
-                    if (lane < NWP) sh->wsm[lane] = wi - w0;
-                    if (lane == 31) sh->wsm[32] = wi;
+                int wtot = 0;
+                for (int w0 = 0; w0 < nwords; w0 += RA_T) {
+                    const int w = w0 + tid;
+                    int tot;
+                    const int at = ra_scan(w < nwords ? __popc(bm[w]) : 0, &tot, sh->wsm);
+                    if (w < nwords) wpre[w] = wtot + at;
+                    wtot += tot;
                 }
                 __syncthreads();
-                const int tbase = sh->wsm[warp] + incl - tsum;
+                // rows of the entries, in order
+                for (int w = tid; w < nwords; w += RA_T) {
+                    int64_t at = obase + wpre[w];
+                    for (uint32_t x = bm[w]; x; x &= x - 1u) a.row_out[at++] = r0 + 32 * w + __ffs(x) - 1;
+                }
+                // ---- sums ----
+                auto products = [&](auto put) {  // put(position, sum)
+                    each_unit([&](int s, int p0, int end) {
+                        const int32_t* rows = rs.rows[s];
+                        const float akj = rs.akj[s];
+                        int rr[RA_UNIT / 32];
+                        unsigned long long q[RA_UNIT / 32];
 #pragma unroll
-                for (int q = 0; q < PER; ++q) wpre[tid * PER + q] = tbase + loc[q];
-                const int wtot = sh->wsm[32];
-                if (tid == 0) sh->next = 0;
-                __syncthreads();
-                // ---- add every product at its row's position ----
-                for (;;) {
-                    int s = 0;
-                    if (lane == 0) s = atomicAdd(&sh->next, 1);
-                    s = __shfl_sync(FULL, s, 0);
-                    if (s >= ns) break;
-                    const int32_t* rows = rs.rows[s];
-                    const int len = rs.len[s];
-                    const float f = rs.akj[s];
-                    for (int pos = cur[s]; pos < nxt[s]; pos += 32) {
-                        const int p = pos + lane;
-                        if (p < nxt[s]) {
-                            const int row = __ldg(rows + p);
-                            const int off = row - r0;
-                            const uint32_t word = bm[off >> 5];
-                            const int rank =
-                                wpre[off >> 5] + __popc(word & ((1u << (off & 31)) - 1u));
-                            unsigned long long q;
+                        for (int c = 0; c < RA_UNIT / 32; ++c) {
+                            const int p = p0 + 32 * c + lane;
+                            rr[c] = p < end ? __ldg(rows + p) : -1;
                             if (STAGE)
-                                q = fx.q(__ldg(reinterpret_cast<const float*>(rs.vals[s]) + p), f);
+                                q[c] = __float_as_uint(
+                                    p < end ? __ldg(reinterpret_cast<const float*>(rs.vals[s]) + p) : 0.0f);
                             else
-                                q = reinterpret_cast<const unsigned long long*>(rs.vals[s])[p];
-                            const int64_t at = obase + rank;
-                            a.row_out[at] = row;
-                            atomicAdd(a.val_out + at, q);
+                                q[c] = p < end ? reinterpret_cast<const unsigned long long*>(rs.vals[s])[p] : 0ull;
                         }
+#pragma unroll
+                        for (int c = 0; c < RA_UNIT / 32; ++c)
+                            if (rr[c] >= 0) {
+                                const int off = rr[c] - r0;
+                                const int rank = wpre[off >> 5] +
+                                                 __popc(bm[off >> 5] & ((1u << (off & 31)) - 1u));
+                                put(rank, STAGE ? fx.q(__uint_as_float((unsigned)q[c]), akj) : q[c]);
+                            }
+                    });
+                };
+                const int npass = (wtot + CAP - 1) / CAP;
+                if (npass <= RA_PASSES) {
+                    for (int e0 = 0; e0 < wtot; e0 += CAP) {
+                        products([&](int rank, unsigned long long q) {
+                            const unsigned e = (unsigned)(rank - e0);
+                            if (e < (unsigned)CAP) {
+                                const unsigned ql = (unsigned)q;
+                                const unsigned old = atomicAdd(lo32 + e, ql);
+                                const unsigned qh = (unsigned)(q >> 32) + (old + ql < old ? 1u : 0u);
+                                if (qh) atomicAdd(hi32 + e, qh);
+                            }
+                        });
+                        const int m = min(CAP, wtot - e0);
+                        for (int e = tid; e < m; e += RA_T) {
+                            a.val_out[obase + e0 + e] = ((unsigned long long)hi32[e] << 32) | lo32[e];
+                            lo32[e] = 0u;
+                            hi32[e] = 0u;
+                        }
+                        __syncthreads();
                     }
+                } else {  // more entries than a few passes hold: 64-bit atomics in global memory
+                    for (int e = tid; e < wtot; e += RA_T) a.val_out[obase + e] = 0ull;
+                    __syncthreads();
+                    products([&](int rank, unsigned long long q) { atomicAdd(a.val_out + obase + rank, q); });
                 }
                 obase += wtot;
                 __syncthreads();
             }
-            int32_t* t = cur;
-            cur = nxt;
-            nxt = t;
             r0 = r1;
         }
         if (!FILL) {
@@ -306,13 +358,14 @@ __global__ void __launch_bounds__(RA_T) k_rank_acc(RankArgs a) {
             block_sum<RA_T>(dd, 0, qq, 1, &sh->bs);
             if (tid == 0) a.nnz_out[j] = qq[0];
         }
+        __syncthreads();
     }
 }
 
-template <bool STAGE, bool FILL>
+template <bool STAGE, bool FILL, class SH>
 static void rank_launch(const RankArgs& a, int num_sms, cudaStream_t s) {
-    const size_t smem = (size_t)RA_WORDS * 4 * (FILL ? 2 : 1) + sizeof(RankShared);
-    auto kern = k_rank_acc<STAGE, FILL>;
+    const size_t smem = (size_t)SH::WORDS * 4 * (FILL ? 2 : 1) + (FILL ? (size_t)SH::CAP * 8 : 0) + sizeof(RankShared);
+    auto kern = k_rank_acc<STAGE, FILL, SH>;
     cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     int occ = 0;
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, RA_T, smem);
@@ -325,20 +378,28 @@ static void rank_launch(const RankArgs& a, int num_sms, cudaStream_t s) {
     count_launches(1);
 }
 
-void launch_split_count(const RankArgs& a, bool stage, int num_sms, cudaStream_t s) {
-    if (a.n == 0) return;
+template <class SH>
+static void rank_any(const RankArgs& a, bool stage, bool fill, int num_sms, cudaStream_t s) {
     if (stage)
-        rank_launch<true, false>(a, num_sms, s);
+        fill ? rank_launch<true, true, SH>(a, num_sms, s) : rank_launch<true, false, SH>(a, num_sms, s);
     else
-        rank_launch<false, false>(a, num_sms, s);
+        fill ? rank_launch<false, true, SH>(a, num_sms, s) : rank_launch<false, false, SH>(a, num_sms, s);
+}
+
+static void rank_shape(const RankArgs& a, bool stage, bool fill, int num_sms, cudaStream_t s) {
+    if (a.n == 0) return;
+    if (a.n <= RankSmall::WORDS * 32)
+        rank_any<RankSmall>(a, stage, fill, num_sms, s);
+    else
+        rank_any<RankLarge>(a, stage, fill, num_sms, s);
+}
+
+void launch_split_count(const RankArgs& a, bool stage, int num_sms, cudaStream_t s) {
+    rank_shape(a, stage, false, num_sms, s);
 }
 
 void launch_split_fill(const RankArgs& a, bool stage, int num_sms, cudaStream_t s) {
-    if (a.n == 0) return;
-    if (stage)
-        rank_launch<true, true>(a, num_sms, s);
-    else
-        rank_launch<false, true>(a, num_sms, s);
+    rank_shape(a, stage, true, num_sms, s);
 }
 
 }  // namespace mcl
