@@ -19,7 +19,6 @@
 #include <cfloat>
 #include <climits>
 #include <cstdint>
-#include <mutex>
 
 #include "mcl_device.cuh"
 #include "mcl_internal.h"
@@ -270,125 +269,173 @@ template void launch_exclusive_scan<int32_t>(const int32_t*, int64_t, int64_t*, 
 // exact symbolic pass: nnz((AA)_*j) with a shared-memory bitmap
 // ---------------------------------------------------------------------------
 
-constexpr int SYM_T = 512;
+// One CTA per column: the rows of its sources set bits of a shared bitmap over
+// the row span (in windows where it exceeds the bitmap), and one pass counts
+// and clears it.  The sources are cut into units of 128 rows that the warps
+// take in turn, all four loads of a lane first: a warp per source left most
+// warps idle behind the longest one, with one load in flight each.
 constexpr int SYM_WORDS = 16384;  // 64 KB bitmap -> 524,288 rows per window
+constexpr int SYM_UNIT = 128;
+constexpr int SYM_BATCH = 512;    // sources whose units are listed at once
 
 struct SymShared {
     BlockScratch bs;
+    int wsm[34];
     int item;
-    int next;
+    int upre[SYM_BATCH + 1];      // first unit of each source of the batch
+    int cnt[SYM_BATCH];           // rows of each source in the window
+    int64_t first[SYM_BATCH];     // and its first entry
 };
 
-__global__ void __launch_bounds__(SYM_T) k_symbolic(CscView A, ExpandBuffers b, int64_t* nnz_out) {
+// words: bitmap words of this launch, a multiple of 4
+template <int T>
+__global__ void __launch_bounds__(T) k_symbolic(CscView A, ExpandBuffers b, int64_t* nnz_out, int words) {
     extern __shared__ __align__(16) unsigned char smem[];
     uint32_t* bm = reinterpret_cast<uint32_t*>(smem);
-    SymShared* sh = reinterpret_cast<SymShared*>(bm + SYM_WORDS);
-    const int tid = threadIdx.x, lane = tid & 31;
-    constexpr int WB = SYM_WORDS * 32;
+    SymShared* sh = reinterpret_cast<SymShared*>(bm + words);
+    constexpr int NW = T / 32, PER = SYM_BATCH / T;
+    static_assert(SYM_BATCH % T == 0, "whole sources per thread");
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int WB = words * 32;
     int32_t* cur = b.cursors + (int64_t)blockIdx.x * 2 * b.cur_stride;
+    uint4* bm4 = reinterpret_cast<uint4*>(bm);
+    for (int i = tid; i < words / 4; i += T) bm4[i] = make_uint4(0u, 0u, 0u, 0u);
     for (;;) {
         if (tid == 0) sh->item = atomicAdd(&b.ctr->work_ctr, 1);
         __syncthreads();
         const int64_t j = sh->item;
-        __syncthreads();
         if (j >= A.n) break;
-        const int64_t cb = A.colptr[j], ce = A.colptr[j + 1];
-        const int d = (int)(ce - cb);
+        const int64_t cb = A.colptr[j];
+        const int d = (int)(A.colptr[j + 1] - cb);
         const int lo = b.rlo[j], hiE = b.rhi[j] + 1;
-        if (d == 0 || hiE <= lo) {
-            if (tid == 0) nnz_out[j] = 0;
-            continue;
-        }
-        const int span = hiE - lo;
-        const bool windows = span > WB;
-        if (windows) {
-            if (d > b.cur_stride) {  // cannot happen: cur_stride >= max degree
-                if (tid == 0) set_err(b.ctr, ERR_CURSOR);
-                continue;
+        const bool windows = hiE - lo > WB;
+        if (d == 0 || hiE <= lo || (windows && d > b.cur_stride)) {
+            if (tid == 0) {
+                nnz_out[j] = 0;
+                if (windows) set_err(b.ctr, ERR_CURSOR);  // cannot happen: cur_stride >= max degree
             }
-            for (int i = tid; i < d; i += SYM_T) cur[i] = 0;
+            __syncthreads();
+            continue;
         }
         long long cnt = 0;
         for (int r0 = lo; r0 < hiE;) {
             const int r1 = (int)min((int64_t)r0 + WB, (int64_t)hiE);
-            const int nwords = (r1 - r0 + 31) >> 5;
-            for (int i = tid; i < nwords; i += SYM_T) bm[i] = 0u;
-            if (tid == 0) sh->next = 0;
-            __syncthreads();
-            for (;;) {
-                int kidx = 0;
-                if (lane == 0) kidx = atomicAdd(&sh->next, 1);
-                kidx = __shfl_sync(FULL, kidx, 0);
-                if (kidx >= d) break;
-                const int k = __ldg(A.rowidx + cb + kidx);
-                const int64_t ks = __ldg(A.colptr + k), ke = __ldg(A.colptr + k + 1);
-                int64_t pos = ks + (windows ? cur[kidx] : 0);
-                while (pos < ke) {
-                    const int64_t q = pos + lane;
-                    const bool valid = q < ke;
-                    const int rr = valid ? __ldg(A.rowidx + q) : INT_MAX;
-                    const bool in = valid && rr < r1;
-                    const unsigned bal = __ballot_sync(FULL, in);
-                    if (in) {
-                        const int off = rr - r0;
-                        const uint32_t bit = 1u << (off & 31);
-                        uint32_t* w = bm + (off >> 5);
-                        if (!(*reinterpret_cast<volatile uint32_t*>(w) & bit)) atomicOr(w, bit);
+            for (int b0 = 0; b0 < d; b0 += SYM_BATCH) {
+                const int m = min(SYM_BATCH, d - b0);
+                int u[PER], usum = 0;
+#pragma unroll
+                for (int q = 0; q < PER; ++q) {
+                    const int i = tid * PER + q;
+                    u[q] = 0;
+                    if (i < m) {
+                        const int k = __ldg(A.rowidx + cb + b0 + i);
+                        const int64_t ks = __ldg(A.colptr + k);
+                        const int len = (int)(__ldg(A.colptr + k + 1) - ks);
+                        int c0 = 0, c1 = len;
+                        if (windows) {  // the source's rows in [r0, r1): [c0, c1)
+                            c0 = r0 == lo ? 0 : cur[b0 + i];
+                            if (r1 < hiE) {
+                                int x = c0;
+                                while (x < c1) {
+                                    const int mid = (x + c1) >> 1;
+                                    if (__ldg(A.rowidx + ks + mid) < r1) x = mid + 1; else c1 = mid;
+                                }
+                            }
+                            cur[b0 + i] = c1;
+                        }
+                        sh->first[i] = ks + c0;
+                        sh->cnt[i] = c1 - c0;
+                        u[q] = (c1 - c0 + SYM_UNIT - 1) / SYM_UNIT;
                     }
-                    const int nin = __popc(bal);
-                    pos += nin;
-                    if (nin < 32) break;
+                    usum += u[q];
                 }
-                if (windows && lane == 0) cur[kidx] = (int)(pos - ks);
+                int incl = usum;
+#pragma unroll
+                for (int o = 1; o < 32; o <<= 1) {
+                    const int y = __shfl_up_sync(FULL, incl, o);
+                    if (lane >= o) incl += y;
+                }
+                if (lane == 31) sh->wsm[warp] = incl;
+                __syncthreads();
+                int at = incl - usum, units = 0;
+#pragma unroll
+                for (int w = 0; w < NW; ++w) {
+                    const int x = sh->wsm[w];
+                    at += w < warp ? x : 0;
+                    units += x;
+                }
+#pragma unroll
+                for (int q = 0; q < PER; ++q) {
+                    sh->upre[tid * PER + q] = at;
+                    at += u[q];
+                }
+                if (tid == T - 1) sh->upre[SYM_BATCH] = units;
+                __syncthreads();
+                int s = 0;
+                for (int un = warp; un < units; un += NW) {
+                    while (sh->upre[s + 1] <= un) ++s;  // ends: upre[SYM_BATCH] = units > un
+                    const int p0 = (un - sh->upre[s]) * SYM_UNIT;
+                    const int rem = sh->cnt[s] - p0 - lane;
+                    const int32_t* rows = A.rowidx + sh->first[s] + p0 + lane;
+                    int off[SYM_UNIT / 32];
+#pragma unroll
+                    for (int c = 0; c < SYM_UNIT / 32; ++c)
+                        off[c] = 32 * c < rem ? __ldg(rows + 32 * c) - r0 : -1;
+#pragma unroll
+                    for (int c = 0; c < SYM_UNIT / 32; ++c)
+                        if (off[c] >= 0) atomicOr(bm + (off[c] >> 5), 1u << (off[c] & 31));
+                }
+                __syncthreads();
             }
-            __syncthreads();
-            for (int i = tid; i < nwords; i += SYM_T) cnt += __popc(bm[i]);
+            const int n4 = (r1 - r0 + 127) >> 7;  // the bitmap's words in fours
+            int c = 0;
+            for (int i = tid; i < n4; i += T) {
+                const uint4 x = bm4[i];
+                c += __popc(x.x) + __popc(x.y) + __popc(x.z) + __popc(x.w);
+                bm4[i] = make_uint4(0u, 0u, 0u, 0u);
+            }
+            cnt += c;
             __syncthreads();
             r0 = r1;
         }
         double dd[1] = {0.0};
         long long qq[1] = {cnt};
-        block_sum<SYM_T>(dd, 0, qq, 1, &sh->bs);
+        block_sum<T>(dd, 0, qq, 1, &sh->bs);
         if (tid == 0) nnz_out[j] = qq[0];
     }
 }
 
+static size_t symbolic_smem(int words) { return (size_t)words * 4 + sizeof(SymShared); }
+
 // The dynamic shared-memory limit is a per-device attribute of the kernel:
-// it is set on the current device before every launch, and the occupancy it
-// gives is cached per device (first use under a lock).
-static void symbolic_set_smem() {
-    cudaFuncSetAttribute(k_symbolic, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)(SYM_WORDS * 4 + sizeof(SymShared)));
+// it is set on the current device before every launch.
+template <int T>
+static int symbolic_occupancy(int words, int num_sms) {
+    cudaFuncSetAttribute(k_symbolic<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                         (int)symbolic_smem(words));
+    int occ = 0;
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_symbolic<T>, T, symbolic_smem(words));
+    return (occ < 1 ? 1 : occ) * num_sms;
 }
 
-int symbolic_grid(int num_sms) {
-    constexpr int kMaxDev = 64;
-    static std::mutex mu;
-    static int occ_dev[kMaxDev] = {0};
-    int dev = 0;
-    cudaGetDevice(&dev);
-    std::lock_guard<std::mutex> lk(mu);
-    int occ = (dev >= 0 && dev < kMaxDev) ? occ_dev[dev] : 0;
-    if (occ < 1) {
-        symbolic_set_smem();
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_symbolic, SYM_T,
-                                                      SYM_WORDS * 4 + sizeof(SymShared));
-        if (occ < 1) occ = 1;
-        if (dev >= 0 && dev < kMaxDev) occ_dev[dev] = occ;
-    }
-    return occ * num_sms;
-}
+// CTAs that the cursor scratch has to serve (several windows: the full bitmap)
+int symbolic_grid(int num_sms) { return symbolic_occupancy<512>(SYM_WORDS, num_sms); }
 
 void launch_symbolic(const CscView& A, const ExpandBuffers& b, int64_t* nnz_out, int num_sms,
                      int grid_cap, cudaStream_t s) {
     if (A.n == 0) return;
-    size_t smem = SYM_WORDS * 4 + sizeof(SymShared);
-    symbolic_set_smem();
-    int grid = symbolic_grid(num_sms);
-    if (grid > grid_cap) grid = grid_cap;
-    if ((int64_t)grid > A.n) grid = (int)A.n;
+    int words = (int)(((int64_t)A.n + 127) / 128 * 4);
+    if (words > SYM_WORDS) words = SYM_WORDS;
+    // few products per column: a warp's work or two
+    const bool small = A.nnz <= (int64_t)A.n * 32 && A.n <= SYM_WORDS;
+    int grid = small ? symbolic_occupancy<128>(words, num_sms) : symbolic_occupancy<512>(words, num_sms);
+    if (A.n > SYM_WORDS * 32 && grid > grid_cap) grid = grid_cap;
+    if ((int64_t)grid > A.n) grid = A.n;
     cudaMemsetAsync(&b.ctr->work_ctr, 0, sizeof(int), s);
-    k_symbolic<<<grid, SYM_T, smem, s>>>(A, b, nnz_out);
+    if (small)
+        k_symbolic<128><<<grid, 128, symbolic_smem(words), s>>>(A, b, nnz_out, words);
+    else
+        k_symbolic<512><<<grid, 512, symbolic_smem(words), s>>>(A, b, nnz_out, words);
     count_launches(1);
 }
 
