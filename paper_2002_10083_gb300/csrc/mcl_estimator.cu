@@ -93,35 +93,39 @@ __global__ void k_features(CscView A, int32_t iteration, const int32_t* iter_dev
         fmin = warp_min(fmin);
         lmax = warp_max(lmax);
         if (lane < NIN) {
-            float f = 0.0f;
+            // lanes that take a logarithm choose its argument first and evaluate it together:
+            // one after the other, the FP64 log1p of four of them took most of this kernel
+            float f = 0.0f, lf = -1.0f;
+            double ld = -1.0;
             const double dd = (double)d;
             switch (lane) {
-                case 0: f = log1pf((float)d); break;
-                case 1: f = (float)log1p((double)sd); break;
-                case 2: f = d ? log1pf((float)md) : 0.0f; break;
-                case 3: f = d ? (float)log1p((double)sd / dd) : 0.0f; break;
+                case 0: lf = (float)d; break;
+                case 1: ld = (double)sd; break;
+                case 2: lf = d ? (float)md : 0.0f; break;
+                case 3: ld = d ? (double)sd / dd : 0.0; break;
                 case 4: {
+                    ld = 0.0;
                     if (d) {
                         const double mean = (double)sd / dd;
-                        double var = (double)sd2 / dd - mean * mean;
-                        f = (float)log1p(var > 0.0 ? var : 0.0);
+                        const double var = (double)sd2 / dd - mean * mean;
+                        ld = var > 0.0 ? var : 0.0;
                     }
                     break;
                 }
                 case 5: f = ma; break;
                 case 6: f = (float)sa; break;
                 case 7: f = (float)sa2; break;
-                case 8:
-                    f = d ? log1pf((float)(A.rowidx[ce - 1] - A.rowidx[cb] + 1)) : 0.0f;
-                    break;
+                case 8: lf = d ? (float)(A.rowidx[ce - 1] - A.rowidx[cb] + 1) : 0.0f; break;
                 case 9: f = d ? (float)((double)huge / dd) : 0.0f; break;
                 case 10: f = logn; break;
                 case 11: f = logit; break;
                 case 12: f = prev_logcf ? prev_logcf[j] : 0.0f; break;
                 case 13: f = d ? (float)(scm / dd) : 0.0f; break;
-                case 14: f = (lmax >= 0) ? (float)log1p((double)(lmax - fmin) + 1.0) : 0.0f; break;
+                case 14: ld = lmax >= 0 ? (double)(lmax - fmin) + 1.0 : 0.0; break;
                 default: f = 1.0f; break;
             }
+            if (lf >= 0.0f) f = log1pf(lf);
+            if (ld >= 0.0) f = (float)log1p(ld);
             feats[j * NIN + lane] = f;
         }
     }
@@ -131,62 +135,120 @@ __global__ void k_features(CscView A, int32_t iteration, const int32_t* iter_dev
 // forward
 // ---------------------------------------------------------------------------
 
-constexpr int FWD_T = 128;
+// Weights in shared memory as FP32, W2's rows padded by four words: the lanes
+// of a warp read four (or eight) rows at once, 16 bytes each, from different
+// banks.
+constexpr int W2P = NH + 4;
 
-__device__ __forceinline__ void load_weights(float* W, const uint16_t* wbits) {
-    for (int i = threadIdx.x; i < NPARAM; i += blockDim.x) W[i] = bf16_bits_to_float(wbits[i]);
+struct MlpWeights {
+    float w1[NH * NIN];
+    float w2[NH * W2P];
+    float w3[NOUT * NH];
+    float b1[NH], b2[NH], b3[4];
+    float mu[NIN], isg[NIN];
+};
+
+__device__ __forceinline__ void load_weights(MlpWeights& M, const uint16_t* wbits, const float* norm) {
+    for (int p = threadIdx.x; p < NPARAM; p += blockDim.x) {
+        const float w = bf16_bits_to_float(wbits[p]);
+        if (p < OFF_B1) M.w1[p] = w;
+        else if (p < OFF_W2) M.b1[p - OFF_B1] = w;
+        else if (p < OFF_B2) M.w2[(p - OFF_W2) / NH * W2P + (p - OFF_W2) % NH] = w;
+        else if (p < OFF_W3) M.b2[p - OFF_B2] = w;
+        else if (p < OFF_B3) M.w3[p - OFF_W3] = w;
+        else M.b3[p - OFF_B3] = w;
+    }
+    if (threadIdx.x < NIN) {
+        M.mu[threadIdx.x] = norm[threadIdx.x];
+        M.isg[threadIdx.x] = 1.0f / norm[NIN + threadIdx.x];
+    }
 }
 
-// One sample per thread.  Writes y (out, n x 2) and/or, when est != NULL,
-// the size estimate est_j = clamp(ceil(expm1(y0) * safety), 1, min(flops, span)).
+// Units e, e + TPS, ... of a layer for one sample: acc[t] = b[o] + sum_i w[o][i] x[i], i
+// ascending in one chain per unit, so that the result does not depend on TPS.
+template <int TPS, int K, int STRIDE>
+__device__ __forceinline__ void mlp_layer(const float* w, const float* b, const float* x, int e,
+                                          float (&acc)[NH / TPS]) {
+#pragma unroll
+    for (int t = 0; t < NH / TPS; ++t) acc[t] = b[t * TPS + e];
+#pragma unroll 2
+    for (int i = 0; i < K; i += 4) {
+        const float4 xv = *reinterpret_cast<const float4*>(x + i);
+#pragma unroll
+        for (int t = 0; t < NH / TPS; ++t) {
+            const float4 wv = *reinterpret_cast<const float4*>(w + (t * TPS + e) * STRIDE + i);
+            acc[t] = fmaf(wv.x, xv.x, acc[t]);
+            acc[t] = fmaf(wv.y, xv.y, acc[t]);
+            acc[t] = fmaf(wv.z, xv.z, acc[t]);
+            acc[t] = fmaf(wv.w, xv.w, acc[t]);
+        }
+    }
+}
+
+// Four threads per sample (16 units each), activations through shared memory.
+// With one thread per sample every multiply-add read its weight alone: bound
+// by shared-memory reads on large inputs, and on a training batch by the one
+// chain of 5,248 multiply-adds per thread on a third of the SMs.
+constexpr int FWD_T = 128, FWD_TPS = 4, FWD_S = FWD_T / FWD_TPS;
+constexpr int HP4 = NH + 4;  // row stride of activations: 16-byte rows, four words apart in the banks
+
+struct FwdShared {
+    MlpWeights m;
+    float z[FWD_S][NIN + 4];
+    float h[FWD_S][HP4];
+    float h2[FWD_S][HP4];
+};
+
+// Writes y (out, n x 2) and/or, when est != NULL, the size estimate
+// est_j = clamp(ceil(expm1(y0) * safety), 1, min(flops, span)).
 __global__ void __launch_bounds__(FWD_T) k_mlp_forward(const float* feats, int64_t n,
                                                        const uint16_t* wbits, const float* norm,
                                                        float* out, int64_t* est, float safety,
                                                        const int64_t* flops, const int32_t* rlo,
                                                        const int32_t* rhi) {
-    __shared__ float W[NPARAM];
-    __shared__ float mu[NIN], isg[NIN];
-    load_weights(W, wbits);
-    if (threadIdx.x < NIN) {
-        mu[threadIdx.x] = norm[threadIdx.x];
-        isg[threadIdx.x] = 1.0f / norm[NIN + threadIdx.x];
-    }
+    __shared__ __align__(16) FwdShared S;
+    load_weights(S.m, wbits, norm);
     __syncthreads();
-    for (int64_t s = (int64_t)blockIdx.x * FWD_T + threadIdx.x; s < n;
-         s += (int64_t)gridDim.x * FWD_T) {
-        float z[NIN];
+    const int q = threadIdx.x / FWD_TPS, e = threadIdx.x % FWD_TPS;
+    // a sample's threads are neighbours in one warp, the only one that touches its rows
+    for (int64_t base = (int64_t)blockIdx.x * FWD_S; base < n; base += (int64_t)gridDim.x * FWD_S) {
+        const int64_t s = base + q;
+        const bool v = s < n;
 #pragma unroll
-        for (int i = 0; i < NIN; ++i) z[i] = (feats[s * NIN + i] - mu[i]) * isg[i];
-        float h1[NH];
+        for (int i = 0; i < NIN; i += FWD_TPS)
+            S.z[q][i + e] = v ? (feats[s * NIN + i + e] - S.m.mu[i + e]) * S.m.isg[i + e] : 0.0f;
+        __syncwarp();
+        float acc[NH / FWD_TPS];
+        mlp_layer<FWD_TPS, NIN, NIN>(S.m.w1, S.m.b1, S.z[q], e, acc);
 #pragma unroll
-        for (int o = 0; o < NH; ++o) {
-            float acc = W[OFF_B1 + o];
+        for (int t = 0; t < NH / FWD_TPS; ++t) S.h[q][t * FWD_TPS + e] = fmaxf(acc[t], 0.0f);
+        __syncwarp();
+        mlp_layer<FWD_TPS, NH, W2P>(S.m.w2, S.m.b2, S.h[q], e, acc);
 #pragma unroll
-            for (int i = 0; i < NIN; ++i) acc = fmaf(W[OFF_W1 + o * NIN + i], z[i], acc);
-            h1[o] = fmaxf(acc, 0.0f);
+        for (int t = 0; t < NH / FWD_TPS; ++t) S.h2[q][t * FWD_TPS + e] = fmaxf(acc[t], 0.0f);
+        __syncwarp();
+        if (e < NOUT && v) {
+            float y = S.m.b3[e];
+#pragma unroll 4
+            for (int o = 0; o < NH; o += 4) {
+                const float4 wv = *reinterpret_cast<const float4*>(S.m.w3 + e * NH + o);
+                const float4 hv = *reinterpret_cast<const float4*>(&S.h2[q][o]);
+                y = fmaf(wv.x, hv.x, y);
+                y = fmaf(wv.y, hv.y, y);
+                y = fmaf(wv.z, hv.z, y);
+                y = fmaf(wv.w, hv.w, y);
+            }
+            if (out) out[s * 2 + e] = y;
+            if (est && e == 0) {
+                int64_t hi = flops[s];
+                const int64_t span = (int64_t)rhi[s] - rlo[s] + 1;
+                if (span < hi) hi = span;
+                if (hi < 1) hi = 1;
+                const double x = ceil(expm1((double)fminf(y, 40.0f)) * (double)safety);
+                est[s] = x < 1.0 ? 1 : (x > (double)hi ? hi : (int64_t)x);
+            }
         }
-        float y0 = W[OFF_B3], y1 = W[OFF_B3 + 1];
-        for (int o = 0; o < NH; ++o) {
-            float acc = W[OFF_B2 + o];
-#pragma unroll
-            for (int i = 0; i < NH; ++i) acc = fmaf(W[OFF_W2 + o * NH + i], h1[i], acc);
-            const float h2 = fmaxf(acc, 0.0f);
-            y0 = fmaf(W[OFF_W3 + o], h2, y0);
-            y1 = fmaf(W[OFF_W3 + NH + o], h2, y1);
-        }
-        if (out) {
-            out[s * 2] = y0;
-            out[s * 2 + 1] = y1;
-        }
-        if (est) {
-            int64_t hi = flops[s];
-            const int64_t span = (int64_t)rhi[s] - rlo[s] + 1;
-            if (span < hi) hi = span;
-            if (hi < 1) hi = 1;
-            const double e = ceil(expm1((double)fminf(y0, 40.0f)) * (double)safety);
-            int64_t v = e < 1.0 ? 1 : (e > (double)hi ? hi : (int64_t)e);
-            est[s] = v;
-        }
+        __syncwarp();
     }
 }
 
@@ -194,111 +256,159 @@ __global__ void __launch_bounds__(FWD_T) k_mlp_forward(const float* feats, int64
 // backward (training)
 // ---------------------------------------------------------------------------
 
-constexpr int BWD_B = 64;     // samples (= threads) per CTA
-constexpr int HP = NH + 1;    // padded row stride
+constexpr int BWD_B = 64;            // samples per CTA
+constexpr int BWD_TPS = 8;           // threads per sample (8 units each)
+constexpr int BWD_T = BWD_B * BWD_TPS;
 
 struct BwdShared {
-    float W[NPARAM];
-    float mu[NIN], isg[NIN];
-    float Z[BWD_B][NIN + 1];
-    float H1[BWD_B][HP];
-    float A2[BWD_B][HP];
-    float D2[BWD_B][HP];
-    float D1[BWD_B][HP];
+    MlpWeights m;
+    float Z[BWD_B][NIN + 4];
+    float H1[BWD_B][HP4];
+    float H2[BWD_B][HP4];
+    float D2[BWD_B][HP4];
+    float D1[BWD_B][HP4];
     float DY[BWD_B][NOUT];
-    double red[BWD_B / 32];
+    double red[BWD_T / 32];
 };
 
 // Gradient of (scale * sum over samples and outputs of (y - t)^2) with
 // respect to the (BF16-valued) weights, added into grad; the loss sum
 // (unscaled) is added into *loss.
-__global__ void __launch_bounds__(BWD_B) k_mlp_backward(const float* feats, const float* targets,
+//
+// Eight threads per sample for the two passes over the layers, then the CTA's
+// weight gradients as register tiles (8 of W2 per thread: six words read per
+// sample for 8 multiply-adds).  A thread per sample with its activations in
+// shared memory left two warps on an SM: latency-bound, 74 us at 8,192 samples.
+__global__ void __launch_bounds__(BWD_T) k_mlp_backward(const float* feats, const float* targets,
                                                         int64_t n, const uint16_t* wbits,
                                                         const float* norm, float scale,
                                                         float* grad, double* loss) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     BwdShared& S = *reinterpret_cast<BwdShared*>(smem_raw);
-    const int b = threadIdx.x;
-    load_weights(S.W, wbits);
-    if (b < NIN) {
-        S.mu[b] = norm[b];
-        S.isg[b] = 1.0f / norm[NIN + b];
-    }
+    const int tid = threadIdx.x, q = tid / BWD_TPS, e = tid % BWD_TPS;
+    load_weights(S.m, wbits, norm);
     __syncthreads();
-    const int64_t s = (int64_t)blockIdx.x * BWD_B + b;
-    double lsum = 0.0;
-    if (s < n) {
-        for (int i = 0; i < NIN; ++i) S.Z[b][i] = (feats[s * NIN + i] - S.mu[i]) * S.isg[i];
+    const int64_t s = (int64_t)blockIdx.x * BWD_B + q;
+    const bool v = s < n;
+    constexpr int U = NH / BWD_TPS;
+#pragma unroll
+    for (int i = 0; i < NIN; i += BWD_TPS)
+        S.Z[q][i + e] = v ? (feats[s * NIN + i + e] - S.m.mu[i + e]) * S.m.isg[i + e] : 0.0f;
+    __syncwarp();
+    float acc[U];
+    mlp_layer<BWD_TPS, NIN, NIN>(S.m.w1, S.m.b1, S.Z[q], e, acc);
+#pragma unroll
+    for (int t = 0; t < U; ++t) S.H1[q][t * BWD_TPS + e] = v ? fmaxf(acc[t], 0.0f) : 0.0f;
+    __syncwarp();
+    mlp_layer<BWD_TPS, NH, W2P>(S.m.w2, S.m.b2, S.H1[q], e, acc);
+    float y0 = 0.0f, y1 = 0.0f;
+#pragma unroll
+    for (int t = 0; t < U; ++t) {
+        const int o = t * BWD_TPS + e;
+        const float h2 = fmaxf(acc[t], 0.0f);
+        S.H2[q][o] = v ? h2 : 0.0f;
+        y0 = fmaf(S.m.w3[o], h2, y0);
+        y1 = fmaf(S.m.w3[NH + o], h2, y1);
+    }
+#pragma unroll
+    for (int o = BWD_TPS / 2; o > 0; o >>= 1) {
+        y0 += __shfl_xor_sync(FULL, y0, o);
+        y1 += __shfl_xor_sync(FULL, y1, o);
+    }
+    y0 += S.m.b3[0];
+    y1 += S.m.b3[1];
+    const float e0 = v ? y0 - targets[s * 2] : 0.0f, e1 = v ? y1 - targets[s * 2 + 1] : 0.0f;
+    double lsum = e == 0 ? (double)e0 * e0 + (double)e1 * e1 : 0.0;
+    const float d0 = 2.0f * e0 * scale, d1 = 2.0f * e1 * scale;
+    if (e == 0) {
+        S.DY[q][0] = d0;
+        S.DY[q][1] = d1;
+    }
+#pragma unroll
+    for (int t = 0; t < U; ++t) {
+        const int o = t * BWD_TPS + e;
+        S.D2[q][o] = acc[t] > 0.0f ? d0 * S.m.w3[o] + d1 * S.m.w3[NH + o] : 0.0f;
+    }
+    __syncwarp();
+    {  // D1 of units 8 e .. 8 e + 7
+        float g[U];
+#pragma unroll
+        for (int t = 0; t < U; ++t) g[t] = 0.0f;
+#pragma unroll 4
         for (int o = 0; o < NH; ++o) {
-            float acc = S.W[OFF_B1 + o];
-            for (int i = 0; i < NIN; ++i) acc = fmaf(S.W[OFF_W1 + o * NIN + i], S.Z[b][i], acc);
-            S.H1[b][o] = fmaxf(acc, 0.0f);
+            const float dd = S.D2[q][o];
+#pragma unroll
+            for (int t = 0; t < U; t += 4) {
+                const float4 wv = *reinterpret_cast<const float4*>(S.m.w2 + o * W2P + e * U + t);
+                g[t] = fmaf(dd, wv.x, g[t]);
+                g[t + 1] = fmaf(dd, wv.y, g[t + 1]);
+                g[t + 2] = fmaf(dd, wv.z, g[t + 2]);
+                g[t + 3] = fmaf(dd, wv.w, g[t + 3]);
+            }
         }
-        float y0 = S.W[OFF_B3], y1 = S.W[OFF_B3 + 1];
-        for (int o = 0; o < NH; ++o) {
-            float acc = S.W[OFF_B2 + o];
-            for (int i = 0; i < NH; ++i) acc = fmaf(S.W[OFF_W2 + o * NH + i], S.H1[b][i], acc);
-            S.A2[b][o] = acc;
-            const float h2 = fmaxf(acc, 0.0f);
-            y0 = fmaf(S.W[OFF_W3 + o], h2, y0);
-            y1 = fmaf(S.W[OFF_W3 + NH + o], h2, y1);
-        }
-        const float e0 = y0 - targets[s * 2], e1 = y1 - targets[s * 2 + 1];
-        lsum = (double)e0 * e0 + (double)e1 * e1;
-        const float d0 = 2.0f * e0 * scale, d1 = 2.0f * e1 * scale;
-        S.DY[b][0] = d0;
-        S.DY[b][1] = d1;
-        for (int i = 0; i < NH; ++i) {
-            const float g = d0 * S.W[OFF_W3 + i] + d1 * S.W[OFF_W3 + NH + i];
-            S.D2[b][i] = S.A2[b][i] > 0.0f ? g : 0.0f;
-        }
-        for (int i = 0; i < NH; ++i) {
-            float g = 0.0f;
-            for (int o = 0; o < NH; ++o) g = fmaf(S.D2[b][o], S.W[OFF_W2 + o * NH + i], g);
-            S.D1[b][i] = S.H1[b][i] > 0.0f ? g : 0.0f;
-        }
-    } else {
-        for (int i = 0; i < NIN; ++i) S.Z[b][i] = 0.0f;
-        for (int i = 0; i < NH; ++i) {
-            S.H1[b][i] = 0.0f;
-            S.A2[b][i] = 0.0f;
-            S.D2[b][i] = 0.0f;
-            S.D1[b][i] = 0.0f;
-        }
-        S.DY[b][0] = 0.0f;
-        S.DY[b][1] = 0.0f;
+#pragma unroll
+        for (int t = 0; t < U; ++t) S.D1[q][e * U + t] = S.H1[q][e * U + t] > 0.0f ? g[t] : 0.0f;
     }
     lsum = warp_sum(lsum);
-    if ((b & 31) == 0) S.red[b >> 5] = lsum;
+    if ((tid & 31) == 0) S.red[tid >> 5] = lsum;
     __syncthreads();
-    if (b == 0) {
+    if (tid == 0) {
         double t = 0.0;
-        for (int w = 0; w < BWD_B / 32; ++w) t += S.red[w];
+        for (int w = 0; w < BWD_T / 32; ++w) t += S.red[w];
         atomicAdd(loss, t);
     }
     // weight gradients: sums over the CTA's samples
-    for (int p = b; p < NPARAM; p += BWD_B) {
-        float acc = 0.0f;
-        if (p < OFF_B1) {
-            const int o = p / NIN, i = p % NIN;
-            for (int q = 0; q < BWD_B; ++q) acc = fmaf(S.D1[q][o], S.Z[q][i], acc);
-        } else if (p < OFF_W2) {
-            const int o = p - OFF_B1;
-            for (int q = 0; q < BWD_B; ++q) acc += S.D1[q][o];
-        } else if (p < OFF_B2) {
-            const int o = (p - OFF_W2) / NH, i = (p - OFF_W2) % NH;
-            for (int q = 0; q < BWD_B; ++q) acc = fmaf(S.D2[q][o], S.H1[q][i], acc);
-        } else if (p < OFF_W3) {
-            const int o = p - OFF_B2;
-            for (int q = 0; q < BWD_B; ++q) acc += S.D2[q][o];
-        } else if (p < OFF_B3) {
-            const int o = (p - OFF_W3) / NH, i = (p - OFF_W3) % NH;
-            for (int q = 0; q < BWD_B; ++q) acc = fmaf(S.DY[q][o], fmaxf(S.A2[q][i], 0.0f), acc);
-        } else {
-            const int o = p - OFF_B3;
-            for (int q = 0; q < BWD_B; ++q) acc += S.DY[q][o];
+    {
+        const int o = tid / 16 * 2, i = tid % 16 * 4;  // W2: units o, o + 1, inputs i .. i + 3
+        float g[8] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
+#pragma unroll 4
+        for (int b = 0; b < BWD_B; ++b) {
+            const float2 dv = *reinterpret_cast<const float2*>(&S.D2[b][o]);
+            const float4 hv = *reinterpret_cast<const float4*>(&S.H1[b][i]);
+            g[0] = fmaf(dv.x, hv.x, g[0]);
+            g[1] = fmaf(dv.x, hv.y, g[1]);
+            g[2] = fmaf(dv.x, hv.z, g[2]);
+            g[3] = fmaf(dv.x, hv.w, g[3]);
+            g[4] = fmaf(dv.y, hv.x, g[4]);
+            g[5] = fmaf(dv.y, hv.y, g[5]);
+            g[6] = fmaf(dv.y, hv.z, g[6]);
+            g[7] = fmaf(dv.y, hv.w, g[7]);
         }
-        atomicAdd(grad + p, acc);
+#pragma unroll
+        for (int t = 0; t < 8; ++t) atomicAdd(grad + OFF_W2 + (o + t / 4) * NH + i + t % 4, g[t]);
+    }
+    {
+        const int o = tid / 8, i = tid % 8 * 2;  // W1: unit o, inputs i, i + 1
+        float g0 = 0.0f, g1 = 0.0f;
+#pragma unroll 4
+        for (int b = 0; b < BWD_B; ++b) {
+            const float dd = S.D1[b][o];
+            const float2 zv = *reinterpret_cast<const float2*>(&S.Z[b][i]);
+            g0 = fmaf(dd, zv.x, g0);
+            g1 = fmaf(dd, zv.y, g1);
+        }
+        atomicAdd(grad + OFF_W1 + o * NIN + i, g0);
+        atomicAdd(grad + OFF_W1 + o * NIN + i + 1, g1);
+    }
+    if (tid < 2 * NH + NOUT * NH + NOUT) {  // b1, b2, W3, b3
+        float g = 0.0f;
+        int p;
+        if (tid < NH) {
+            p = OFF_B1 + tid;
+            for (int b = 0; b < BWD_B; ++b) g += S.D1[b][tid];
+        } else if (tid < 2 * NH) {
+            p = OFF_B2 + tid - NH;
+            for (int b = 0; b < BWD_B; ++b) g += S.D2[b][tid - NH];
+        } else if (tid < 2 * NH + NOUT * NH) {
+            const int o = (tid - 2 * NH) / NH, i = tid % NH;
+            p = OFF_W3 + o * NH + i;
+            for (int b = 0; b < BWD_B; ++b) g = fmaf(S.DY[b][o], S.H2[b][i], g);
+        } else {
+            const int o = tid - 2 * NH - NOUT * NH;
+            p = OFF_B3 + o;
+            for (int b = 0; b < BWD_B; ++b) g += S.DY[b][o];
+        }
+        atomicAdd(grad + p, g);
     }
 }
 
@@ -342,8 +452,8 @@ void launch_mlp_forward(const float* feats, int64_t n, const uint16_t* wbits, co
                         float* out, int64_t* est, float safety, const int64_t* flops,
                         const int32_t* rlo, const int32_t* rhi, cudaStream_t s) {
     if (n == 0) return;
-    int64_t blocks = (n + FWD_T - 1) / FWD_T;
-    if (blocks > 152 * 32) blocks = 152 * 32;
+    int64_t blocks = (n + FWD_S - 1) / FWD_S;
+    if (blocks > 152 * 8) blocks = 152 * 8;
     k_mlp_forward<<<(unsigned)blocks, FWD_T, 0, s>>>(feats, n, wbits, norm, out, est, safety,
                                                       flops, rlo, rhi);
     count_launches(1);
@@ -356,7 +466,7 @@ void launch_mlp_backward(const float* feats, const float* targets, int64_t n,
     const size_t smem = sizeof(BwdShared);
     cudaFuncSetAttribute(k_mlp_backward, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     const int64_t blocks = (n + BWD_B - 1) / BWD_B;
-    k_mlp_backward<<<(unsigned)blocks, BWD_B, smem, s>>>(feats, targets, n, wbits, norm, scale,
+    k_mlp_backward<<<(unsigned)blocks, BWD_T, smem, s>>>(feats, targets, n, wbits, norm, scale,
                                                           grad, loss);
     count_launches(1);
 }
