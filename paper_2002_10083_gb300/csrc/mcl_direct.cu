@@ -47,8 +47,10 @@ constexpr int DIR_W = 10240;      // rows of a window
 constexpr int DIR_HEAD = 2048;    // candidates beyond ksel that the buffer holds
 constexpr int DIR_LONG = 64;      // sources shared by all warps
 // Below this many products per source and window, the products go through
-// window buckets.
-constexpr int DIR_BUCKET_MAX = 32;
+// window buckets: a visit costs a warp a round of 128 products whatever it
+// finds (200k-vertex graph, columns of 200k-800k products: 1.32M-3.73M clocks
+// per CTA with cursors at 41 products per visit, 1.03M-2.61M with buckets).
+constexpr int DIR_BUCKET_MAX = 128;
 // The sums' low and high words are two arrays (all banks serve each), each
 // followed by 32 words that idle lanes add 0 to.
 constexpr int DIR_HI = DIR_W + 32;
@@ -497,59 +499,46 @@ __global__ void __launch_bounds__(DIR_T, DIR_MINB) k_expand_direct(DirectArgs a)
                 uint4* pl = reinterpret_cast<uint4*>(lo32 + h);
                 uint4* ph = reinterpret_cast<uint4*>(hi32 + h);
                 const uint4 l4 = *pl, h4 = *ph;
-                *pl = make_uint4(0u, 0u, 0u, 0u);
-                *ph = make_uint4(0u, 0u, 0u, 0u);
                 const unsigned xl[4] = {l4.x, l4.y, l4.z, l4.w}, xh[4] = {h4.x, h4.y, h4.z, h4.w};
                 const unsigned zb = zany ? (zbm[h >> 5] >> (h & 31)) & 15u : 0u;
-                bool big = false;
+                unsigned big = 0;  // rows to look at
 #pragma unroll
                 for (int u = 0; u < 4; ++u) {
                     const unsigned long long q = ((unsigned long long)xh[u] << 32) | xl[u];
-                    s_n += q != 0ull;
-                    big |= q >= qmin;
+                    const bool here = q != 0ull || ((zb >> u) & 1u);
+                    s_n += here;
+                    big |= here && q >= qmin ? 1u << u : 0u;
                 }
-                if (zany) {
-                    s_n = s_n + __popc(zb);
-#pragma unroll
-                    for (int u = 0; u < 4; ++u) s_n -= ((xl[u] | xh[u]) != 0u) && ((zb >> u) & 1u);
-                }
-                if (!__any_sync(FULL, big)) continue;
-                uint64_t key[4];
-                int mine = 0;
-#pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    const unsigned long long q = ((unsigned long long)xh[u] << 32) | xl[u];
-                    key[u] = 0;
-                    if (q >= qmin && (q != 0ull || ((zb >> u) & 1u))) {
+                while (__any_sync(FULL, big != 0u)) {  // one row per lane and round: few have any
+                    uint64_t key = 0;
+                    if (big) {
+                        const unsigned g = h + (unsigned)__ffs(big) - 1u;
+                        big &= big - 1u;
+                        const unsigned long long q = ((unsigned long long)hi32[g] << 32) | lo32[g];
                         const float v = fx.value(q);
                         if (v >= theta) {
                             ++s_t;
                             s_mt += q;
                         }
-                        key[u] = make_key(v, r0 + (int)h + u);
+                        key = make_key(v, r0 + (int)g);
                     }
-                    mine += key[u] > tau;
-                }
-                if (!__any_sync(FULL, mine > 0)) continue;
-                // candidates to the buffer, in any order; those it has no room for to the spill
-                int incl = mine;
-#pragma unroll
-                for (int o = 1; o < 32; o <<= 1) {
-                    const int y = __shfl_up_sync(FULL, incl, o);
-                    if (lane >= o) incl += y;
-                }
-                int base = 0;
-                if (lane == 31) base = atomicAdd(&ds->cand, incl);
-                int at = ntop + __shfl_sync(FULL, base, 31) + incl - mine;
-#pragma unroll
-                for (int u = 0; u < 4; ++u)
-                    if (key[u] > tau) {
-                        if (at < topcap)
-                            top[at] = key[u];
-                        else
-                            spill[at - topcap] = key[u];
-                        ++at;
+                    // candidates to the buffer, in any order; those it has no room for to the spill
+                    const bool take = key > tau;
+                    const unsigned m = __ballot_sync(FULL, take);
+                    if (m) {
+                        int base = 0;
+                        if (lane == 0) base = atomicAdd(&ds->cand, __popc(m));
+                        const int at = ntop + __shfl_sync(FULL, base, 0) + __popc(m & lanemask_lt());
+                        if (take) {
+                            if (at < topcap)
+                                top[at] = key;
+                            else
+                                spill[at - topcap] = key;
+                        }
                     }
+                }
+                *pl = make_uint4(0u, 0u, 0u, 0u);
+                *ph = make_uint4(0u, 0u, 0u, 0u);
             }
             __syncthreads();
             const int have = ntop + ds->cand;
