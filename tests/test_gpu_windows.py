@@ -1,6 +1,7 @@
 """The numeric pass's ways to hold a column's sums, at the sizes where they can
 go wrong, against each other (the sums are exact, so every way gives the same
 bits) and against the FP64 oracle."""
+import numpy as np
 import pytest
 
 from paper_2002_10083_gb300 import synth
@@ -77,3 +78,53 @@ def test_direct_windows_equal_hashed_ones(ctx, n, d, K, theta, zeros, budget):
     assert nnz_b == ctx.stats()["nnz_b"] and ch == ch_ref
     assert torch.equal(out.colptr, ref.colptr) and torch.equal(out.rowidx, ref.rowidx)
     assert torch.equal(out.val.view(torch.int32), ref.val.view(torch.int32))
+
+
+# several passes of sums per window, 64-bit global atomics (more than four passes), the large
+# bitmap, several bitmap windows; merges of 2 to 4 and a last merge of leftovers
+@pytest.mark.parametrize("n,d,ns", [(12000, 130, 4), (45000, 250, 2), (140000, 20, 3), (600000, 5, 2), (33, 5, 7)])
+def test_split_shapes_equal_one_pass(ctx, n, d, ns):
+    from paper_2002_10083_gb300 import mcl
+    A = _random(n, d, seed=n, zeros=n < 20000)
+    prm = mcl.Params(threshold=1e-4, select_k=200, recover_pct=0.9, inflation=2.0)
+    ref, ch_ref = ctx.expand(A, prm)
+    out, ch, _ = ctx.expand_split(A, prm, ns)
+    assert ch == ch_ref and torch.equal(out.colptr, ref.colptr) and torch.equal(out.rowidx, ref.rowidx)
+    assert torch.equal(out.val.view(torch.int32), ref.val.view(torch.int32))
+
+
+# both CTA sizes, more sources than one batch lists, several bitmap windows
+@pytest.mark.parametrize("n,d", [(1, 1), (100, 7), (4500, 700), (17000, 20), (30000, 60), (600000, 5)])
+def test_symbolic_shapes(ctx, n, d):
+    import scipy.sparse as sp
+    A = _random(n, d, seed=3 * n + d)
+    P = sp.csc_matrix((torch.ones(A.nnz).numpy(), A.rowidx.cpu().numpy(), A.colptr.cpu().numpy()), shape=(n, n))
+    B = P @ P
+    flops, nnz = ctx.symbolic(A)
+    assert (nnz.cpu().numpy() == B.indptr[1:] - B.indptr[:-1]).all()
+    assert (flops.cpu().numpy() == np.asarray(B.sum(axis=0)).ravel()).all()
+
+
+@pytest.mark.parametrize("n", [1, 31, 33, 64, 65, 5000])
+def test_mlp_sample_counts(ctx, n):
+    """Forward: a sample's outputs do not depend on the samples beside it.  Backward: against
+    FP64; sums of n FP32 gradients, each a few hundred roundings (2^-24) of terms near its size."""
+    from paper_2002_10083_gb300 import estimator, mcl
+    w_bits, norm, _, _ = estimator.load()
+    w = torch.as_tensor(w_bits.astype("int16")).cuda()
+    norm = torch.from_numpy(norm).cuda()
+    g = torch.Generator(device="cuda").manual_seed(n)
+    feats = (norm[:16] + norm[16:] * torch.randn(5000, 16, generator=g, device="cuda")).contiguous()
+    t = torch.randn(n, 2, generator=g, device="cuda")
+    y = ctx.mlp_forward(feats[:n].contiguous(), w, norm)
+    assert torch.equal(y, ctx.mlp_forward(feats, w, norm)[:n])
+    grad, loss = torch.zeros(mcl.MLP_NPARAM, device="cuda"), torch.zeros(1, dtype=torch.float64, device="cuda")
+    ctx.mlp_backward(feats[:n].contiguous(), t, w, norm, 1.0 / n, grad, loss)
+    p = w.view(torch.bfloat16).double().requires_grad_()
+    z = (feats[:n].double() - norm[:16].double()) / norm[16:].double()
+    h = torch.relu(z @ p[:1024].view(64, 16).t() + p[1024:1088])
+    h = torch.relu(h @ p[1088:5184].view(64, 64).t() + p[5184:5248])
+    total = (h @ p[5248:5376].view(2, 64).t() + p[5376:] - t.double()).square().sum()
+    (total / n).backward()
+    assert abs(float(loss) / float(total.detach()) - 1) < 1e-5
+    assert float((grad.double() - p.grad).abs().max()) < 1e-4 * float(p.grad.abs().max())
