@@ -919,7 +919,7 @@ mcl_status mcl_prune_select_recover(mcl_ctx* c, const mcl_csc* B, const mcl_para
     ExpandBuffers b = buffers(c);
     const CscView Bv = view(B);
     CUDA_TRY(c, cudaMemsetAsync(c->ctr.p, 0, sizeof(DevCounters), s));
-    launch_colstats(Bv, pp, b, c->num_sms, s);  // validation
+    launch_colstats(Bv, pp, b, c->num_sms, s, false);  // validation, column sums
     if ((st = read_counters(c, s))) return st;
     if ((st = err_flags(c, c->hctr->err))) return st;
     launch_prune_cap(Bv, pp.Krec, b, s);

@@ -380,6 +380,17 @@ __device__ __forceinline__ float u64_to_float(unsigned long long x) {
     return __fmul_rn(__uint2float_rn(lead), __int_as_float((32 - z + 127) << 23));
 }
 
+// FP32 to FP64 by shifting the fields: the conversion runs on the FP64 pipe
+// (see u64_to_float), which the sums need.  Zeros, subnormals, infinities and
+// NaN take the conversion.
+__device__ __forceinline__ double float_to_double(float v) {
+    const unsigned b = __float_as_uint(v);
+    const unsigned e = (b >> 23) & 255u;
+    if (e == 0u || e == 255u) return (double)v;
+    const unsigned hi = (b & 0x80000000u) | (((b & 0x7FFFFFFFu) >> 3) + 0x38000000u);
+    return __hiloint2double((int)hi, (int)(b << 29));
+}
+
 // Fixed-point scale of a column: q = trunc(v * 2^f), x = q * is1 * is2 (two
 // exact power-of-two factors, each a normal FP32 number).
 struct FixScale {

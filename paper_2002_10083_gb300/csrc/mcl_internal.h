@@ -107,7 +107,7 @@ long long launches_total();
 
 // --- launchers (mcl_kernels.cu) ---
 void launch_colstats(const CscView& A, const PruneParams& pp, const ExpandBuffers& b,
-                     int num_sms, cudaStream_t s);
+                     int num_sms, cudaStream_t s, bool product = true);
 int64_t scan_tmp_len_for(int64_t n);
 template <typename TIn>
 void launch_exclusive_scan(const TIn* in, int64_t n, int64_t* out, int64_t* tmp,

@@ -38,7 +38,10 @@ __device__ __forceinline__ void set_err(DevCounters* c, unsigned bit) { atomicOr
 // Warp per column.  Checks colptr bounds, row range and strict order,
 // values finite and >= 0; every read is guarded so malformed input only
 // raises flags.  Then flops_j = sum_{k in col j} nnz(col k), the span
-// [rlo_j, rhi_j] of product rows and cap_j = min(Krec, flops_j, span_j).
+// [rlo_j, rhi_j] of product rows and cap_j = min(Krec, flops_j, span_j)
+// (PRODUCT; a caller that forms no product wants the checks and the column
+// sums alone, without the four gathers per entry).
+template <bool PRODUCT>
 __global__ void k_colstats(CscView A, int32_t Krec, ExpandBuffers b) {
     const int lane = threadIdx.x & 31;
     const int64_t gw = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -67,16 +70,18 @@ __global__ void k_colstats(CscView A, int32_t Krec, ExpandBuffers b) {
         int mn = INT_MAX, mx = -1;
         unsigned bad = 0;
         double csum = 0.0;
+#pragma unroll 4
         for (int64_t p = cb + lane; p < ce; p += 32) {
             const int k = A.rowidx[p];
             const float v = A.val[p];
-            csum += (double)v;
+            csum += float_to_double(v);
             if (!(v >= 0.0f) || !(v <= FLT_MAX)) bad |= ERR_VALUE;
             if (p > cb && A.rowidx[p - 1] >= k) bad |= ERR_ROW_ORDER;
             if ((unsigned)k >= (unsigned)A.n) {
                 bad |= ERR_ROW_RANGE;
                 continue;
             }
+            if (!PRODUCT) continue;
             const int64_t ks = A.colptr[k], ke = A.colptr[k + 1];
             if (ks < 0 || ke < ks || ke > A.nnz) {
                 bad |= ERR_COLPTR;
@@ -122,13 +127,16 @@ __global__ void k_colstats(CscView A, int32_t Krec, ExpandBuffers b) {
 }
 
 void launch_colstats(const CscView& A, const PruneParams& pp, const ExpandBuffers& b, int num_sms,
-                     cudaStream_t s) {
+                     cudaStream_t s, bool product) {
     if (A.n == 0) return;
     int64_t warps = A.n;
     int64_t blocks = (warps * 32 + 255) / 256;
     int64_t maxb = (int64_t)num_sms * 8;
     if (blocks > maxb) blocks = maxb;
-    k_colstats<<<(unsigned)blocks, 256, 0, s>>>(A, pp.Krec, b);
+    if (product)
+        k_colstats<true><<<(unsigned)blocks, 256, 0, s>>>(A, pp.Krec, b);
+    else
+        k_colstats<false><<<(unsigned)blocks, 256, 0, s>>>(A, pp.Krec, b);
     count_launches(1);
 }
 
@@ -712,7 +720,11 @@ void launch_finalize_stats(int32_t n, const ExpandBuffers& b, cudaStream_t s) {
     count_launches(1);
 }
 
-// Warp per column: v <- v^r / sum v^r (FP32 power, FP64 sum).
+// Warp per column: v <- v^r / sum v^r (FP32 power, FP64 sum).  The quotient is
+// u (hi + lo) with 1 / sum as two FP32 numbers, one rounding of a product that
+// is exact to 2^-48: an FP64 division per entry ran at the FP64 pipe's 2 lanes
+// per clock and SM (351 us for 13.5M entries; 8 bytes of traffic each take 32).
+// Sums whose reciprocal or whose terms leave FP32's range divide in FP64.
 __global__ void k_inflate_normalize(int32_t n, const int64_t* colptr, float* val, float r) {
     const int lane = threadIdx.x & 31;
     const int64_t gw = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -720,11 +732,22 @@ __global__ void k_inflate_normalize(int32_t n, const int64_t* colptr, float* val
     for (int64_t j = gw; j < n; j += nw) {
         const int64_t cb = colptr[j], ce = colptr[j + 1];
         double s = 0.0;
-        for (int64_t p = cb + lane; p < ce; p += 32) s += (double)inflate_value(val[p], r);
+#pragma unroll 4
+        for (int64_t p = cb + lane; p < ce; p += 32) s += float_to_double(inflate_value(val[p], r));
         s = warp_sum(s);
-        for (int64_t p = cb + lane; p < ce; p += 32) {
-            const float u = inflate_value(val[p], r);
-            val[p] = s > 0.0 ? (float)((double)u / s) : 0.0f;
+        if (s > 1e-25 && s < 1e25) {
+            const double inv = 1.0 / s;
+            const float hi = (float)inv, lo = (float)(inv - (double)hi);
+#pragma unroll 4
+            for (int64_t p = cb + lane; p < ce; p += 32) {
+                const float u = inflate_value(val[p], r);
+                val[p] = fmaf(u, hi, __fmul_rn(u, lo));
+            }
+        } else {
+            for (int64_t p = cb + lane; p < ce; p += 32) {
+                const float u = inflate_value(val[p], r);
+                val[p] = s > 0.0 ? (float)((double)u / s) : 0.0f;
+            }
         }
     }
 }
@@ -747,12 +770,16 @@ __global__ void k_chaos(int32_t n, const int64_t* colptr, const float* val, doub
     double best = 0.0;
     for (int64_t j = gw; j < n; j += nw) {
         const int64_t cb = colptr[j], ce = colptr[j + 1];
-        double mx = 0.0, sq = 0.0;
+        float mf = 0.0f;
+        double sq = 0.0;
+#pragma unroll 4
         for (int64_t p = cb + lane; p < ce; p += 32) {
-            const double a = (double)val[p];
-            mx = a > mx ? a : mx;
+            const float v = val[p];
+            const double a = float_to_double(v);
+            mf = fmaxf(mf, v);
             sq += a * a;
         }
+        double mx = (double)mf;
         mx = warp_max(mx);
         sq = warp_sum(sq);
         double c = mx - sq;

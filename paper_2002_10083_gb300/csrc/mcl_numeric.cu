@@ -729,130 +729,110 @@ void launch_numeric(int conf, const CscView& A, const PruneParams& pp, const Exp
 // a column's entries are already row-ordered)
 // ---------------------------------------------------------------------------
 
-constexpr int PR_T = 256, PR_VC = 2048;
+constexpr int PR_T = 256, PR_IPT = 8, PR_VC = PR_T * PR_IPT;
 
-struct ColumnChunkEnum {
-    const int32_t* rows;
-    const float* vals;
-    int i0, i1;
-    __device__ int count(uint64_t tau) const {
-        int c = 0;
-        for (int i = i0; i < i1; ++i) c += make_key(vals[i], rows[i]) > tau;
-        return c;
-    }
-    __device__ void emit(uint64_t tau, uint64_t* dst, int base) const {
-        dst += base;
-        for (int i = i0; i < i1; ++i) {
-            const uint64_t k = make_key(vals[i], rows[i]);
-            if (k > tau) *dst++ = k;
-        }
-    }
+struct PruneShared {
+    WinShared w;
+    int cnt[2][PR_IPT * PR_T / 32];  // candidates per round and warp, by chunk parity
 };
 
-struct PruneArgs2 {
-    CscView B;
-    PruneParams pp;
-    ExpandBuffers b;
-};
-
-__global__ void __launch_bounds__(PR_T) k_prune(PruneArgs2 a) {
-    extern __shared__ __align__(16) unsigned char smem[];
-    const int ksel = a.pp.ksel;
-    const int topcap = ksel + PR_VC;
-    uint64_t* top = reinterpret_cast<uint64_t*>(smem);
-    unsigned* hist = reinterpret_cast<unsigned*>(top + topcap);
-    unsigned long long* mhist = reinterpret_cast<unsigned long long*>(hist + 256);
-    WinShared* sh = reinterpret_cast<WinShared*>(mhist + 256);
-    const int tid = threadIdx.x;
-    const CscView& B = a.B;
-    const ExpandBuffers& b = a.b;
-    for (;;) {
-        if (tid == 0) sh->item = atomicAdd(&b.ctr->work_ctr, 1);
-        __syncthreads();
-        const int64_t j = sh->item;
-        __syncthreads();
-        if (j >= B.n) break;
-        const int64_t cb = B.colptr[j], ce = B.colptr[j + 1];
-        int ntop = 0;
-        uint64_t tau = 0;
-        double s_sum = 0.0, s_mt = 0.0;
-        long long s_t = 0;
-        for (int64_t base = cb; base < ce; base += PR_VC) {
-            const int cnt = (int)min((int64_t)PR_VC, ce - base);
-            const int per = (cnt + PR_T - 1) / PR_T;
-            ColumnChunkEnum en{B.rowidx + base, B.val + base, min(cnt, tid * per),
-                               min(cnt, tid * per + per)};
-            int c = 0;
-            for (int i = en.i0; i < en.i1; ++i) {
-                const float v = en.vals[i];
-                s_sum += (double)v;
-                if (v >= a.pp.theta) {
+// The candidates and statistics of one column of m entries, in row order.
+// load(i, &row, &q) gives entry i with its fixed-point value; a chunk of 2,048
+// entries is read once, coalesced, and kept in registers while the positions
+// of its candidates are counted (ballots per round and warp, in entry order).
+template <class Load>
+__device__ __forceinline__ void prune_candidates(int64_t m, const FixScale& fx, float theta, Load load,
+                                                 uint64_t* top, int topcap, int ksel, unsigned* hist,
+                                                 PruneShared* ps, int& ntop, long long& s_t,
+                                                 unsigned long long& s_mt) {
+    constexpr int NW = PR_T / 32;
+    static_assert(PR_IPT * NW == 64, "two counts per lane");
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    uint64_t tau = 0;
+    int par = 0;
+    for (int64_t base = 0; base < m; base += PR_VC, par ^= 1) {
+        uint64_t key[PR_IPT];
+#pragma unroll
+        for (int u = 0; u < PR_IPT; ++u) {
+            const int64_t i = base + u * PR_T + tid;
+            key[u] = 0;
+            if (i < m) {
+                int row;
+                float v;
+                unsigned long long q;
+                load(i, row, v, q);
+                if (v >= theta) {
                     ++s_t;
-                    s_mt += (double)v;
+                    s_mt += q;
                 }
-                c += make_key(v, en.rows[i]) > tau;
+                key[u] = make_key(v, row);
             }
-            append_candidates<PR_T, 8>(en, top, topcap, ksel, ntop, tau, c, hist, sh);
         }
-        double dv[2] = {s_sum, s_mt};
-        long long qv[1] = {s_t};
-        block_sum<PR_T>(dv, 2, qv, 1, &sh->bs);
-        int mstar = 0;
-        double ch = 0.0;
-        const int64_t obase = b.off[j];
-        finish_column<PR_T, 8, true>(top, ntop, topcap, a.pp, dv[0], dv[1], qv[0], b.cap[j],
-                                     b.tmp_row + (obase - b.tmp_off0),
-                                     b.tmp_val + (obase - b.tmp_off0), hist, mhist, sh, b.ctr, 0,
-                                     0, nullptr, &mstar, &ch);
-        if (tid == 0) {
-            b.kept[j] = mstar;
-            b.chaos[j] = ch;
-            b.bnnz[j] = ce - cb;
+        auto count = [&](int* cnt, int& at) {  // at: this lane's two counts' exclusive offset
+#pragma unroll
+            for (int u = 0; u < PR_IPT; ++u) {
+                const unsigned b = __ballot_sync(FULL, key[u] > tau);
+                if (lane == 0) cnt[u * NW + warp] = __popc(b);
+            }
+            __syncthreads();
+            const int c0 = cnt[2 * lane], c1 = cnt[2 * lane + 1];
+            int incl = c0 + c1;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int y = __shfl_up_sync(FULL, incl, o);
+                if (lane >= o) incl += y;
+            }
+            at = incl - c0 - c1;
+            return __shfl_sync(FULL, incl, 31);
+        };
+        int* cnt = ps->cnt[par];
+        int at;
+        int C = count(cnt, at);
+        if (ntop + C > topcap) {  // C <= PR_VC = topcap - ksel, so ntop > ksel here
+            tau = block_select_count<PR_T>(top, ntop, top, 0, ksel, hist, &ps->w.bs);
+            ntop = compact_stable<PR_T, PR_IPT>(top, ntop, tau, ps->w.wsm);
+            C = count(cnt, at);
         }
+#pragma unroll
+        for (int u = 0; u < PR_IPT; ++u) {
+            const int f = u * NW + warp;  // its offset: lane f / 2, plus the lane's first count if odd
+            int o = __shfl_sync(FULL, at, f >> 1);
+            if (f & 1) o += cnt[f - 1];
+            const bool take = key[u] > tau;
+            const unsigned b = __ballot_sync(FULL, take);
+            if (take) top[ntop + o + __popc(b & lanemask_lt())] = key[u];
+        }
+        ntop += C;
+        __syncthreads();
     }
 }
 
-// The prune rule, inflation and renormalisation of a merged product whose
-// entries are the exact 64-bit fixed-point sums of the numeric pass
-// (rows sorted per column; column j's scale from the column sum bsum[j]):
-// the statistics and keys of the numeric pass, so the same iteration.
-struct FixedChunkEnum {
-    const int32_t* rows;
-    const unsigned long long* q;
-    FixScale fx;
-    int i0, i1;
-    __device__ int count(uint64_t tau) const {
-        int c = 0;
-        for (int i = i0; i < i1; ++i) c += make_key(fx.value(q[i]), rows[i]) > tau;
-        return c;
-    }
-    __device__ void emit(uint64_t tau, uint64_t* dst, int base) const {
-        dst += base;
-        for (int i = i0; i < i1; ++i) {
-            const uint64_t k = make_key(fx.value(q[i]), rows[i]);
-            if (k > tau) *dst++ = k;
-        }
-    }
-};
-
-struct PruneFixedArgs {
+// FIXED: a merged product whose entries are the exact 64-bit fixed-point sums
+// of the numeric pass (rows sorted per column; column j's scale from the
+// column sum bsum[j]): the statistics and keys of the numeric pass, so the
+// same iteration.  Otherwise FP32 values, whose mass at or above the threshold
+// is summed in the fixed point of the column's own sum.
+struct PruneArgs {
     int32_t n;
     const int64_t* colptr;
     const int32_t* rowidx;
+    const float* val;
     const unsigned long long* q;
-    const double* bsum;
+    const double* sum;
     PruneParams pp;
     ExpandBuffers b;
 };
 
-__global__ void __launch_bounds__(PR_T) k_prune_fixed(PruneFixedArgs a) {
+template <bool FIXED>
+__global__ void __launch_bounds__(PR_T) k_prune(PruneArgs a) {
     extern __shared__ __align__(16) unsigned char smem[];
     const int ksel = a.pp.ksel;
     const int topcap = ksel + PR_VC;
     uint64_t* top = reinterpret_cast<uint64_t*>(smem);
     unsigned* hist = reinterpret_cast<unsigned*>(top + topcap);
     unsigned long long* mhist = reinterpret_cast<unsigned long long*>(hist + 256);
-    WinShared* sh = reinterpret_cast<WinShared*>(mhist + 256);
+    PruneShared* ps = reinterpret_cast<PruneShared*>(mhist + 256);
+    WinShared* sh = &ps->w;
     const int tid = threadIdx.x;
     const ExpandBuffers& b = a.b;
     for (;;) {
@@ -861,31 +841,29 @@ __global__ void __launch_bounds__(PR_T) k_prune_fixed(PruneFixedArgs a) {
         const int64_t j = sh->item;
         __syncthreads();
         if (j >= a.n) break;
-        const int64_t cb = a.colptr[j], ce = a.colptr[j + 1];
-        const double S = a.bsum[j];
+        const int64_t cb = a.colptr[j], m = a.colptr[j + 1] - cb;
+        const double S = a.sum[j];
         FixScale fx;
         fx.init(S);
         int ntop = 0;
-        uint64_t tau = 0;
         unsigned long long s_mt = 0;
         long long s_t = 0;
-        for (int64_t base = cb; base < ce; base += PR_VC) {
-            const int cnt = (int)min((int64_t)PR_VC, ce - base);
-            const int per = (cnt + PR_T - 1) / PR_T;
-            FixedChunkEnum en{a.rowidx + base, a.q + base, fx, min(cnt, tid * per),
-                              min(cnt, tid * per + per)};
-            int c = 0;
-            for (int i = en.i0; i < en.i1; ++i) {
-                const unsigned long long qi = en.q[i];
-                const float v = fx.value(qi);
-                if (v >= a.pp.theta) {
-                    ++s_t;
-                    s_mt += qi;
+        const int32_t* rows = a.rowidx + cb;
+        const float* vals = FIXED ? nullptr : a.val + cb;
+        const unsigned long long* qs = FIXED ? a.q + cb : nullptr;
+        prune_candidates(
+            m, fx, a.pp.theta,
+            [&](int64_t i, int& row, float& v, unsigned long long& q) {
+                row = rows[i];
+                if (FIXED) {
+                    q = qs[i];
+                    v = fx.value(q);
+                } else {
+                    v = vals[i];
+                    q = fx.qv(v);
                 }
-                c += make_key(v, en.rows[i]) > tau;
-            }
-            append_candidates<PR_T, 8>(en, top, topcap, ksel, ntop, tau, c, hist, sh);
-        }
+            },
+            top, topcap, ksel, hist, ps, ntop, s_t, s_mt);
         double dv[1] = {0.0};
         long long qv[2] = {s_t, (long long)s_mt};
         block_sum<PR_T>(dv, 0, qv, 2, &sh->bs);
@@ -900,40 +878,36 @@ __global__ void __launch_bounds__(PR_T) k_prune_fixed(PruneFixedArgs a) {
         if (tid == 0) {
             b.kept[j] = mstar;
             b.chaos[j] = ch;
-            b.bnnz[j] = ce - cb;
+            b.bnnz[j] = m;
         }
     }
+}
+
+template <bool FIXED>
+static void prune_launch(const PruneArgs& a, int num_sms, cudaStream_t s) {
+    if (a.n == 0) return;
+    const size_t smem = (size_t)(a.pp.ksel + PR_VC) * 8 + 256 * 4 + 256 * 8 + sizeof(PruneShared);
+    cudaFuncSetAttribute(k_prune<FIXED>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    int occ = 0;
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_prune<FIXED>, PR_T, smem);
+    if (occ < 1) occ = 1;
+    int grid = occ * num_sms;
+    if ((int64_t)grid > a.n) grid = (int)a.n;
+    cudaMemsetAsync(&a.b.ctr->work_ctr, 0, sizeof(int), s);
+    k_prune<FIXED><<<grid, PR_T, smem, s>>>(a);
+    count_launches(1);
 }
 
 void launch_prune_fixed(int32_t n, const int64_t* colptr, const int32_t* rowidx,
                         const unsigned long long* q, const double* bsum, const PruneParams& pp,
                         const ExpandBuffers& b, int num_sms, cudaStream_t s) {
-    if (n == 0) return;
-    const size_t smem = (size_t)(pp.ksel + PR_VC) * 8 + 256 * 4 + 256 * 8 + sizeof(WinShared);
-    cudaFuncSetAttribute(k_prune_fixed, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    int occ = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_prune_fixed, PR_T, smem);
-    if (occ < 1) occ = 1;
-    int grid = occ * num_sms;
-    if ((int64_t)grid > n) grid = (int)n;
-    cudaMemsetAsync(&b.ctr->work_ctr, 0, sizeof(int), s);
-    k_prune_fixed<<<grid, PR_T, smem, s>>>(PruneFixedArgs{n, colptr, rowidx, q, bsum, pp, b});
-    count_launches(1);
+    prune_launch<true>(PruneArgs{n, colptr, rowidx, nullptr, q, bsum, pp, b}, num_sms, s);
 }
 
+// Column sums of B in b.colsum.
 void launch_prune(const CscView& B, const PruneParams& pp, const ExpandBuffers& b, int num_sms,
                   cudaStream_t s) {
-    if (B.n == 0) return;
-    const size_t smem = (size_t)(pp.ksel + PR_VC) * 8 + 256 * 4 + 256 * 8 + sizeof(WinShared);
-    cudaFuncSetAttribute(k_prune, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    int occ = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_prune, PR_T, smem);
-    if (occ < 1) occ = 1;
-    int grid = occ * num_sms;
-    if ((int64_t)grid > B.n) grid = (int)B.n;
-    cudaMemsetAsync(&b.ctr->work_ctr, 0, sizeof(int), s);
-    k_prune<<<grid, PR_T, smem, s>>>(PruneArgs2{B, pp, b});
-    count_launches(1);
+    prune_launch<false>(PruneArgs{B.n, B.colptr, B.rowidx, B.val, nullptr, b.colsum, pp, b}, num_sms, s);
 }
 
 }  // namespace mcl
