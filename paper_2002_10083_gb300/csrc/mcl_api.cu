@@ -225,6 +225,12 @@ mcl_status read_counters(mcl_ctx* c, cudaStream_t s) {
     return MCL_OK;
 }
 
+// after a kernel that has written the mirror itself
+mcl_status sync_stream(mcl_ctx* c, cudaStream_t s) {
+    CUDA_TRY(c, cudaStreamSynchronize(s));
+    return MCL_OK;
+}
+
 double chaos_from_bits(unsigned long long b) {
     double d;
     memcpy(&d, &b, 8);
@@ -451,15 +457,23 @@ static mcl_status expand_impl(mcl_ctx* c, const mcl_csc* A, const mcl_params* pr
         launch_cohen(Av, c->cohen_r, c->cohen_seed, (float*)c->cohen_m.p, (float*)c->cohen_e.p, s);
         launch_cohen_to_est((int32_t)n, (const float*)c->cohen_e.p, 1.0f, b, s);
     } else {
-        launch_symbolic(Av, b, b.est, c->num_sms, grid_max, s);
-        // exact counts bound each column's output: cap_j = min(cap_j, nnz_j)
-        launch_cap_tighten((int32_t)n, b.est, b.cap, active, s);
+        launch_symbolic(Av, b, b.est, c->num_sms, grid_max, s, true);
     }
-    if (c->est_milli != 1000) launch_scale_est(A->n, b.est, c->est_milli, s);
-    if ((st = check_launch(c, "estimate"))) return st;
-    launch_exclusive_scan<int64_t>(b.cap, n, b.off, b.scan_tmp, &b.ctr->cap_total, s);
-    cudaEventRecord(c->ev[2], s);
-    if ((st = read_counters(c, s))) return st;
+    const bool exact = sizing == 0;  // exact counts bound each column's output: cap_j = min(cap_j, nnz_j)
+    const bool small = plan_is_small(n) && c->est_milli == 1000 && c->phase_budget == 0;
+    if (small) {
+        launch_plan_small((int32_t)n, exact, -1, pp, b, c->conf_mask, c->hctr_dev, s);
+        if ((st = check_launch(c, "estimate"))) return st;
+        cudaEventRecord(c->ev[2], s);
+        CUDA_TRY(c, cudaStreamSynchronize(s));
+    } else {
+        if (exact) launch_cap_tighten((int32_t)n, b.est, b.cap, active, s);
+        if (c->est_milli != 1000) launch_scale_est(A->n, b.est, c->est_milli, s);
+        if ((st = check_launch(c, "estimate"))) return st;
+        launch_exclusive_scan<int64_t>(b.cap, n, b.off, b.scan_tmp, &b.ctr->cap_total, s);
+        cudaEventRecord(c->ev[2], s);
+        if ((st = read_counters(c, s))) return st;
+    }
     const int64_t cap_total = (int64_t)c->hctr->cap_total;
     // column batches (phases): the output staging of a batch fits the budget
     int64_t budget_entries = c->phase_budget > 0 ? (int64_t)(c->phase_budget / 8) : 0;
@@ -475,7 +489,7 @@ static mcl_status expand_impl(mcl_ctx* c, const mcl_csc* A, const mcl_params* pr
     // ---- binning + numeric over the columns a mask selects ----
     int used = 0;
     auto run_numeric = [&](const ExpandBuffers& bb) -> mcl_status {
-        launch_binning(Av, pp, bb, c->conf_mask, s);
+        if (!small) launch_binning(Av, pp, bb, c->conf_mask, s);
         // product buckets for multi-window columns (optional: without them the windows
         // walk per-source cursors); the two configurations run one after the other and
         // share them
@@ -492,7 +506,11 @@ static mcl_status expand_impl(mcl_ctx* c, const mcl_csc* A, const mcl_params* pr
         for (int q = NCONF - 1; q >= 0; --q) {
             if (!conf_on(c, q)) continue;
             const int g = numeric_grid(q, pp, c->num_sms);
-            launch_numeric(q, Av, pp, with_buckets(c, bb, q, g, bkt_bytes), g, s);
+            // the host has a small plan's column counts; none binned: no launch
+            int cols = small ? c->hctr->bin_off[(q + 1) * NZ] - c->hctr->bin_off[q * NZ] : g;
+            if (q == CONF_DIRECT && c->hctr->max_span <= DIRECT_MIN_SPAN) cols = 0;
+            if (cols > 0)
+                launch_numeric(q, Av, pp, with_buckets(c, bb, q, g, bkt_bytes), cols < g ? cols : g, s);
             ++used;
         }
         return check_launch(c, "numeric");
@@ -506,18 +524,22 @@ static mcl_status expand_impl(mcl_ctx* c, const mcl_csc* A, const mcl_params* pr
         cudaEventRecord(c->ev[3], s);
         if ((st = run_numeric(b))) return st;
         cudaEventRecord(c->ev[4], s);
-        launch_finalize_stats(A->n, b, s);
+        if (!small) launch_finalize_stats(A->n, b, s);
         // ---- output ----
         colptr_out = (int64_t*)dev_alloc(c, (size_t)(n + 1) * 8, s);
         if (!colptr_out) return fail(c, MCL_ERR_OOM, "output colptr allocation failed");
-        if (active) launch_fill_inactive(Av, active, b.kept, s);  // carried columns keep their length
-        launch_exclusive_scan<int32_t>(b.kept, n, colptr_out, b.scan_tmp, &b.ctr->nnz_out, s);
+        if (small) {
+            launch_result_small(Av, b, colptr_out, c->hctr_dev, s);
+        } else {
+            if (active) launch_fill_inactive(Av, active, b.kept, s);  // carried columns keep their length
+            launch_exclusive_scan<int32_t>(b.kept, n, colptr_out, b.scan_tmp, &b.ctr->nnz_out, s);
+        }
         if ((st = check_launch(c, "scan"))) {
             dev_free(c, colptr_out, s);
             return st;
         }
         cudaEventRecord(c->ev[5], s);
-        if ((st = read_counters(c, s)) || (st = err_flags(c, c->hctr->err))) {
+        if ((st = small ? sync_stream(c, s) : read_counters(c, s)) || (st = err_flags(c, c->hctr->err))) {
             dev_free(c, colptr_out, s);
             return st;
         }
@@ -1159,6 +1181,7 @@ static void graph_release(mcl_ctx* c, GraphRun& G, cudaStream_t s, int keep) {
 // One batched iteration in -> out on stream s: kernel launches and memsets
 // only (capturable).  in.nnz is read as a capacity bound.
 static void static_iteration(mcl_ctx* c, const mcl_params* prm, const PruneParams& pp, int ncomp,
+                             int64_t max_comp,
                              const mcl_csc& in, const mcl_csc& out, int64_t cap, int sizing,
                              int64_t stride, cudaStream_t s) {
     const int32_t n = in.n;
@@ -1186,21 +1209,30 @@ static void static_iteration(mcl_ctx* c, const mcl_params* prm, const PruneParam
         launch_cohen(Av, c->cohen_r, c->cohen_seed, (float*)c->cohen_m.p, (float*)c->cohen_e.p, s);
         launch_cohen_to_est(n, (const float*)c->cohen_e.p, 1.0f, b, s);
     } else {
-        launch_symbolic(Av, b, b.est, c->num_sms, grid_max, s);
-        launch_cap_tighten(n, b.est, b.cap, b.active, s);
+        launch_symbolic(Av, b, b.est, c->num_sms, grid_max, s, true);
     }
-    if (c->est_milli != 1000) launch_scale_est(n, b.est, c->est_milli, s);
-    launch_exclusive_scan<int64_t>(b.cap, n, b.off, b.scan_tmp, &b.ctr->cap_total, s);
-    launch_staging_guard(b.ctr, cap, s);
-    launch_binning(Av, pp, b, c->conf_mask, s);
+    const bool small = plan_is_small(n) && c->est_milli == 1000;
+    if (small) {
+        launch_plan_small(n, sizing == 0, cap, pp, b, c->conf_mask, nullptr, s);
+    } else {
+        if (sizing == 0) launch_cap_tighten(n, b.est, b.cap, b.active, s);
+        if (c->est_milli != 1000) launch_scale_est(n, b.est, c->est_milli, s);
+        launch_exclusive_scan<int64_t>(b.cap, n, b.off, b.scan_tmp, &b.ctr->cap_total, s);
+        launch_staging_guard(b.ctr, cap, s);
+        launch_binning(Av, pp, b, c->conf_mask, s);
+    }
     for (int q = NCONF - 1; q >= 0; --q) {
-        if (!conf_on(c, q)) continue;
+        if (!conf_on(c, q) || (q == CONF_DIRECT && max_comp <= DIRECT_MIN_SPAN)) continue;
         const int g = numeric_grid(q, pp, c->num_sms);
         launch_numeric(q, Av, pp, with_buckets(c, b, q, g, c->bucket_row.p ? c->bucket_row.bytes : 0), g, s);
     }
-    launch_finalize_stats(n, b, s);
-    launch_fill_inactive(Av, b.active, b.kept, s);
-    launch_exclusive_scan<int32_t>(b.kept, n, out.colptr, b.scan_tmp, &b.ctr->nnz_out, s);
+    if (small) {
+        launch_result_small(Av, b, out.colptr, nullptr, s);
+    } else {
+        launch_finalize_stats(n, b, s);
+        launch_fill_inactive(Av, b.active, b.kept, s);
+        launch_exclusive_scan<int32_t>(b.kept, n, out.colptr, b.scan_tmp, &b.ctr->nnz_out, s);
+    }
     launch_compact(Av, b, out.colptr, out.rowidx, out.val, s);
     cudaMemsetAsync(c->comp_bits.p, 0, (size_t)ncomp * 8, s);
     launch_comp_chaos(n, (const int32_t*)c->comp_of_col.p, b.active, b.chaos,
@@ -1221,8 +1253,10 @@ static mcl_status graph_prepare(mcl_ctx* c, const mcl_params* prm, const PrunePa
                                 GraphRun& G, cudaStream_t s) {
     const int32_t n = cur->n;
     int64_t cap = 0;  // entries of an iteration's output: column j keeps <= min(K_rec, |comp(j)|)
+    int64_t max_comp = 0;
     for (int q = 0; q < ncomp; ++q) {
         const int64_t sz = comp_offsets[q + 1] - comp_offsets[q];
+        if (sz > max_comp) max_comp = sz;
         cap += sz * (sz < pp.Krec ? sz : pp.Krec);
     }
     if (c->graph_cap > 0 && c->graph_cap < cap) cap = c->graph_cap;
@@ -1287,7 +1321,7 @@ static mcl_status graph_prepare(mcl_ctx* c, const mcl_params* prm, const PrunePa
     const long long l0 = launches_total();
     for (int q = 0; q < 2; ++q) {
         CUDA_TRY(c, cudaStreamBeginCapture(G.gs, cudaStreamCaptureModeRelaxed));
-        static_iteration(c, prm, pp, ncomp, G.buf[q], G.buf[q ^ 1], cap, sizing, stride, G.gs);
+        static_iteration(c, prm, pp, ncomp, max_comp, G.buf[q], G.buf[q ^ 1], cap, sizing, stride, G.gs);
         CUDA_TRY(c, cudaStreamEndCapture(G.gs, &G.g[q]));
         CUDA_TRY(c, cudaGraphInstantiate(&G.x[q], G.g[q], 0));
     }

@@ -25,22 +25,26 @@ struct WinShared {
     int ovf2[2];   // the window exceeded its table
     int went2[2];  // entries of the window's table
     int next2[2];  // source counter of the warp-per-source insert
-    double red;    // result of an ordered sum
+    double red;    // result of a mass
+    double red4[4];  // partial results of an ordered sum
+    int flag;
 };
 
-// Sum of f(s[i]) over i < m in an order that does not depend on the block
-// size: warp 0 alone, lane l taking i = l, l + 32, ..., then a fixed
-// butterfly; the result is broadcast to the block.  Two barriers.
+// Sum of f(i) over i < m in an order that does not depend on the block size
+// (at least SUM_T threads): thread t of the first SUM_T takes i = t, t + SUM_T,
+// ..., each warp adds its lanes by a fixed butterfly and the warps' sums are
+// added in turn; the result is broadcast to the block.  Two barriers.
+constexpr int SUM_T = 128;
 template <class F>
-__device__ __forceinline__ double ordered_sum(const uint64_t* s, int m, F f, double* slot) {
-    if (threadIdx.x < 32) {
+__device__ __forceinline__ double ordered_sum(int m, F f, double* slots) {
+    if (threadIdx.x < SUM_T) {
         double x = 0.0;
-        for (int i = threadIdx.x; i < m; i += 32) x += f(s[i]);
+        for (int i = threadIdx.x; i < m; i += SUM_T) x += f(i);
         x = warp_sum(x);
-        if (threadIdx.x == 0) *slot = x;
+        if ((threadIdx.x & 31) == 0) slots[threadIdx.x >> 5] = x;
     }
     __syncthreads();
-    const double r = *slot;
+    const double r = ((slots[0] + slots[1]) + slots[2]) + slots[3];
     __syncthreads();
     return r;
 }
@@ -209,6 +213,72 @@ __device__ void block_radix_sort_hi(uint64_t* s, uint64_t* tmp, int n, int bits,
     }
 }
 
+// Sorts s[0..n) ascending by the field s[i] >> 32 (distinct values below
+// span) by distribution: NB buckets of equal width, a scan of their counts, and
+// a thread per bucket for the few keys in it.  About eight barriers, where
+// three radix passes take twenty-four.  Returns false, with s as it was, when a
+// bucket has more than BSORT_MAX keys (rows bunched together).  tmp holds n
+// elements; cnt holds NB counters, NB a multiple of T.
+constexpr int BSORT_MAX = 12;
+template <int T>
+__device__ bool block_bucket_sort_hi(uint64_t* s, uint64_t* tmp, int n, unsigned span, unsigned* cnt,
+                                     int* wsm, int* flag) {
+    constexpr int NB = T / 32 * 256, PER = NB / T;
+    const int tid = threadIdx.x;
+    // bucket = floor(x scale / 2^32) < NB for x < span <= 2^31
+    const unsigned scale = span > (unsigned)NB ? (unsigned)(((unsigned long long)NB << 32) / span) : 0u;
+    auto bucket = [&](uint64_t x) {
+        const unsigned r = (unsigned)(x >> 32);
+        return scale ? __umulhi(r, scale) : r;
+    };
+    for (int i = tid; i < NB; i += T) cnt[i] = 0u;
+    if (tid == 0) *flag = 0;
+    __syncthreads();
+    for (int i = tid; i < n; i += T)
+        if (atomicAdd(cnt + bucket(s[i]), 1u) >= (unsigned)BSORT_MAX) *flag = 1;
+    __syncthreads();
+    if (*flag) {
+        __syncthreads();
+        return false;
+    }
+    unsigned c[PER];
+    int sum = 0;
+#pragma unroll
+    for (int q = 0; q < PER; ++q) {
+        c[q] = cnt[tid * PER + q];
+        sum += (int)c[q];
+    }
+    int total;
+    int at = block_scan_excl<T>(sum, &total, wsm);
+    const int first = at;
+#pragma unroll
+    for (int q = 0; q < PER; ++q) {
+        cnt[tid * PER + q] = (unsigned)at;
+        at += (int)c[q];
+    }
+    __syncthreads();
+    for (int i = tid; i < n; i += T) {
+        const uint64_t x = s[i];
+        tmp[atomicAdd(cnt + bucket(x), 1u)] = x;
+    }
+    __syncthreads();
+    // this thread's buckets, ordered by insertion, back to s
+    at = first;
+#pragma unroll
+    for (int q = 0; q < PER; ++q) {
+        const int m = (int)c[q];
+        for (int a = 0; a < m; ++a) {
+            const uint64_t x = tmp[at + a];
+            int b = a;
+            for (; b > 0 && s[at + b - 1] > x; --b) s[at + b] = s[at + b - 1];
+            s[at + b] = x;
+        }
+        at += m;
+    }
+    __syncthreads();
+    return true;
+}
+
 // Value mass of the keys >= cut in a[0..n), as an exact integer sum of the
 // values in fixed point (each truncated at 2^-50 of the largest value), so
 // that it does not depend on the order of a's elements.  Warp 0 sums; the
@@ -240,12 +310,113 @@ __device__ double mass_at_or_above(const uint64_t* a, int n, uint64_t cut, WinSh
     return r;
 }
 
+// Few keys: every rank by counting.  FEW_KEYS keys at most (one per thread).
+constexpr int FEW_KEYS = 128;
+
+// The prune rule (below) on top[0..ntop), ntop <= FEW_KEYS: on return the kept
+// keys are the first m* of top, in row order.  Where the cut is the threshold
+// a key needs no rank; otherwise it is compared with every other: its rank,
+// and the mass of the keys from it up in the fixed point of block_select_mass
+// (mhist holds the keys' masses), give the same cuts as the radix selects,
+// whose passes cost more than this column's whole work.
+template <int T>
+__device__ int finish_few(uint64_t* top, int ntop, const PruneParams& pp, double S, double MT, long long Tt,
+                          int64_t cap, unsigned* hist, unsigned long long* mhist, WinShared* sh,
+                          DevCounters* ctr) {
+    static_assert(FEW_KEYS <= T && FEW_KEYS <= 256, "one key per thread");
+    const int tid = threadIdx.x;
+    const bool mine = tid < ntop;
+    const uint64_t x = mine ? top[tid] : 0ull;
+    const double target = (double)pp.p * S;
+    const int q = (int)(Tt < (long long)pp.K ? Tt : (long long)pp.K);
+    int mstar;
+    bool kept;
+    if (q < pp.Krec && Tt <= pp.K && (target <= 0.0 || MT >= target)) {
+        mstar = (int)Tt;  // the entries >= theta, all among the candidates
+        kept = mine && x >= ((uint64_t)__float_as_uint(pp.theta) << 32);
+    } else {
+        int rank = 0;
+        if (q >= pp.Krec) {
+            mstar = pp.Krec;
+            if (mine)
+                for (int k = 0; k < ntop; ++k) rank += top[k] > x;
+        } else {
+            // scale of the masses: the largest value below 2^e
+            if (tid < FEW_KEYS) {
+                const uint64_t y = warp_max(x);
+                if ((tid & 31) == 0) sh->bs.q[3][tid >> 5] = (long long)y;
+            }
+            __syncthreads();
+            uint64_t kmax = 0;
+#pragma unroll
+            for (int w = 0; w < FEW_KEYS / 32; ++w) {
+                const uint64_t y = (uint64_t)sh->bs.q[3][w];
+                kmax = y > kmax ? y : kmax;
+            }
+            int e = 0;
+            const float maxv = key_val(kmax);
+            frexpf(maxv > 0.0f ? maxv : 1.0f, &e);
+            const int s50 = 50 - e;
+            if (mine) mhist[tid] = __float2ull_rz(ldexpf(key_val(x), s50));
+            if (tid == 0) {
+                sh->red = 0.0;
+                sh->flag = INT_MAX;
+            }
+            __syncthreads();
+            unsigned long long mass = 0;
+            if (mine)
+                for (int k = 0; k < ntop; ++k) {
+                    const uint64_t y = top[k];
+                    rank += y > x;
+                    mass += y >= x ? mhist[k] : 0ull;
+                }
+            double mq = MT;
+            if (Tt > pp.K) {
+                if (mine && rank == pp.K - 1) sh->red = ldexp((double)mass, -s50);
+                __syncthreads();
+                mq = sh->red;
+            }
+            if (target <= 0.0 || mq >= target) {
+                mstar = q;
+            } else {
+                const double tf = ceil(ldexp(target, s50));
+                if (tf < 9.0e18 && mine && mass >= (unsigned long long)tf) atomicMin(&sh->flag, rank + 1);
+                __syncthreads();
+                mstar = min(sh->flag, ntop);
+            }
+        }
+        if (mstar > pp.Krec) mstar = pp.Krec;
+        if (mstar > ntop) mstar = ntop;
+        if ((int64_t)mstar > cap) {  // cannot happen for validated input; never write past cap
+            if (tid == 0) set_err2(ctr, ERR_INTERNAL);
+            mstar = (int)cap;
+        }
+        kept = mine && rank < mstar;
+    }
+    // positions: the kept keys' low words are larger for smaller rows, and never 0
+    if (tid < FEW_KEYS) hist[tid] = kept ? (uint32_t)x : 0u;
+    __syncthreads();
+    int at = 0;
+    if (kept) {
+        const uint32_t r = (uint32_t)x;
+        const uint4* h4 = reinterpret_cast<const uint4*>(hist);
+        for (int k = 0; k < ntop; k += 4) {
+            const uint4 y = h4[k >> 2];
+            at += (y.x > r) + (y.y > r) + (y.z > r) + (y.w > r);
+        }
+    }
+    __syncthreads();
+    if (kept && (int64_t)at < cap) top[at] = x;
+    __syncthreads();
+    return (int64_t)mstar > cap ? (int)cap : mstar;
+}
+
 // Finish a column: prune rule on the candidate keys top[0..ntop) plus exact
 // statistics, then the kept keys in row order (sorted here unless the
 // buffer is already row-ordered) written with inflation (pp.inflate) or
 // their B values; returns m* and chaos_j via the pointers.
 // For an unordered buffer, rows lie in [row_lo, row_lo + row_span); the
-// radix sort uses top[m .. topcap) and rscratch ((T / 32) * 256 counters)
+// row sort uses top[m .. topcap) and rscratch ((T / 32) * 256 counters)
 // as scratch when they suffice, the bitonic network otherwise.
 template <int T, int IPT, bool ROW_ORDERED>
 __device__ void finish_column(uint64_t* top, int ntop, int topcap, const PruneParams& pp, double S,
@@ -254,6 +425,10 @@ __device__ void finish_column(uint64_t* top, int ntop, int topcap, const PrunePa
                               WinShared* sh, DevCounters* ctr, int row_lo, int row_span,
                               unsigned* rscratch, int* mstar_out, double* chaos_out) {
     const int tid = threadIdx.x;
+    int m;
+    if (ntop <= FEW_KEYS) {
+        m = finish_few<T>(top, ntop, pp, S, MT, Tt, cap, hist, mhist, sh, ctr);
+    } else {
     const double target = (double)pp.p * S;
     const int q = (int)(Tt < (long long)pp.K ? Tt : (long long)pp.K);
     double mq = 0.0;
@@ -309,7 +484,7 @@ __device__ void finish_column(uint64_t* top, int ntop, int topcap, const PrunePa
             cut = block_select_count<T>(top, ntop, top, 0, mstar, hist, &sh->bs);
     }
     // the kept keys (exactly m* of them: keys are distinct) to the front
-    int m = mstar > 0 ? compact_stable<T, IPT>(top, ntop, cut, sh->wsm) : 0;
+    m = mstar > 0 ? compact_stable<T, IPT>(top, ntop, cut, sh->wsm) : 0;
     if (m != mstar) {
         if (tid == 0) set_err2(ctr, ERR_INTERNAL);
         m = m < mstar ? m : mstar;
@@ -323,7 +498,8 @@ __device__ void finish_column(uint64_t* top, int ntop, int topcap, const PrunePa
         __syncthreads();
         if (rscratch != nullptr && topcap - m >= m) {
             const int bits = 32 - __clz(row_span - 1);
-            block_radix_sort_hi<T>(top, top + m, m, bits, rscratch, sh->wsm);
+            if (!block_bucket_sort_hi<T>(top, top + m, m, (unsigned)row_span, rscratch, sh->wsm, &sh->flag))
+                block_radix_sort_hi<T>(top, top + m, m, bits, rscratch, sh->wsm);
         } else {
             block_sort_asc<T>(top, m);
         }
@@ -333,31 +509,33 @@ __device__ void finish_column(uint64_t* top, int ntop, int topcap, const PrunePa
         }
         __syncthreads();
     }
-    const float rr = pp.r;
-    const double U = pp.inflate ? ordered_sum(top, m, [rr](uint64_t x) {
-        return (double)inflate_value(key_val(x), rr); }, &sh->red) : 0.0;
-    const double invU = U > 0.0 ? 1.0 / U : 0.0;
-    double amax = 0.0;
-    for (int i = tid; i < m; i += T) {
-        const uint64_t x = top[i];
-        const float v = key_val(x);
-        float outv = v;
-        if (pp.inflate) {
-            const double a = (double)inflate_value(v, pp.r) * invU;
-            outv = (float)a;
-            amax = a > amax ? a : amax;
-        }
-        out_row[i] = key_row(x);
-        out_val[i] = outv;
     }
+    // ---- inflation, renormalisation, chaos_j and the output ----
+    const float rr = pp.r;
+    const double U = pp.inflate ? ordered_sum(m, [top, rr](int i) {
+        return float_to_double(inflate_value(key_val(top[i]), rr)); }, sh->red4) : 0.0;
+    const double invU = U > 0.0 ? 1.0 / U : 0.0;
     double ch = 0.0;
     if (pp.inflate) {
-        const double mx = block_max_d<T>(amax, &sh->bs);
-        const double sq = ordered_sum(top, m, [rr, invU](uint64_t x) {
-            const double a = (double)inflate_value(key_val(x), rr) * invU;
-            return a * a; }, &sh->red);
+        float umax = 0.0f;
+        const double sq = ordered_sum(m, [&](int i) {
+            const uint64_t x = top[i];
+            const float u = inflate_value(key_val(x), rr);
+            const double a = float_to_double(u) * invU;
+            umax = fmaxf(umax, u);
+            out_row[i] = key_row(x);
+            out_val[i] = (float)a;
+            return a * a; }, sh->red4);
+        // the largest u gives the largest a (rounding is monotone)
+        const double mx = block_max_d<T>((double)umax * invU, &sh->bs);
         ch = mx - sq;
         if (ch < 0.0) ch = 0.0;
+    } else {
+        for (int i = tid; i < m; i += T) {
+            const uint64_t x = top[i];
+            out_row[i] = key_row(x);
+            out_val[i] = key_val(x);
+        }
     }
     if (tid == 0) {
         *mstar_out = m;

@@ -12,6 +12,7 @@ namespace mcl {
 // row for columns that are dense in their span (mcl_direct.cu).
 constexpr int NCONF = 3;
 constexpr int CONF_LARGE = 1, CONF_DIRECT = 2;
+constexpr int DIRECT_MIN_SPAN = 2048;    // spans of CONF_DIRECT are longer
 constexpr int NZ = 8;                    // size classes per configuration
 constexpr int NBUCKET = NCONF * NZ;
 // device-side counters (one small block of memory per context)
@@ -113,7 +114,7 @@ template <typename TIn>
 void launch_exclusive_scan(const TIn* in, int64_t n, int64_t* out, int64_t* tmp,
                            unsigned long long* total, cudaStream_t s);
 void launch_symbolic(const CscView& A, const ExpandBuffers& b, int64_t* nnz_out, int num_sms,
-                     int grid_cap, cudaStream_t s);
+                     int grid_cap, cudaStream_t s, bool fresh = false);
 int symbolic_grid(int num_sms);
 void launch_scale_est(int32_t n, int64_t* est, int milli, cudaStream_t s);
 void launch_cap_tighten(int32_t n, const int64_t* est, int64_t* cap, const uint8_t* active,
@@ -121,6 +122,13 @@ void launch_cap_tighten(int32_t n, const int64_t* est, int64_t* cap, const uint8
 void launch_est_from_flops(const CscView& A, const ExpandBuffers& b, cudaStream_t s);
 void launch_binning(const CscView& A, const PruneParams& pp, const ExpandBuffers& b, int mask,
                     cudaStream_t s);
+// Up to SMALL_PLAN_N columns one CTA does the steps around the numeric pass.
+constexpr int SMALL_PLAN_N = 16384;
+bool plan_is_small(int64_t n);
+void launch_plan_small(int32_t n, bool exact, int64_t staging, const PruneParams& pp,
+                       const ExpandBuffers& b, int mask, DevCounters* host, cudaStream_t s);
+void launch_result_small(const CscView& A, const ExpandBuffers& b, int64_t* colptr, DevCounters* host,
+                         cudaStream_t s);
 int numeric_grid(int conf, const PruneParams& pp, int num_sms);
 constexpr int WINDOW_MAX = 4096;  // windows per column in bucket mode
 int direct_grid(int ksel, int num_sms);

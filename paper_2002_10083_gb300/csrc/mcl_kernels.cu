@@ -430,7 +430,7 @@ static int symbolic_occupancy(int words, int num_sms) {
 int symbolic_grid(int num_sms) { return symbolic_occupancy<512>(SYM_WORDS, num_sms); }
 
 void launch_symbolic(const CscView& A, const ExpandBuffers& b, int64_t* nnz_out, int num_sms,
-                     int grid_cap, cudaStream_t s) {
+                     int grid_cap, cudaStream_t s, bool fresh) {
     if (A.n == 0) return;
     int words = (int)(((int64_t)A.n + 127) / 128 * 4);
     if (words > SYM_WORDS) words = SYM_WORDS;
@@ -439,7 +439,7 @@ void launch_symbolic(const CscView& A, const ExpandBuffers& b, int64_t* nnz_out,
     int grid = small ? symbolic_occupancy<128>(words, num_sms) : symbolic_occupancy<512>(words, num_sms);
     if (A.n > SYM_WORDS * 32 && grid > grid_cap) grid = grid_cap;
     if ((int64_t)grid > A.n) grid = A.n;
-    cudaMemsetAsync(&b.ctr->work_ctr, 0, sizeof(int), s);
+    if (!fresh) cudaMemsetAsync(&b.ctr->work_ctr, 0, sizeof(int), s);
     if (small)
         k_symbolic<128><<<grid, 128, symbolic_smem(words), s>>>(A, b, nnz_out, words);
     else
@@ -501,7 +501,7 @@ void launch_est_from_flops(const CscView& A, const ExpandBuffers& b, cudaStream_
 // Clocks of an SM per column, hashed and direct: 1M-row spans 912k and 977k at
 // 200k products, 1.51M and 1.16M at 390k; 20k-row spans 51k and 55k at 6k
 // products, 65k and 60k at 12k.
-constexpr int DIRECT_MIN_SPAN = 2048, DIRECT_SPARSE = 4;
+constexpr int DIRECT_SPARSE = 4;
 
 // Configuration 0 (small CTA) takes columns whose estimate fits one small
 // window's value capacity and whose span needs few windows; CONF_DIRECT takes
@@ -584,6 +584,156 @@ void launch_binning(const CscView& A, const PruneParams& pp, const ExpandBuffers
         k_bin_scatter<<<(unsigned)((A.n + 255) / 256), 256, 0, s>>>(A.n, b);
         count_launches(1);
     }
+}
+
+// ---------------------------------------------------------------------------
+// small graphs: the steps around the two large kernels of an iteration in one
+// CTA each, instead of a chain of launches that each cost more than their work
+// ---------------------------------------------------------------------------
+
+constexpr int SMALL_T = 1024;
+
+bool plan_is_small(int64_t n) { return n <= SMALL_PLAN_N; }
+
+// Warp w of the CTA takes the columns [w seg, (w + 1) seg), 32 at a time with
+// a running sum, so that one barrier joins the warps' sums: f(j) gives column
+// j's count (32 bits hold the sum of SMALL_PLAN_N columns of at most as many
+// entries), put(j, x) takes its exclusive prefix.  Returns the total.
+template <class F, class P>
+__device__ __forceinline__ int small_scan(int n, int* ws, F f, P put) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int seg = ((n + SMALL_T - 1) / SMALL_T) * 32;
+    const int j0 = warp * seg, j1 = min(n, j0 + seg);
+    int sum = 0;
+    for (int j = j0 + lane; j < j1; j += 32) sum += f(j);
+    sum = (int)__reduce_add_sync(FULL, (unsigned)sum);
+    if (lane == 0) ws[warp] = sum;
+    __syncthreads();
+    const int x = ws[lane];
+    const int total = (int)__reduce_add_sync(FULL, (unsigned)x);
+    int carry = (int)__reduce_add_sync(FULL, lane < warp ? (unsigned)x : 0u);
+    for (int b = j0; b < j1; b += 32) {
+        const int j = b + lane;
+        const int c = j < j1 ? f(j) : 0;
+        int v = c;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int y = __shfl_up_sync(FULL, v, o);
+            if (lane >= o) v += y;
+        }
+        if (j < j1) put(j, carry + v - c);
+        carry += __shfl_sync(FULL, v, 31);
+    }
+    __syncthreads();
+    return total;
+}
+
+__device__ __forceinline__ void small_copy_counters(const DevCounters* src, DevCounters* dst) {
+    __syncthreads();  // the CTA's own counters are written
+    constexpr int W = (int)(sizeof(DevCounters) / 8);
+    if (threadIdx.x < W)
+        reinterpret_cast<unsigned long long*>(dst)[threadIdx.x] =
+            reinterpret_cast<const volatile unsigned long long*>(src)[threadIdx.x];
+}
+
+// cap_tighten (exact estimates), the scan of the capacities, the staging guard,
+// binning and the copy of the counters to the host.
+__global__ void __launch_bounds__(SMALL_T) k_plan_small(int32_t n, int exact, int64_t staging, int mask,
+                                                        int small_max, ExpandBuffers b, DevCounters* host) {
+    __shared__ int ws[32];
+    __shared__ int hist[NBUCKET], fill[NBUCKET];
+    const int tid = threadIdx.x;
+    for (int i = tid; i < NBUCKET; i += SMALL_T) hist[i] = 0;
+    __syncthreads();
+#pragma unroll 4
+    for (int j = tid; j < n; j += SMALL_T) {
+        int bk = -1;
+        if (!b.active || b.active[j]) {
+            const int64_t est = b.est[j];
+            if (exact && est < b.cap[j]) b.cap[j] = est;
+            bk = bucket_of(est, b.flops[j], b.rhi[j] - b.rlo[j] + 1, mask, small_max);
+            atomicAdd(&hist[bk], 1);
+        }
+        b.bucket[j] = bk;
+    }
+    __syncthreads();
+    const int total = small_scan(n, ws, [&](int j) { return (int)b.cap[j]; },
+                                 [&](int j, int x) { b.off[j] = x; });
+    if (tid == 0) {
+        b.off[n] = total;
+        b.ctr->cap_total = (unsigned long long)total;
+        if (staging >= 0 && total > staging) atomicOr(&b.ctr->err, ERR_STAGING);
+        int run = 0;
+        for (int i = 0; i < NBUCKET; ++i) {
+            b.ctr->bin_cnt[i] = hist[i];
+            b.ctr->bin_off[i] = run;
+            fill[i] = run;
+            run += hist[i];
+        }
+        b.ctr->bin_off[NBUCKET] = run;
+        for (int q = 0; q < NCONF; ++q) b.ctr->conf_ctr[q] = 0;
+    }
+    __syncthreads();
+#pragma unroll 4
+    for (int j = tid; j < n; j += SMALL_T) {
+        const int bk = b.bucket[j];
+        if (bk >= 0) b.work[atomicAdd(&fill[bk], 1)] = j;
+    }
+    if (host) small_copy_counters(b.ctr, host);
+}
+
+void launch_plan_small(int32_t n, bool exact, int64_t staging, const PruneParams& pp,
+                       const ExpandBuffers& b, int mask, DevCounters* host, cudaStream_t s) {
+    k_plan_small<<<1, SMALL_T, 0, s>>>(n, exact ? 1 : 0, staging, mask, pp.small_max, b, host);
+    count_launches(1);
+}
+
+// finalize_stats, carried columns' counts (A given), the scan of the kept
+// counts into colptr and the copy of the counters to the host.
+__global__ void __launch_bounds__(SMALL_T) k_result_small(CscView A, ExpandBuffers b, int64_t* colptr,
+                                                          DevCounters* host) {
+    __shared__ int ws[32];
+    __shared__ long long ss[32];
+    __shared__ double smax[32];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int n = A.n;
+    long long sb = 0;
+    double mx = 0.0;
+#pragma unroll 4
+    for (int j = tid; j < n; j += SMALL_T) {
+        if (b.active && !b.active[j]) {
+            b.kept[j] = (int32_t)(A.colptr[j + 1] - A.colptr[j]);
+        } else {
+            mx = fmax(mx, b.chaos[j]);
+            sb += b.bnnz[j];
+        }
+    }
+    mx = warp_max(mx);
+    sb = warp_sum(sb);
+    if (lane == 0) {
+        smax[warp] = mx;
+        ss[warp] = sb;
+    }
+    __syncthreads();
+    const int total = small_scan(n, ws, [&](int j) { return b.kept[j]; },
+                                 [&](int j, int x) { colptr[j] = x; });
+    if (tid < 32) {
+        mx = warp_max(smax[tid]);
+        sb = warp_sum(ss[tid]);
+        if (tid == 0) {
+            colptr[n] = total;
+            b.ctr->nnz_out = (unsigned long long)total;
+            b.ctr->chaos_bits = (unsigned long long)__double_as_longlong(mx);
+            b.ctr->nnz_b = (unsigned long long)sb;
+        }
+    }
+    if (host) small_copy_counters(b.ctr, host);
+}
+
+void launch_result_small(const CscView& A, const ExpandBuffers& b, int64_t* colptr, DevCounters* host,
+                         cudaStream_t s) {
+    k_result_small<<<1, SMALL_T, 0, s>>>(A, b, colptr, host);
+    count_launches(1);
 }
 
 // cap_j for the standalone prune: min(Krec, nnz(B_*j))

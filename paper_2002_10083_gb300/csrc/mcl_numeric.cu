@@ -729,6 +729,7 @@ void launch_numeric(int conf, const CscView& A, const PruneParams& pp, const Exp
 // a column's entries are already row-ordered)
 // ---------------------------------------------------------------------------
 
+constexpr int PR_MINB = 4;  // 64 registers: the selects and scans need the warps
 constexpr int PR_T = 256, PR_IPT = 8, PR_VC = PR_T * PR_IPT;
 
 struct PruneShared {
@@ -824,14 +825,14 @@ struct PruneArgs {
 };
 
 template <bool FIXED>
-__global__ void __launch_bounds__(PR_T) k_prune(PruneArgs a) {
+__global__ void __launch_bounds__(PR_T, PR_MINB) k_prune(PruneArgs a) {
     extern __shared__ __align__(16) unsigned char smem[];
     const int ksel = a.pp.ksel;
     const int topcap = ksel + PR_VC;
-    uint64_t* top = reinterpret_cast<uint64_t*>(smem);
-    unsigned* hist = reinterpret_cast<unsigned*>(top + topcap);
-    unsigned long long* mhist = reinterpret_cast<unsigned long long*>(hist + 256);
-    PruneShared* ps = reinterpret_cast<PruneShared*>(mhist + 256);
+    unsigned long long* mhist = reinterpret_cast<unsigned long long*>(smem);
+    unsigned* hist = reinterpret_cast<unsigned*>(mhist + 256);  // 16-byte aligned whatever ksel is
+    uint64_t* top = reinterpret_cast<uint64_t*>(hist + 256);
+    PruneShared* ps = reinterpret_cast<PruneShared*>(top + topcap);
     WinShared* sh = &ps->w;
     const int tid = threadIdx.x;
     const ExpandBuffers& b = a.b;

@@ -128,3 +128,46 @@ def test_mlp_sample_counts(ctx, n):
     (total / n).backward()
     assert abs(float(loss) / float(total.detach()) - 1) < 1e-5
     assert float((grad.double() - p.grad).abs().max()) < 1e-4 * float(p.grad.abs().max())
+
+
+# columns whose candidates are ranked by counting (up to 128 keys) and by radix selects, with the
+# cut at the threshold, at K, at the mass and at nothing
+@pytest.mark.parametrize("K,theta,p", [(1000, 1e-3, 0.9), (40, 0.0, 0.5), (40, 5e-3, 0.99), (1000, 0.05, 1.0),
+                                       (127, 0.0, 0.0), (128, 1e-4, 0.95), (5, 1.0, 0.3)])
+def test_few_candidates(ctx, K, theta, p):
+    from tests.test_gpu_expand import _check, _prm
+    A = synth.random_sparse(700, 0.016, seed=21, w="lognormal")
+    _check(ctx, A, _prm(theta=theta, K=K, p=p))
+
+
+def test_bunched_rows_are_sorted(ctx):
+    """Kept rows in a few places of a wide span: more keys per bucket of the row sort than it
+    orders, and the radix passes take over."""
+    import scipy.sparse as sp
+    from tests.test_gpu_expand import _check, _prm
+    n, m = 60000, 900
+    rng = np.random.default_rng(4)
+    B = sp.random(m, m, 0.2, random_state=5, format="coo")
+    row, col = np.concatenate([B.row, [n - 1] * m]), np.concatenate([B.col, np.arange(m)])
+    M = sp.csc_matrix((rng.uniform(0.1, 1, len(row)), (row, col)), shape=(n, n)) + sp.identity(n, format="csc")
+    M.sort_indices()
+    A = synth.CSC(n, M.indptr.astype(np.int64), M.indices.astype(np.int32), M.data)
+    _check(ctx, A, _prm(K=600, theta=1e-5), cols=np.arange(0, m, 7).astype(np.int32))
+
+
+# every graph that one CTA plans, and the first that it does not
+@pytest.mark.parametrize("n", [1, 1023, 1025, 16384, 16385])
+def test_small_plan_sizes(ctx, n):
+    from paper_2002_10083_gb300 import mcl
+    A = _random(n, 12, seed=n)
+    prm = mcl.Params(threshold=1e-4, select_k=30, recover_pct=0.9, inflation=2.0)
+    out, ch = ctx.expand(A, prm)
+    st = ctx.stats()
+    try:
+        ctx.set_option(mcl.OPT_PHASE_BUDGET, 1 << 34)  # the steps kernel by kernel
+        ref, ch_ref = ctx.expand(A, prm)
+    finally:
+        ctx.set_option(mcl.OPT_PHASE_BUDGET, 0)
+    assert ch == ch_ref and torch.equal(out.colptr, ref.colptr) and torch.equal(out.rowidx, ref.rowidx)
+    assert torch.equal(out.val.view(torch.int32), ref.val.view(torch.int32))
+    assert all(st[k] == ctx.stats()[k] for k in ("flops", "nnz_b", "nnz_out", "estimator_misses"))
