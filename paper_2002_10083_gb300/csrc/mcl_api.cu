@@ -452,7 +452,7 @@ static mcl_status expand_impl(mcl_ctx* c, const mcl_csc* A, const mcl_params* pr
         launch_est_from_flops(Av, b, s);
     } else if (sizing == 3) {
         const size_t n1 = (size_t)n + 1;
-        if (!ensure(c, c->cohen_m, n1 * c->cohen_r * 4, s) || !ensure(c, c->cohen_e, n1 * 4, s))
+        if (!ensure(c, c->cohen_m, cohen_scratch_bytes((int64_t)n1, c->cohen_r), s) || !ensure(c, c->cohen_e, n1 * 4, s))
             return fail(c, MCL_ERR_OOM, "estimator scratch allocation failed");
         launch_cohen(Av, c->cohen_r, c->cohen_seed, (float*)c->cohen_m.p, (float*)c->cohen_e.p, s);
         launch_cohen_to_est((int32_t)n, (const float*)c->cohen_e.p, 1.0f, b, s);
@@ -1128,7 +1128,7 @@ mcl_status mcl_cohen_estimate(mcl_ctx* c, const mcl_csc* A, int32_t keys, uint64
     launch_colstats(view(A), pp, b, c->num_sms, s);
     if ((st = read_counters(c, s))) return st;
     if ((st = err_flags(c, c->hctr->err))) return st;
-    if (!ensure(c, c->cohen_m, ((size_t)A->n + 1) * keys * 4, s))
+    if (!ensure(c, c->cohen_m, cohen_scratch_bytes(A->n, keys), s))
         return fail(c, MCL_ERR_OOM, "estimator scratch allocation failed");
     launch_cohen(view(A), keys, seed, (float*)c->cohen_m.p, est, s);
     return check_launch(c, "cohen");
@@ -1284,7 +1284,7 @@ static mcl_status graph_prepare(mcl_ctx* c, const mcl_params* prm, const PrunePa
         const int32_t it2 = 2;
         CUDA_TRY(c, cudaMemcpyAsync(c->iter_dev.p, &it2, 4, cudaMemcpyHostToDevice, s));
     } else if (sizing == 3) {
-        if (!ensure(c, c->cohen_m, n1 * c->cohen_r * 4, s) || !ensure(c, c->cohen_e, n1 * 4, s))
+        if (!ensure(c, c->cohen_m, cohen_scratch_bytes((int64_t)n1, c->cohen_r), s) || !ensure(c, c->cohen_e, n1 * 4, s))
             return fail(c, MCL_ERR_OOM, "estimator scratch allocation failed");
     }
     if (capb >= 1024 && ensure(c, c->bucket_row, (size_t)g1 * capb * 8, s) &&

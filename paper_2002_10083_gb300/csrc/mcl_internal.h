@@ -214,6 +214,7 @@ void launch_logcf(int32_t n, const int64_t* flops, const int64_t* bnnz, float* l
 
 // --- Cohen's estimator (mcl_cohen.cu) ---
 int cohen_max_r();
+size_t cohen_scratch_bytes(int64_t n, int r);  // of launch_cohen's m
 void launch_cohen(const CscView& A, int r, uint64_t seed, float* m, float* est, cudaStream_t s);
 void launch_cohen_to_est(int32_t n, const float* e, float safety, const ExpandBuffers& b,
                          cudaStream_t s);
