@@ -165,7 +165,7 @@ __global__ void k_features(CscView A, int32_t iteration, const int32_t* iter_dev
 // banks.
 constexpr int W2P = NH + 4;
 
-struct MlpWeights {
+struct __align__(16) MlpWeights {
     float w1[NH * NIN];
     float w2[NH * W2P];
     float w3[NOUT * NH];
@@ -174,15 +174,31 @@ struct MlpWeights {
 };
 
 __device__ __forceinline__ void load_weights(MlpWeights& M, const uint16_t* wbits, const float* norm) {
-    for (int p = threadIdx.x; p < NPARAM; p += blockDim.x) {
-        const float w = bf16_bits_to_float(wbits[p]);
-        if (p < OFF_B1) M.w1[p] = w;
-        else if (p < OFF_W2) M.b1[p - OFF_B1] = w;
-        else if (p < OFF_B2) M.w2[(p - OFF_W2) / NH * W2P + (p - OFF_W2) % NH] = w;
-        else if (p < OFF_W3) M.b2[p - OFF_B2] = w;
-        else if (p < OFF_B3) M.w3[p - OFF_W3] = w;
-        else M.b3[p - OFF_B3] = w;
+    // Eight weights at once where the pointer allows it (every section starts at a multiple of
+    // eight): the weights are read once per CTA, and one by one that took half of a small batch.
+    static_assert(OFF_B1 % 8 == 0 && OFF_W2 % 8 == 0 && OFF_B2 % 8 == 0 && OFF_W3 % 8 == 0 && OFF_B3 % 8 == 0,
+                  "eight weights lie in one section");
+    auto place = [&](int p) -> float* {
+        return p < OFF_B1 ? M.w1 + p
+             : p < OFF_W2 ? M.b1 + (p - OFF_B1)
+             : p < OFF_B2 ? M.w2 + (p - OFF_W2) / NH * W2P + (p - OFF_W2) % NH
+             : p < OFF_W3 ? M.b2 + (p - OFF_B2)
+             : p < OFF_B3 ? M.w3 + (p - OFF_W3) : M.b3 + (p - OFF_B3);
+    };
+    int done = 0;
+    if (((uintptr_t)wbits & 15) == 0) {
+        done = NPARAM & ~7;
+#pragma unroll 4
+        for (int p = threadIdx.x * 8; p < done; p += blockDim.x * 8) {
+            const uint4 x = *reinterpret_cast<const uint4*>(wbits + p);
+            float4* d = reinterpret_cast<float4*>(place(p));
+            d[0] = make_float4(__uint_as_float(x.x << 16), __uint_as_float(x.x & 0xFFFF0000u),
+                               __uint_as_float(x.y << 16), __uint_as_float(x.y & 0xFFFF0000u));
+            d[1] = make_float4(__uint_as_float(x.z << 16), __uint_as_float(x.z & 0xFFFF0000u),
+                               __uint_as_float(x.w << 16), __uint_as_float(x.w & 0xFFFF0000u));
+        }
     }
+    for (int p = done + threadIdx.x; p < NPARAM; p += blockDim.x) *place(p) = bf16_bits_to_float(wbits[p]);
     if (threadIdx.x < NIN) {
         M.mu[threadIdx.x] = norm[threadIdx.x];
         M.isg[threadIdx.x] = 1.0f / norm[NIN + threadIdx.x];

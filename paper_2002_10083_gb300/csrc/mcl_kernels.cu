@@ -434,8 +434,8 @@ void launch_symbolic(const CscView& A, const ExpandBuffers& b, int64_t* nnz_out,
     if (A.n == 0) return;
     int words = (int)(((int64_t)A.n + 127) / 128 * 4);
     if (words > SYM_WORDS) words = SYM_WORDS;
-    // few products per column: a warp's work or two
-    const bool small = A.nnz <= (int64_t)A.n * 32 && A.n <= SYM_WORDS;
+    // a short bitmap: more columns at once beat more warps on one
+    const bool small = A.n <= SYM_WORDS;
     int grid = small ? symbolic_occupancy<128>(words, num_sms) : symbolic_occupancy<512>(words, num_sms);
     if (A.n > SYM_WORDS * 32 && grid > grid_cap) grid = grid_cap;
     if ((int64_t)grid > A.n) grid = A.n;
