@@ -64,7 +64,7 @@ struct mcl_ctx {
     Buf cohen_m, cohen_e;
     // inner-dimension split
     Buf split_cnt, split_scratch;
-    Buf spill;  // candidates of the direct configuration
+    Buf spill;  // candidates beyond the CTAs' buffers
 };
 
 namespace {
@@ -436,7 +436,7 @@ static mcl_status expand_impl(mcl_ctx* c, const mcl_csc* A, const mcl_params* pr
     if (b.cur_stride < 32) b.cur_stride = 32;
     const int grid_max = max_numeric_grid(c, pp);
     if (!ensure(c, c->cursors, (size_t)grid_max * 6 * b.cur_stride * 4, s) ||
-        !ensure(c, c->spill, direct_spill_bytes(direct_grid(pp.ksel, c->num_sms)), s))
+        !ensure(c, c->spill, numeric_spill_bytes(pp, c->num_sms), s))
         return fail(c, MCL_ERR_OOM, "cursor scratch allocation failed");
     b.cursors = (int32_t*)c->cursors.p;
     b.spill = (uint64_t*)c->spill.p;
@@ -1272,7 +1272,7 @@ static mcl_status graph_prepare(mcl_ctx* c, const mcl_params* prm, const PrunePa
     const size_t n1 = (size_t)n + 1;
     if (!ensure(c, c->tmp_row, (size_t)cap * 4 + 4, s) || !ensure(c, c->tmp_val, (size_t)cap * 4 + 4, s) ||
         !ensure(c, c->cursors, (size_t)grid_max * 6 * stride * 4, s) ||
-        !ensure(c, c->spill, direct_spill_bytes(direct_grid(pp.ksel, c->num_sms)), s) ||
+        !ensure(c, c->spill, numeric_spill_bytes(pp, c->num_sms), s) ||
         !ensure(c, c->comp_bits, (size_t)ncomp * 8, s))
         return fail(c, MCL_ERR_OOM, "graph replay scratch allocation failed");
     if (sizing == 2) {

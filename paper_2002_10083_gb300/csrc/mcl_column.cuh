@@ -18,36 +18,14 @@ struct WinShared {
     BlockScratch bs;
     int wsm[34];
     int item;
-    int next;
-    // window plan published by thread 0 (rows [pr0, pr1) when prs)
-    int pf0, pf1, pr0, pr1, prs, pdone;
-    // per-window flags, double-buffered by window parity
-    int ovf2[2];   // the window exceeded its table
-    int went2[2];  // entries of the window's table
-    int next2[2];  // source counter of the warp-per-source insert
     double red;    // result of a mass
-    double red4[4];  // partial results of an ordered sum
+    double sum4[2][4];  // partial sums of the warps
+    float max4[4];
+    double inv;         // 1 / sum, and as two FP32 numbers
+    float inv_hi, inv_lo;
+    double chaos;
     int flag;
 };
-
-// Sum of f(i) over i < m in an order that does not depend on the block size
-// (at least SUM_T threads): thread t of the first SUM_T takes i = t, t + SUM_T,
-// ..., each warp adds its lanes by a fixed butterfly and the warps' sums are
-// added in turn; the result is broadcast to the block.  Two barriers.
-constexpr int SUM_T = 128;
-template <class F>
-__device__ __forceinline__ double ordered_sum(int m, F f, double* slots) {
-    if (threadIdx.x < SUM_T) {
-        double x = 0.0;
-        for (int i = threadIdx.x; i < m; i += SUM_T) x += f(i);
-        x = warp_sum(x);
-        if ((threadIdx.x & 31) == 0) slots[threadIdx.x >> 5] = x;
-    }
-    __syncthreads();
-    const double r = ((slots[0] + slots[1]) + slots[2]) + slots[3];
-    __syncthreads();
-    return r;
-}
 
 // Exclusive block scan of one int per thread; *total gets the sum.  Three
 // barriers (the last protects the scratch for the next call).
@@ -300,7 +278,7 @@ __device__ double mass_at_or_above(const uint64_t* a, int n, uint64_t cut, WinSh
         const int s50 = 50 - e;
         unsigned long long acc = 0;
         for (int i = lane; i < n; i += 32)
-            if (a[i] >= cut) acc += __float2ull_rz(ldexpf(key_val(a[i]), s50));
+            if (a[i] >= cut) acc += fixed_of(key_val(a[i]), s50);
         acc = warp_sum(acc);
         if (lane == 0) sh->red = ldexp((double)acc, -s50);
     }
@@ -309,6 +287,8 @@ __device__ double mass_at_or_above(const uint64_t* a, int n, uint64_t cut, WinSh
     __syncthreads();
     return r;
 }
+
+constexpr int SUM_T = 128;  // threads that add a column's powers
 
 // Few keys: every rank by counting.  FEW_KEYS keys at most (one per thread).
 constexpr int FEW_KEYS = 128;
@@ -320,18 +300,17 @@ constexpr int FEW_KEYS = 128;
 // (mhist holds the keys' masses), give the same cuts as the radix selects,
 // whose passes cost more than this column's whole work.
 template <int T>
-__device__ int finish_few(uint64_t* top, int ntop, const PruneParams& pp, double S, double MT, long long Tt,
-                          int64_t cap, unsigned* hist, unsigned long long* mhist, WinShared* sh,
+__device__ int finish_few(uint64_t* top, int ntop, const PruneParams& pp, double S, bool theta_cut,
+                          long long Tt, int64_t cap, unsigned* hist, unsigned long long* mhist, WinShared* sh,
                           DevCounters* ctr) {
     static_assert(FEW_KEYS <= T && FEW_KEYS <= 256, "one key per thread");
     const int tid = threadIdx.x;
     const bool mine = tid < ntop;
     const uint64_t x = mine ? top[tid] : 0ull;
-    const double target = (double)pp.p * S;
     const int q = (int)(Tt < (long long)pp.K ? Tt : (long long)pp.K);
     int mstar;
     bool kept;
-    if (q < pp.Krec && Tt <= pp.K && (target <= 0.0 || MT >= target)) {
+    if (theta_cut) {
         mstar = (int)Tt;  // the entries >= theta, all among the candidates
         kept = mine && x >= ((uint64_t)__float_as_uint(pp.theta) << 32);
     } else {
@@ -357,7 +336,7 @@ __device__ int finish_few(uint64_t* top, int ntop, const PruneParams& pp, double
             const float maxv = key_val(kmax);
             frexpf(maxv > 0.0f ? maxv : 1.0f, &e);
             const int s50 = 50 - e;
-            if (mine) mhist[tid] = __float2ull_rz(ldexpf(key_val(x), s50));
+            if (mine) mhist[tid] = fixed_of(key_val(x), s50);
             if (tid == 0) {
                 sh->red = 0.0;
                 sh->flag = INT_MAX;
@@ -370,13 +349,14 @@ __device__ int finish_few(uint64_t* top, int ntop, const PruneParams& pp, double
                     rank += y > x;
                     mass += y >= x ? mhist[k] : 0ull;
                 }
-            double mq = MT;
+            const double target = (double)pp.p * S;
+            bool enough = false;  // Tt <= K: known to fall short
             if (Tt > pp.K) {
                 if (mine && rank == pp.K - 1) sh->red = ldexp((double)mass, -s50);
                 __syncthreads();
-                mq = sh->red;
+                enough = target <= 0.0 || sh->red >= target;
             }
-            if (target <= 0.0 || mq >= target) {
+            if (enough) {
                 mstar = q;
             } else {
                 const double tf = ceil(ldexp(target, s50));
@@ -420,26 +400,34 @@ __device__ int finish_few(uint64_t* top, int ntop, const PruneParams& pp, double
 // as scratch when they suffice, the bitonic network otherwise.
 template <int T, int IPT, bool ROW_ORDERED>
 __device__ void finish_column(uint64_t* top, int ntop, int topcap, const PruneParams& pp, double S,
-                              double MT, long long Tt, int64_t cap, int32_t* out_row,
+                              unsigned long long mt, int f, long long Tt, int64_t cap, int32_t* out_row,
                               float* out_val, unsigned* hist, unsigned long long* mhist,
                               WinShared* sh, DevCounters* ctr, int row_lo, int row_span,
                               unsigned* rscratch, int* mstar_out, double* chaos_out) {
-    const int tid = threadIdx.x;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    // FP64 work is one warp's, not every warp's: its instructions take 16 clocks
+    // of the SM each, and a column of a few entries took 23k clocks in here
+    const int q = (int)(Tt < (long long)pp.K ? Tt : (long long)pp.K);
+    bool theta_cut = false;  // the entries >= theta are at most K and carry the mass to recover
+    if (q < pp.Krec && Tt <= pp.K) {
+        if (tid == 0) {
+            const double goal = (double)pp.p * S;
+            sh->flag = goal <= 0.0 || ldexp((double)mt, -f) >= goal;
+        }
+        __syncthreads();
+        theta_cut = sh->flag != 0;
+        __syncthreads();
+    }
     int m;
     if (ntop <= FEW_KEYS) {
-        m = finish_few<T>(top, ntop, pp, S, MT, Tt, cap, hist, mhist, sh, ctr);
+        m = finish_few<T>(top, ntop, pp, S, theta_cut, Tt, cap, hist, mhist, sh, ctr);
     } else {
-    const double target = (double)pp.p * S;
-    const int q = (int)(Tt < (long long)pp.K ? Tt : (long long)pp.K);
     double mq = 0.0;
     uint64_t kq = 0;
     // q >= Krec: m* = min(Krec, max(q, m_rec)) = Krec whatever the recovery
     // finds, so neither the top-q mass nor m_rec is needed
     const bool krec_bound = q >= pp.Krec;
-    if (krec_bound) {
-    } else if (Tt <= pp.K) {
-        mq = MT;
-    } else {
+    if (!krec_bound && Tt > pp.K) {
         kq = block_select_count<T>(top, ntop, top, 0, pp.K, hist, &sh->bs);
         mq = mass_at_or_above<T>(top, ntop, kq, sh);
     }
@@ -448,7 +436,7 @@ __device__ void finish_column(uint64_t* top, int ntop, int topcap, const PrunePa
     bool have_cut = false;
     if (krec_bound) {
         mstar = pp.Krec;
-    } else if (target <= 0.0 || mq >= target) {
+    } else if (theta_cut || (Tt > pp.K && ((double)pp.p * S <= 0.0 || mq >= (double)pp.p * S))) {
         mstar = q;
         if (mstar <= pp.Krec) {
             if (Tt <= pp.K) {
@@ -461,9 +449,10 @@ __device__ void finish_column(uint64_t* top, int ntop, int topcap, const PrunePa
     } else {
         uint64_t kr = 0;
         int mr = 0;
-        const int f = block_select_mass<T>(top, ntop, target, &kr, &mr, hist, mhist, &sh->bs);
-        mstar = f ? mr : ntop;
-        if (f && mstar <= pp.Krec) {
+        const int found =
+            block_select_mass<T>(top, ntop, (double)pp.p * S, &kr, &mr, hist, mhist, &sh->bs);
+        mstar = found ? mr : ntop;
+        if (found && mstar <= pp.Krec) {
             cut = kr;
             have_cut = true;
         }
@@ -511,59 +500,80 @@ __device__ void finish_column(uint64_t* top, int ntop, int topcap, const PrunePa
     }
     }
     // ---- inflation, renormalisation, chaos_j and the output ----
+    // U = sum u and the sum of u^2 over the kept u = v^r, in an order that does not depend on
+    // the block size: thread t of the first SUM_T takes i = t, t + SUM_T, ..., a warp's lanes
+    // are added by a fixed butterfly and the warps' sums in turn (warps beyond m add 0).
+    // a = u / U is written as u (hi + lo), 1 / U as two FP32 numbers: one rounding of a product
+    // exact to 2^-48.
     const float rr = pp.r;
-    const double U = pp.inflate ? ordered_sum(m, [top, rr](int i) {
-        return float_to_double(inflate_value(key_val(top[i]), rr)); }, sh->red4) : 0.0;
-    const double invU = U > 0.0 ? 1.0 / U : 0.0;
-    double ch = 0.0;
-    if (pp.inflate) {
-        float umax = 0.0f;
-        const double sq = ordered_sum(m, [&](int i) {
-            const uint64_t x = top[i];
-            const float u = inflate_value(key_val(x), rr);
-            const double a = float_to_double(u) * invU;
-            umax = fmaxf(umax, u);
-            out_row[i] = key_row(x);
-            out_val[i] = (float)a;
-            return a * a; }, sh->red4);
-        // the largest u gives the largest a (rounding is monotone)
-        const double mx = block_max_d<T>((double)umax * invU, &sh->bs);
-        ch = mx - sq;
-        if (ch < 0.0) ch = 0.0;
-    } else {
+    if (!pp.inflate) {
         for (int i = tid; i < m; i += T) {
             const uint64_t x = top[i];
             out_row[i] = key_row(x);
             out_val[i] = key_val(x);
         }
+        if (tid == 0) {
+            *mstar_out = m;
+            *chaos_out = 0.0;
+        }
+        __syncthreads();
+        return;
     }
-    if (tid == 0) {
-        *mstar_out = m;
-        *chaos_out = ch;
+    if (tid < SUM_T) {
+        double su = 0.0, su2 = 0.0;
+        float mu = 0.0f;
+        if (warp * 32 < m) {
+            for (int i = tid; i < m; i += SUM_T) {
+                const float u = inflate_value(key_val(top[i]), rr);
+                const double x = float_to_double(u);
+                su += x;
+                su2 += x * x;
+                mu = fmaxf(mu, u);
+            }
+            su = warp_sum(su);
+            su2 = warp_sum(su2);
+            mu = __uint_as_float(__reduce_max_sync(FULL, __float_as_uint(mu)));  // mu >= 0
+        }
+        if (lane == 0) {
+            sh->sum4[0][warp] = su;
+            sh->sum4[1][warp] = su2;
+            sh->max4[warp] = mu;
+        }
     }
     __syncthreads();
-}
-
-// Append the candidates an enumerator yields to top[0..ntop); first cuts
-// the buffer back to ksel entries if they would not fit.  `count(tau)`
-// returns this thread's number of keys > tau; `emit(tau, dst, base)` writes
-// this thread's keys at dst[base ...] (base: its exclusive scan offset).
-template <int T, int IPT, class Enum>
-__device__ __forceinline__ void append_candidates(Enum& en, uint64_t* top, int topcap, int ksel,
-                                                  int& ntop, uint64_t& tau, int c, unsigned* hist,
-                                                  WinShared* sh) {
-    int C;
-    int base = block_scan_excl<T>(c, &C, sh->wsm);
-    if (ntop + C > topcap) {
-        // invariant: C <= window capacity = topcap - ksel, so ntop > ksel here
-        const uint64_t kap = block_select_count<T>(top, ntop, top, 0, ksel, hist, &sh->bs);
-        ntop = compact_stable<T, IPT>(top, ntop, kap, sh->wsm);
-        tau = kap;
-        c = en.count(tau);
-        base = block_scan_excl<T>(c, &C, sh->wsm);
+    if (tid == 0) {
+        const double U = ((sh->sum4[0][0] + sh->sum4[0][1]) + sh->sum4[0][2]) + sh->sum4[0][3];
+        const double U2 = ((sh->sum4[1][0] + sh->sum4[1][1]) + sh->sum4[1][2]) + sh->sum4[1][3];
+        const float mu = fmaxf(fmaxf(sh->max4[0], sh->max4[1]), fmaxf(sh->max4[2], sh->max4[3]));
+        const double inv = U > 0.0 ? 1.0 / U : 0.0;
+        const float hi = (float)inv;
+        sh->inv = inv;
+        sh->inv_hi = hi;
+        sh->inv_lo = (float)(inv - (double)hi);
+        sh->flag = U > 1e-25 && U < 1e25;
+        // max a - sum a^2; the largest u gives the largest a
+        const double ch = (double)mu * inv - (U2 * inv) * inv;
+        sh->chaos = ch < 0.0 ? 0.0 : ch;
+        *mstar_out = m;
+        *chaos_out = sh->chaos;
     }
-    en.emit(tau, top + ntop, base);
-    ntop += C;
+    __syncthreads();
+    if (sh->flag) {
+        const float hi = sh->inv_hi, lo = sh->inv_lo;
+        for (int i = tid; i < m; i += T) {
+            const uint64_t x = top[i];
+            const float u = inflate_value(key_val(x), rr);
+            out_row[i] = key_row(x);
+            out_val[i] = fmaf(u, hi, __fmul_rn(u, lo));
+        }
+    } else {
+        const double inv = sh->inv;
+        for (int i = tid; i < m; i += T) {
+            const uint64_t x = top[i];
+            out_row[i] = key_row(x);
+            out_val[i] = (float)((double)inflate_value(key_val(x), rr) * inv);
+        }
+    }
     __syncthreads();
 }
 

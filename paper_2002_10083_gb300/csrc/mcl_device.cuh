@@ -187,6 +187,8 @@ __device__ uint64_t block_select_count(const uint64_t* A, int na, const uint64_t
     return prefix;
 }
 
+__device__ __forceinline__ unsigned long long fixed_of(float v, int f);
+
 // Radix select by mass over the distinct keys of A[0..na): the smallest m
 // such that the m largest keys carry value mass >= target (target > 0).
 // Returns 1 and sets *kappa (a lower bound whose >= set is exactly those m
@@ -242,7 +244,7 @@ __device__ int block_select_mass(const uint64_t* A, int na, double target, uint6
                 const unsigned grp = __match_any_sync(act, dg);
                 // group sum of the fixed-point masses (< 2^50 each) as two
                 // 25-bit halves, each summed exactly in 32 bits
-                const unsigned long long fx = __float2ull_rz(ldexpf(key_val(x), sh50));
+                const unsigned long long fx = fixed_of(key_val(x), sh50);
                 const unsigned lo25 = __reduce_add_sync(grp, (unsigned)(fx & 0x1FFFFFFull));
                 const unsigned hi25 = __reduce_add_sync(grp, (unsigned)(fx >> 25));
                 if (__ffs(grp) - 1 == lane) {
@@ -398,8 +400,10 @@ struct FixScale {
     int f;
     __device__ static float pow2(int e) { return __int_as_float((e + 127) << 23); }
     __device__ void init(double s) {
-        int e = 0;
-        frexp(s > 0.0 ? s * (1.0 + 1.0 / 1048576.0) : 1.0, &e);  // s (with margin) < 2^e
+        // s plus 2^-19 of its power of two is below 2^e; from its bits, since every
+        // thread does this and FP64 instructions run at 2 lanes per clock and SM
+        const unsigned hi = s > 0.0 ? (unsigned)__double2hiint(s) + (1u << 1) : 0x3FF00000u;
+        const int e = (int)(hi >> 20) - 1022;
         f = 62 - e;
         // both factors are normal numbers
         const int f1 = max(-126, min(126, f)), f2 = max(-126, min(126, f - f1));
@@ -432,10 +436,17 @@ struct FixScale {
     }
     // a lower bound of every sum whose value is >= v
     __device__ __forceinline__ unsigned long long lower(float v) const {
-        const double x = ldexp((double)v * (1.0 - 1.0 / 1048576.0), f);
-        return x < 9.0e18 ? (unsigned long long)x : 9000000000000000000ull;
+        const unsigned long long x = qv(v);
+        return x - (x >> 20) - (x != 0ull);
     }
 };
+
+// trunc(v * 2^f) of 0 <= v < 2^(62 - f), by shifts where the scale allows them
+__device__ __forceinline__ unsigned long long fixed_of(float v, int f) {
+    FixScale fx;
+    fx.f = f;
+    return fx.qv(v);
+}
 
 // Inflation (Alg. 1, Hadamard power r) of one FP32 value.
 __device__ __forceinline__ float inflate_value(float v, float r) {

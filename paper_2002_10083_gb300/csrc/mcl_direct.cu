@@ -572,12 +572,11 @@ __global__ void __launch_bounds__(DIR_T, DIR_MINB) k_expand_direct(DirectArgs a)
         double dv[1] = {0.0};
         long long qv[3] = {s_t, (long long)s_n, (long long)s_mt};
         block_sum<T>(dv, 0, qv, 3, &sh->bs);
-        const double MT = ldexp((double)(unsigned long long)qv[2], -fx.f);
         int mstar = 0;
         double ch = 0.0;
         const int64_t obase = b.off[j];
         // the table is free (and zero) here: radix counters of the row sort
-        finish_column<T, IPT, false>(top, ntop, topcap, a.pp, S, MT, qv[0], b.cap[j],
+        finish_column<T, IPT, false>(top, ntop, topcap, a.pp, S, (unsigned long long)qv[2], fx.f, qv[0], b.cap[j],
                                      b.tmp_row + (obase - b.tmp_off0), b.tmp_val + (obase - b.tmp_off0),
                                      hist, mhist, sh, ctr, lo, span, lo32, &mstar, &ch);
         for (int i = tid; i < NW * 256; i += T) lo32[i] = 0u;

@@ -94,7 +94,7 @@ struct ExpandBuffers {
     int32_t* bucket_row;   // per CTA: bucket_cap (row, bits(a_ik * a_kj)) pairs (int2)
     int32_t* woff;         // per CTA: window offsets into the bucket (WINDOW_MAX + 1)
     int64_t bucket_cap;
-    uint64_t* spill;    // CONF_DIRECT, per CTA: candidates beyond the shared buffer
+    uint64_t* spill;    // per CTA: candidates beyond the shared buffer, one window's at most
     int64_t* scan_tmp;  // tile sums
     int64_t scan_tmp_len;
     DevCounters* ctr;
@@ -129,6 +129,7 @@ void launch_plan_small(int32_t n, bool exact, int64_t staging, const PruneParams
                        const ExpandBuffers& b, int mask, DevCounters* host, cudaStream_t s);
 void launch_result_small(const CscView& A, const ExpandBuffers& b, int64_t* colptr, DevCounters* host,
                          cudaStream_t s);
+size_t numeric_spill_bytes(const PruneParams& pp, int num_sms);
 int numeric_grid(int conf, const PruneParams& pp, int num_sms);
 constexpr int WINDOW_MAX = 4096;  // windows per column in bucket mode
 int direct_grid(int ksel, int num_sms);

@@ -19,19 +19,25 @@
 //
 //   1. insert:  every product of the window is added into its slot: row - r0
 //               in a window of at most HS rows, else linear probing from a
-//               multiplicative hash (int32 row keys claimed by
-//               compare-and-swap, uint64 sums added with integer atomics);
-//   2. extract: over the table, the ranking key (FP32 value bits, row) of
-//               every entry replaces its sum in place, with the exact column
-//               statistics (count, count and mass at or above the
-//               threshold); the keys above the running top-k bound tau go to
-//               a candidate buffer that is cut back to the top ksel keys
-//               (radix select) when full;
-//   3. clear:   the table.
+//               multiplicative hash (keys claimed by compare-and-swap), the
+//               sum as two 32-bit words.  Four products per lane and round:
+//               their first probes are issued together, then their low words'
+//               additions, then the high words' with the carries;
+//   2. extract: one scan of the table, which clears it: sums below both the
+//               threshold and the running top-k bound are only counted, the
+//               others update the statistics, and ranking keys (FP32 value
+//               bits, row) above the bound go to a candidate buffer and past
+//               its end to a spill in global memory; when the buffer was too
+//               small it is cut back to the top ksel keys (radix select).
+//
+// A window takes two or three barriers.  (With the plan of each window
+// published by one thread, a block scan for the candidates' positions and
+// separate passes for extraction, emission and clearing there were ten.)
 //
 // Windows come from per-window product buckets (a counting pass and a
-// scatter of (row, FP32 product) into window order) or, without bucket
-// space, from per-source cursors over the sorted rows.  A hashed window whose
+// scatter of (row, FP32 product) into window order); a column that is one
+// small window from its sources, product by product; without bucket space
+// from per-source cursors over the sorted rows.  A hashed window whose
 // probe runs exceed PMAX slots is split by rows and redone (counted as a
 // split), and the rest of the column starts at the width that fitted;
 // results never depend on the size estimate.  Finally the prune rule picks
@@ -46,94 +52,17 @@
 
 namespace mcl {
 
-// ---------------------------------------------------------------------------
-// the accumulator: int32 row keys and uint64 fixed-point sums per slot
-// ---------------------------------------------------------------------------
+constexpr int PMAX = 64;          // probe run that marks a hashed window as overflowed
+constexpr int FLAT_SOURCES = 256; // a column of so few sources and products in one window:
+constexpr int FLAT_PRODUCTS = 65536;  // every lane finds its own products' sources
 
-constexpr int KEY_EMPTY = -1;
-constexpr int PMAX = 64;  // probe run that marks a hashed window as overflowed
-
-// *p += v in shared memory, as two 32-bit atomics: the low word's returns the
-// old value, whose carry goes into the high word's.  A 64-bit shared-memory
-// addition is a compare-and-swap loop on this GPU: 1.7 per clock and SM at
-// random slots against 3.9 (11 for a 32-bit one).
-__device__ __forceinline__ void red_add_u64(unsigned long long* p, unsigned long long v) {
-    unsigned* w = reinterpret_cast<unsigned*>(p);
-    const unsigned lo = (unsigned)v;
-    const unsigned old = atomicAdd(w, lo);
-    const unsigned hi = (unsigned)(v >> 32) + (old + lo < old ? 1u : 0u);
-    if (hi) atomicAdd(w + 1, hi);
-}
-
-__device__ __forceinline__ int cas_shared(int* p, int cmp, int val) {
-    int old;
-    asm volatile("atom.shared.cas.b32 %0, [%1], %2, %3;"
-                 : "=r"(old)
-                 : "r"((unsigned)__cvta_generic_to_shared(p)), "r"(cmp), "r"(val)
-                 : "memory");
-    return old;
-}
-
-// Home slot of a row in a hashed window: multiplicative hash scaled to HS
-// slots (any HS).
-template <int HS>
-__device__ __forceinline__ int table_home(int row) {
-    return (int)(((uint64_t)((uint32_t)row * 0x9E3779B1u) * (uint64_t)HS) >> 32);
-}
-
-// Add q at `row`: slot row - r0 in an identity window (rows of the window
-// span at most HS slots; every writer of a slot stores the same row), else
-// linear probing from the row's hash, an empty slot claimed by
-// compare-and-swap.  A probe run of PMAX slots sets *ovf and adds nothing.
-template <int HS, bool IDENT>
-__device__ __forceinline__ void acc_add(int row, unsigned long long q, int r0, int* keys,
-                                        unsigned long long* vals, int* ovf) {
-    if (IDENT) {
-        const unsigned h = (unsigned)(row - r0);
-        if (h >= (unsigned)HS) {  // cannot happen: a window's segments hold rows in [r0, r1)
-            *ovf = 2;
-            return;
-        }
-        keys[h] = row;
-        red_add_u64(vals + h, q);
-        return;
-    }
-    int h = table_home<HS>(row);
-    for (int p = 0; p < PMAX; ++p) {
-        int k = *reinterpret_cast<volatile int*>(keys + h);
-        if (k == KEY_EMPTY) {
-            k = cas_shared(keys + h, KEY_EMPTY, row);
-            if (k == KEY_EMPTY) k = row;
-        }
-        if (k == row) {
-            red_add_u64(vals + h, q);
-            return;
-        }
-        if (++h == HS) h = 0;
-    }
-    *ovf = 1;
-}
-
-// Expected entries per source and window below which a window walks its
-// sources one per lane instead of one per warp.
-constexpr int LANE_MODE_MAX = 12;
-
-// The ranking keys of a window's table after extraction (0: empty slot;
-// thread t takes slots t, t + T, ...).
-template <int T, int HS>
-struct KeyEnum {
-    const uint64_t* vk;
-    __device__ int count(uint64_t tau) const {
-        int c = 0;
-        for (int h = threadIdx.x; h < HS; h += T) c += vk[h] > tau;
-        return c;
-    }
-    __device__ void emit(uint64_t tau, uint64_t* dst, int base) const {
-        for (int h = threadIdx.x; h < HS; h += T) {
-            const uint64_t k = vk[h];
-            if (k > tau) dst[base++] = k;
-        }
-    }
+struct ExpandShared {
+    WinShared w;
+    int cand;       // candidates of the window
+    int went[2];    // entries of the window, by window parity
+    int next[2];    // source counters, by window parity
+    int full;       // a bucket, or a hashed window, was too small
+    int upre[FLAT_SOURCES + 1];  // first product of each source
 };
 
 struct ExpandArgs {
@@ -147,25 +76,28 @@ struct ExpandArgs {
 template <int T, int HS>
 struct ExpandLayout {
     static constexpr size_t bytes(int ksel) {
-        return (size_t)HS * 12 + (size_t)(ksel + HS) * 8 + 256 * 4 + 256 * 8 + sizeof(WinShared);
+        return (size_t)HS * 12 + 2 * 32 * 4 + 256 * 4 + 256 * 8 + sizeof(ExpandShared) + (size_t)(ksel + HS) * 8;
     }
 };
 
 template <int T, int HS, int MINB>
 __global__ void __launch_bounds__(T, MINB) k_expand(ExpandArgs a) {
     const int PLAN = a.plan;  // distinct rows a window is planned for
-    constexpr int IPT = 8;
+    constexpr int IPT = 8, NW = T / 32;
     static_assert(HS >= (T / 32) * 256, "the row sort's counters fit in the key array");
+    static_assert(HS % (T * 4) == 0, "the scan takes four slots per thread");
     extern __shared__ __align__(16) unsigned char smem[];
-    unsigned long long* vals = reinterpret_cast<unsigned long long*>(smem);
-    int* keys = reinterpret_cast<int*>(vals + HS);
-    uint64_t* vkeys = reinterpret_cast<uint64_t*>(vals);  // ranking keys after extraction
-    uint64_t* top = reinterpret_cast<uint64_t*>(keys + HS);
+    // sums' words and keys (row + 1, 0 = empty); idle lanes add 0 beyond the slots
+    unsigned* lo32 = reinterpret_cast<unsigned*>(smem);
+    unsigned* hi32 = lo32 + HS + 32;
+    int* keys = reinterpret_cast<int*>(hi32 + HS + 32);
+    unsigned long long* mhist = reinterpret_cast<unsigned long long*>(keys + HS);
+    unsigned* hist = reinterpret_cast<unsigned*>(mhist + 256);
     const int ksel = a.pp.ksel;
-    const int topcap = ksel + HS;  // a window adds at most HS candidates
-    unsigned* hist = reinterpret_cast<unsigned*>(top + topcap);
-    unsigned long long* mhist = reinterpret_cast<unsigned long long*>(hist + 256);
-    WinShared* sh = reinterpret_cast<WinShared*>(mhist + 256);
+    const int topcap = ksel + HS;
+    uint64_t* top = reinterpret_cast<uint64_t*>(hist + 256);
+    ExpandShared* es = reinterpret_cast<ExpandShared*>(top + topcap);
+    WinShared* sh = &es->w;
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const CscView& A = a.A;
@@ -178,54 +110,45 @@ __global__ void __launch_bounds__(T, MINB) k_expand(ExpandArgs a) {
     // window starts and ends in the bucket (per CTA: WINDOW_MAX + 1 of each)
     int32_t* woff = b.woff ? b.woff + (int64_t)blockIdx.x * 2 * (WINDOW_MAX + 1) : nullptr;
     int32_t* wlim = woff ? woff + (WINDOW_MAX + 1) : nullptr;
+    uint64_t* spill = b.spill + (int64_t)blockIdx.x * HS;
     const int wbeg = ctr->bin_off[a.conf * NZ], wend = ctr->bin_off[a.conf * NZ + NZ];
     if (ctr->err & ERR_STAGING) return;  // the iteration is redone without the graph
 
-    for (int i = tid; i < HS; i += T) {
-        keys[i] = KEY_EMPTY;
-        vals[i] = 0ull;
-    }
+    for (int i = tid; i < HS + 32; i += T) lo32[i] = hi32[i] = 0u;
+    for (int i = tid; i < HS; i += T) keys[i] = 0;
     const float theta = a.pp.theta;
     for (;;) {
-        if (tid == 0) sh->item = atomicAdd(&ctr->conf_ctr[a.conf], 1);
+        if (tid == 0) {
+            sh->item = atomicAdd(&ctr->conf_ctr[a.conf], 1);
+            es->cand = 0;
+            es->went[0] = 0;
+            es->went[1] = 0;
+            es->next[0] = 0;
+            es->full = 0;
+        }
         __syncthreads();
         const int item = sh->item;
-        __syncthreads();
         if (wbeg + item >= wend) break;
         const int j = b.work[wbeg + item];
         const int64_t cb = A.colptr[j], ce = A.colptr[j + 1];
         const int d = (int)(ce - cb);
         const int lo = b.rlo[j], hiE = b.rhi[j] + 1;
-        if (d == 0 || hiE <= lo) {
+        const bool empty = d == 0 || hiE <= lo;
+        if (empty || d > b.cur_stride) {
             if (tid == 0) {
+                if (!empty) set_err2(ctr, ERR_CURSOR);
                 b.kept[j] = 0;
                 b.chaos[j] = 0.0;
                 b.bnnz[j] = 0;
             }
-            continue;
-        }
-        if (d > b.cur_stride) {
-            if (tid == 0) {
-                set_err2(ctr, ERR_CURSOR);
-                b.kept[j] = 0;
-                b.chaos[j] = 0.0;
-                b.bnnz[j] = 0;
-            }
+            __syncthreads();
             continue;
         }
         const int span = hiE - lo;
         const int64_t flops_j = b.flops[j];
+        const double S = b.bsum[j];
         int64_t est = b.est[j];
         if (est < 1) est = 1;
-        for (int i = tid; i < d; i += T) {
-            const int k = A.rowidx[cb + i];
-            const int64_t ks = A.colptr[k];
-            const float akj = A.val[cb + i];
-            meta.ks[i] = ks;
-            meta.len[i] = (int)(A.colptr[k + 1] - ks);
-            meta.cur[i] = 0;
-            meta.akj[i] = akj;
-        }
         // ---- plan: about est / PLAN windows of equal row width.  With bucket
         // space the products go to per-window buckets, and a window that
         // overflows the table is split by rows (later windows of the column
@@ -251,30 +174,72 @@ __global__ void __launch_bounds__(T, MINB) k_expand(ExpandArgs a) {
             }
         }
         const int nwin = (int)(((int64_t)span + width - 1) / width);
+        if (nwin == 1) bucket = false;  // one window: straight from the sources
+        const bool flat = nwin == 1 && d <= FLAT_SOURCES && flops_j <= FLAT_PRODUCTS;
+        if (flat) {
+            // the sources' first products by a scan over the block
+            constexpr int PER = (FLAT_SOURCES + T - 1) / T;
+            int len[PER], sum = 0;
+#pragma unroll
+            for (int q = 0; q < PER; ++q) {
+                const int i = tid * PER + q;
+                len[q] = 0;
+                if (i < d) {
+                    const int k = A.rowidx[cb + i];
+                    const int64_t ks = A.colptr[k];
+                    len[q] = (int)(A.colptr[k + 1] - ks);
+                    meta.ks[i] = ks;
+                    meta.len[i] = len[q];
+                    meta.cur[i] = 0;
+                    meta.akj[i] = A.val[cb + i];
+                }
+                sum += len[q];
+            }
+            int tot;
+            int at = block_scan_excl<T>(sum, &tot, sh->wsm);
+#pragma unroll
+            for (int q = 0; q < PER; ++q) {
+                const int i = tid * PER + q;
+                if (i < d) es->upre[i] = at;
+                at += len[q];
+            }
+            if (tid == 0) es->upre[d] = tot;
+        } else {
+            for (int i = tid; i < d; i += T) {
+                const int k = A.rowidx[cb + i];
+                const int64_t ks = A.colptr[k];
+                meta.ks[i] = ks;
+                meta.len[i] = (int)(A.colptr[k + 1] - ks);
+                meta.cur[i] = 0;
+                meta.akj[i] = A.val[cb + i];
+            }
+        }
         int ntop = 0;
         uint64_t tau = 0;
+        unsigned long long qmin = 0;  // sums below it are neither candidates nor >= theta
         unsigned long long s_mt = 0;
-        long long s_t = 0, s_n = 0;
-        FastDiv fdiv;
-        fdiv.init((uint32_t)width);
-        __syncthreads();
-        const double S = b.bsum[j];
+        long long s_t = 0;
+        unsigned s_n = 0;
         FixScale fx;
         fx.init(S);
+        const bool plain = fx.plain();
+        __syncthreads();
 
         if (bucket) {
-            int* wcnt = reinterpret_cast<int*>(vals);  // nwin <= HS counters each
-            int* wcur = wcnt + HS;
+            int* wcnt = reinterpret_cast<int*>(lo32);  // nwin <= HS counters each
+            int* wcur = reinterpret_cast<int*>(hi32);
+            FastDiv fdiv;
+            fdiv.init((uint32_t)width);
             // Scatter (row, a_ik * a_kj) into the window buckets from the cursors wcur;
             // with a capacity capw per window (window w owns [w capw, (w + 1) capw))
-            // a run that would pass its window's end sets sh->next2[1] and writes
+            // a run that would pass its window's end sets es->full and writes
             // nothing past it.
             auto scatter = [&](int capw) {
-                if (tid == 0) sh->next = 0;
+                if (tid == 0) es->next[1] = 0;
                 __syncthreads();
                 for (;;) {
                     int kidx = 0;
-                    if (lane == 0) kidx = atomicAdd(&sh->next, 1);
+                    if (lane == 0) kidx = atomicAdd(&es->next[1], 1);
                     kidx = __shfl_sync(FULL, kidx, 0);
                     if (kidx >= d) break;
                     const int len = meta.len[kidx];
@@ -316,7 +281,7 @@ __global__ void __launch_bounds__(T, MINB) k_expand(ExpandArgs a) {
                                 const int end = after ? __ffs(after) - 1 : __popc(act);
                                 base = atomicAdd(wcur + w, end - lane);
                                 if (capw > 0 && base + (end - lane) > ((int)w + 1) * capw)
-                                    sh->next2[1] = 1;
+                                    es->full = 1;
                             }
                             // the head of this lane's run: the highest head at or below it
                             const int hl = 31 - __clz(heads & ((2u << lane) - 1u));
@@ -345,10 +310,10 @@ __global__ void __launch_bounds__(T, MINB) k_expand(ExpandArgs a) {
             if (capw64 * nwin <= b.bucket_cap) {
                 const int capw = (int)capw64;
                 for (int i = tid; i < nwin; i += T) wcur[i] = i * capw;
-                if (tid == 0) sh->next2[1] = 0;
+                if (tid == 0) es->full = 0;
                 __syncthreads();
                 scatter(capw);
-                counted = sh->next2[1] != 0;  // a window was fuller than its capacity
+                counted = es->full != 0;  // a window was fuller than its capacity
                 if (!counted)
                     for (int i = tid; i < nwin; i += T) {
                         woff[i] = i * capw;
@@ -359,11 +324,11 @@ __global__ void __launch_bounds__(T, MINB) k_expand(ExpandArgs a) {
             if (counted) {
                 // ---- count the products of every window ----
                 for (int i = tid; i < nwin; i += T) wcnt[i] = 0;
-                if (tid == 0) sh->next = 0;
+                if (tid == 0) es->next[1] = 0;
                 __syncthreads();
                 for (;;) {
                     int kidx = 0;
-                    if (lane == 0) kidx = atomicAdd(&sh->next, 1);
+                    if (lane == 0) kidx = atomicAdd(&es->next[1], 1);
                     kidx = __shfl_sync(FULL, kidx, 0);
                     if (kidx >= d) break;
                     const int len = meta.len[kidx];
@@ -413,247 +378,274 @@ __global__ void __launch_bounds__(T, MINB) k_expand(ExpandArgs a) {
                 __syncthreads();
                 scatter(0);
             }
-            for (int i = tid; i < HS; i += T) vals[i] = 0ull;
+            for (int i = tid; i < nwin; i += T) {
+                wcnt[i] = 0;
+                wcur[i] = 0;
+            }
+            if (tid == 0) es->full = 0;
+            __syncthreads();
         }
 
-        // ---- windows ----
-        // Thread 0 plans every window and publishes it; bucket mode: bucket
-        // window f0 = [f0, f1) (rows [r0, r1) of it while it is split);
-        // cursor mode: rows [r0, r1).
-        int f0 = 0, f1 = 0;
-        bool rowsplit = false;
-        int split_w = 0;  // > 0: rows per piece when windows are being split
-        int r0 = lo, r1 = lo;
-        int cwidth = width;  // cursor mode: current window width
+        // four products per lane (row h + r0 of the window for h < wr) into their slots' sums
+        auto add4 = [&](const unsigned (&h)[4], const float (&v)[4], unsigned wr, int r0, bool hash) {
+            unsigned slot[4], ql[4], qh[4], old[4];
+            int key[4];
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+                const bool in = h[c] < wr;
+                const unsigned long long q = plain ? fx.qplain(v[c]) : fx.qv(v[c]);
+                ql[c] = in ? (unsigned)q : 0u;
+                qh[c] = in ? (unsigned)(q >> 32) : 0u;
+                key[c] = in ? (int)h[c] + r0 + 1 : 0;
+                slot[c] = hash ? __umulhi((unsigned)key[c] * 0x9E3779B1u, (unsigned)HS) : h[c];
+            }
+            if (hash) {
+                int got[4];
+#pragma unroll
+                for (int c = 0; c < 4; ++c) got[c] = key[c] ? atomicCAS(keys + slot[c], 0, key[c]) : 0;
+#pragma unroll
+                for (int c = 0; c < 4; ++c) {
+                    for (int p = 0; got[c] != 0 && got[c] != key[c]; ++p) {
+                        if (p == PMAX) {
+                            es->full = 1;
+                            key[c] = 0;
+                            ql[c] = 0u;
+                            qh[c] = 0u;
+                            break;
+                        }
+                        slot[c] = slot[c] + 1 == HS ? 0 : slot[c] + 1;
+                        got[c] = atomicCAS(keys + slot[c], 0, key[c]);
+                    }
+                }
+            }
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+                if (!hash && key[c]) keys[slot[c]] = key[c];
+                slot[c] = key[c] ? slot[c] : (unsigned)(HS + lane);
+            }
+#pragma unroll
+            for (int c = 0; c < 4; ++c) old[c] = atomicAdd(lo32 + slot[c], ql[c]);
+#pragma unroll
+            for (int c = 0; c < 4; ++c) atomicAdd(hi32 + slot[c], qh[c] + (old[c] + ql[c] < old[c] ? 1u : 0u));
+        };
+
+        // ---- windows: w counts the bucket windows; pw rows at once of the window's rows up to
+        // we (all of them unless it has to be split); without buckets one window, pw rows at once ----
         int32_t* cur = meta.cur;
         int32_t* nxt = meta.nxt;
-        const bool lane_mode =
-            !bucket && (double)flops_j * (double)width < (double)LANE_MODE_MAX * (double)d * (double)span;
-        auto plan = [&](int f) {  // thread 0 only
-            while (f < nwin && wlim[f] == woff[f]) ++f;  // empty windows
-            f0 = f;
-            f1 = f;
-            rowsplit = false;
-            if (f >= nwin) return;
-            if (split_w > 0) {
-                const int ws = lo + f * width;
-                const int we = (int)min((int64_t)ws + width, (int64_t)hiE);
-                if (split_w < we - ws) {
-                    rowsplit = true;
-                    f1 = f + 1;
-                    r0 = ws;
-                    r1 = ws + split_w;
-                    return;
-                }
-                split_w = 0;
+        const int batch = max(1, min(32, d / (4 * NW)));  // sources a warp takes at once
+        int w = 0, pw = width;
+        int we = bucket ? (int)min((int64_t)lo + width, (int64_t)hiE) : hiE;
+        int r0 = lo, r1 = (int)min((int64_t)r0 + pw, (int64_t)we);
+        for (int it = 0; r0 < hiE; ++it) {
+            const unsigned wr = (unsigned)(r1 - r0);
+            const bool hash = wr > (unsigned)HS;
+            if (tid == 0) {
+                es->next[(it + 1) & 1] = 0;
+                es->went[(it + 1) & 1] = 0;
             }
-            f1 = f + 1;
-        };
-        auto publish = [&](int nextpar) {  // thread 0 only
-            sh->pf0 = f0;
-            sh->pf1 = f1;
-            sh->pr0 = r0;
-            sh->pr1 = r1;
-            sh->prs = rowsplit ? 1 : 0;
-            sh->pdone = bucket ? f0 >= nwin : r0 >= hiE;
-            sh->ovf2[nextpar] = 0;
-            sh->went2[nextpar] = 0;
-            sh->next2[nextpar] = 0;
-        };
-        if (tid == 0) {
-            if (bucket)
-                plan(0);
-            else
-                r1 = (int)min((int64_t)lo + cwidth, (int64_t)hiE);
-            publish(0);
-        }
-        for (int it = 0;; ++it) {
-            const int par = it & 1;
-            __syncthreads();  // this window's plan and flags are published
-            if (sh->pdone) break;
-            const int F0 = sh->pf0, R0 = sh->pr0, R1 = sh->pr1;
-            const bool RS = sh->prs != 0;
-            int* ovfp = &sh->ovf2[par];
-            // rows of this window: a bucket window (or its split piece) or the cursor range;
-            // at most HS rows wide, it maps row - wr0 to its slot (no hashing)
-            const int wr0 = bucket ? (RS ? R0 : lo + F0 * width) : R0;
-            const int wr1 =
-                bucket ? (RS ? R1 : (int)min((int64_t)lo + (int64_t)(F0 + 1) * width, (int64_t)hiE))
-                       : R1;
-            const bool ident = wr1 - wr0 <= HS;
-            auto add = [&](int row, unsigned long long q) {
-                if (ident)
-                    acc_add<HS, true>(row, q, wr0, keys, vals, ovfp);
-                else
-                    acc_add<HS, false>(row, q, wr0, keys, vals, ovfp);
-            };
             // ---- 1. insert the products of the window ----
             if (bucket) {
-                const int bs = woff[F0], be = wlim[F0];
-                // four products per lane in flight while the previous four update
-                // the table (the loads are issued before the shared atomics)
+                const int be = wlim[w];
+                int pb = woff[w] + warp * 128;
                 int2 cx[4];
-                int pb = bs + warp * 128;
 #pragma unroll
                 for (int u = 0; u < 4; ++u) {
                     const int p = pb + 32 * u + lane;
-                    cx[u] = p < be ? bkt[p] : make_int2(-1, 0);
+                    cx[u] = p < be ? bkt[p] : make_int2(INT_MAX, 0);
                 }
-                for (; pb < be; pb += T * 4) {
-                    int2 nx[4];
+                while (pb < be) {
+                    unsigned h[4];
+                    float v[4];
 #pragma unroll
                     for (int u = 0; u < 4; ++u) {
-                        const int p = pb + T * 4 + 32 * u + lane;
-                        nx[u] = p < be ? bkt[p] : make_int2(-1, 0);
+                        h[u] = (unsigned)(cx[u].x - r0);
+                        v[u] = __int_as_float(cx[u].y);
                     }
+                    pb += T * 4;
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) {  // the next round's, while these are added
+                        const int p = pb + 32 * u + lane;
+                        cx[u] = p < be ? bkt[p] : make_int2(INT_MAX, 0);
+                    }
+                    add4(h, v, wr, r0, hash);
+                }
+            } else if (flat && r0 == lo && r1 == hiE) {
+                const int F = (int)flops_j;
+                for (int tb = warp * 128; tb < F; tb += T * 4) {
+                    unsigned h[4];
+                    float v[4];
 #pragma unroll
                     for (int u = 0; u < 4; ++u) {
-                        const int row = cx[u].x;
-                        bool valid = row >= 0;
-                        if (RS) valid = valid && row >= R0 && row < R1;
-                        if (valid) add(row, fx.qv(__int_as_float(cx[u].y)));
+                        const int t = tb + 32 * u + lane;
+                        h[u] = 0xFFFFFFFFu;
+                        v[u] = 0.0f;
+                        if (t < F) {
+                            int s0 = 0, s1 = d;  // upre[s0] <= t < upre[s1]
+                            while (s1 - s0 > 1) {
+                                const int m = (s0 + s1) >> 1;
+                                if (es->upre[m] <= t) s0 = m; else s1 = m;
+                            }
+                            const int64_t p = meta.ks[s0] + (t - es->upre[s0]);
+                            h[u] = (unsigned)(__ldg(A.rowidx + p) - r0);
+                            v[u] = __fmul_rn(__ldg(A.val + p), meta.akj[s0]);
+                        }
                     }
-#pragma unroll
-                    for (int u = 0; u < 4; ++u) cx[u] = nx[u];
-                }
-            } else if (lane_mode) {
-                for (int kidx = tid; kidx < d; kidx += T) {
-                    const int64_t ks = meta.ks[kidx];
-                    const int32_t* rows = A.rowidx + ks;
-                    const float* vv = A.val + ks;
-                    const float akj = meta.akj[kidx];
-                    const int len = meta.len[kidx];
-                    int pos = cur[kidx];
-                    for (; pos < len; ++pos) {
-                        const int row = __ldg(rows + pos);
-                        if (row >= R1) break;
-                        add(row, fx.q(__ldg(vv + pos), akj));
-                    }
-                    nxt[kidx] = pos;
+                    add4(h, v, wr, r0, hash);
                 }
             } else {
+                int* next = &es->next[it & 1];
                 for (;;) {
-                    int kidx = 0;
-                    if (lane == 0) kidx = atomicAdd(&sh->next2[par], 1);
-                    kidx = __shfl_sync(FULL, kidx, 0);
-                    if (kidx >= d) break;
-                    const int64_t ks = meta.ks[kidx];
-                    const int32_t* rows = A.rowidx + ks;
-                    const float* vv = A.val + ks;
-                    const float akj = meta.akj[kidx];
-                    const int len = meta.len[kidx];
-                    int pos = cur[kidx];
-                    while (pos < len) {
-                        const int p = pos + lane;
-                        const int row = p < len ? __ldg(rows + p) : INT_MAX;
-                        const bool valid = row < R1;
-                        if (valid) add(row, fx.q(__ldg(vv + p), akj));
-                        const int nin = __popc(__ballot_sync(FULL, valid));
-                        pos += nin;
-                        if (nin < 32) break;
+                    int k0 = 0;
+                    if (lane == 0) k0 = atomicAdd(next, batch);
+                    k0 = __shfl_sync(FULL, k0, 0);
+                    if (k0 >= d) break;
+                    const int nb = min(batch, d - k0);
+                    for (int s = k0; s < k0 + nb; ++s) {
+                        const int len = meta.len[s];
+                        const int64_t ks = meta.ks[s];
+                        const float akj = meta.akj[s];
+                        int pos = cur[s];
+                        while (pos < len) {
+                            unsigned h[4];
+                            float v[4];
+#pragma unroll
+                            for (int c = 0; c < 4; ++c) {
+                                const int p = pos + 32 * c + lane;
+                                h[c] = (unsigned)((p < len ? __ldg(A.rowidx + ks + p) : INT_MAX) - r0);
+                                v[c] = p < len ? __ldg(A.val + ks + p) : 0.0f;
+                            }
+                            int nin = 0;
+#pragma unroll
+                            for (int c = 0; c < 4; ++c) {
+                                v[c] = __fmul_rn(v[c], akj);
+                                nin += __popc(__ballot_sync(FULL, h[c] < wr));
+                            }
+                            add4(h, v, wr, r0, hash);
+                            pos += nin;
+                            if (nin < 128) break;
+                        }
+                        if (lane == 0) nxt[s] = pos;
                     }
-                    if (lane == 0) nxt[kidx] = pos;
                 }
             }
             __syncthreads();
-            if (*ovfp) {
+            if (es->full) {  // split: a quarter of the rows at once from here on
                 for (int i = tid; i < HS; i += T) {
-                    keys[i] = KEY_EMPTY;
-                    vals[i] = 0ull;
+                    lo32[i] = 0u;
+                    hi32[i] = 0u;
+                    keys[i] = 0;
                 }
-                if (*ovfp == 2 && tid == 0) set_err2(ctr, ERR_INTERNAL);  // cannot happen
+                __syncthreads();
                 if (tid == 0) {
+                    es->full = 0;
                     atomicAdd(&ctr->splits, 1ull);
-                    if (bucket && !rowsplit) {
-                        // split the window's rows (a single row never overflows)
-                        rowsplit = true;
-                        r0 = lo + f0 * width;
-                        const int we = (int)min((int64_t)r0 + width, (int64_t)hiE);
-                        r1 = r0 + (we - r0) / 2;
-                    } else {
-                        r1 = r0 + (r1 - r0) / 2;
-                        cwidth = r1 - r0;
-                    }
-                    publish(par ^ 1);
                 }
+                pw = max(1, (r1 - r0) / 4);
+                r1 = r0 + pw;
                 continue;
             }
-            // ---- 2. statistics and candidates: every entry becomes its ranking key
-            // in place (exact statistics from the fixed-point sums), row keys cleared ----
-            KeyEnum<T, HS> en{vkeys};
-            int c = 0, cnt = 0;
-            for (int h = tid; h < HS; h += T) {
-                const int row = keys[h];
-                if (row != KEY_EMPTY) {
-                    const unsigned long long q = vals[h];
-                    const float v = fx.value(q);
-                    const uint64_t key = make_key(v, row);
-                    ++cnt;
-                    if (v >= theta) {
-                        ++s_t;
-                        s_mt += q;
-                    }
-                    c += key > tau;
-                    vkeys[h] = key;
-                    keys[h] = KEY_EMPTY;
+            // ---- 2. extract: one scan of the table, which it clears ----
+            const unsigned slots = hash ? (unsigned)HS : (wr + 127u) & ~127u;
+            unsigned n0 = s_n;
+            for (unsigned h = tid * 4; h < slots; h += T * 4) {  // four slots; whole warps
+                uint4* pl = reinterpret_cast<uint4*>(lo32 + h);
+                uint4* ph = reinterpret_cast<uint4*>(hi32 + h);
+                int4* pk = reinterpret_cast<int4*>(keys + h);
+                const uint4 l4 = *pl, h4 = *ph;
+                const int4 k4 = *pk;
+                const unsigned xl[4] = {l4.x, l4.y, l4.z, l4.w}, xh[4] = {h4.x, h4.y, h4.z, h4.w};
+                const int kk[4] = {k4.x, k4.y, k4.z, k4.w};
+                unsigned big = 0;  // slots to look at
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    const unsigned long long q = ((unsigned long long)xh[u] << 32) | xl[u];
+                    s_n += kk[u] != 0;
+                    big |= kk[u] != 0 && q >= qmin ? 1u << u : 0u;
                 }
-            }
-            s_n += cnt;
-            {
-                const int wc = warp_sum(cnt);
-                if (lane == 0 && wc) atomicAdd(&sh->went2[par], wc);
-            }
-            append_candidates<T, IPT>(en, top, topcap, ksel, ntop, tau, c, hist, sh);
-            // ---- 3. clear the table ----
-            for (int i = tid; i < HS; i += T) vkeys[i] = 0ull;
-            if (!bucket) {  // cursors advance past the window
-                int32_t* t = cur;
-                cur = nxt;
-                nxt = t;
-            }
-            // ---- 4. next window ----
-            if (tid == 0) {
-                const int went = sh->went2[par];  // complete: append_candidates ends with a barrier
-                if (bucket) {
-                    if (rowsplit) {
-                        const int we =
-                            (int)min((int64_t)lo + (int64_t)(f0 + 1) * width, (int64_t)hiE);
-                        int wd = r1 - r0;
-                        if (went < PLAN / 2 && wd < width) wd *= 2;
-                        r0 = r1;
-                        if (r0 >= we) {
-                            split_w = wd;
-                            plan(f0 + 1);
-                        } else {
-                            r1 = min(we, r0 + wd);
+                while (__any_sync(FULL, big != 0u)) {  // one slot per lane and round
+                    uint64_t key = 0;
+                    if (big) {
+                        const unsigned g = h + (unsigned)__ffs(big) - 1u;
+                        big &= big - 1u;
+                        const unsigned long long q = ((unsigned long long)hi32[g] << 32) | lo32[g];
+                        const float v = fx.value(q);
+                        if (v >= theta) {
+                            ++s_t;
+                            s_mt += q;
                         }
-                    } else {
-                        plan(f1);
+                        key = make_key(v, keys[g] - 1);
                     }
-                } else {
-                    r0 = r1;
-                    if (went < PLAN / 2 && cwidth < (1 << 29))
-                        cwidth *= 2;
-                    else if (went > PLAN + PLAN / 2 && cwidth > 1)
-                        cwidth /= 2;
-                    r1 = (int)min((int64_t)r0 + cwidth, (int64_t)hiE);
+                    const bool take = key > tau;
+                    const unsigned m = __ballot_sync(FULL, take);
+                    if (m) {
+                        int base = 0;
+                        if (lane == 0) base = atomicAdd(&es->cand, __popc(m));
+                        const int at = ntop + __shfl_sync(FULL, base, 0) + __popc(m & lanemask_lt());
+                        if (take) {
+                            if (at < topcap)
+                                top[at] = key;
+                            else
+                                spill[at - topcap] = key;
+                        }
+                    }
                 }
-                publish(par ^ 1);
+                *pl = make_uint4(0u, 0u, 0u, 0u);
+                *ph = make_uint4(0u, 0u, 0u, 0u);
+                *pk = make_int4(0, 0, 0, 0);
             }
+            n0 = __reduce_add_sync(FULL, s_n - n0);
+            if (lane == 0 && n0) atomicAdd(&es->went[it & 1], (int)n0);
+            __syncthreads();
+            const int have = ntop + es->cand, went = es->went[it & 1];
+            __syncthreads();
+            if (tid == 0) es->cand = 0;
+            if (have > topcap) {  // cut back to the ksel largest
+                const int over = have - topcap;
+                tau = block_select_count<T>(top, topcap, spill, over, ksel, hist, &sh->bs);
+                ntop = compact_stable<T, IPT>(top, topcap, tau, sh->wsm);
+                for (int i = tid; i < over; i += T) {
+                    const uint64_t x = spill[i];
+                    if (x >= tau) top[ntop + atomicAdd(&es->cand, 1)] = x;
+                }
+                __syncthreads();
+                ntop = ksel;
+                if (tid == 0) es->cand = 0;
+                qmin = fx.lower(fminf(theta, key_val(tau)));
+                __syncthreads();
+            } else {
+                ntop = have;
+            }
+            // ---- 3. next window ----
+            int32_t* t = cur;  // cursors advance past the window
+            cur = nxt;
+            nxt = t;
+            const bool whole = r1 - r0 >= width;
+            if (went < PLAN / 2 && (bucket ? !whole : pw < (1 << 29))) {
+                pw = bucket ? min(width, pw * 2) : pw * 2;
+            } else if (!bucket && went > PLAN + PLAN / 2 && pw > 1) {
+                pw /= 2;
+            }
+            r0 = r1;
+            if (bucket && r0 >= we) {
+                do ++w; while (w < nwin && wlim[w] == woff[w]);  // empty windows
+                r0 = w < nwin ? lo + w * width : hiE;
+                we = (int)min((int64_t)r0 + width, (int64_t)hiE);
+            }
+            r1 = (int)min((int64_t)r0 + pw, (int64_t)we);
         }
         double dv[1] = {0.0};
-        long long qv[3] = {s_t, s_n, (long long)s_mt};
+        long long qv[3] = {s_t, (long long)s_n, (long long)s_mt};
         block_sum<T>(dv, 0, qv, 3, &sh->bs);
-        const double MT = ldexp((double)(unsigned long long)qv[2], -fx.f);
         int mstar = 0;
         double ch = 0.0;
         const int64_t obase = b.off[j];
-        // the table's key array is free here: radix counters of the row sort
-        finish_column<T, IPT, false>(top, ntop, topcap, a.pp, S, MT, qv[0], b.cap[j],
+        // the table's key array is free here: counters of the row sort
+        finish_column<T, IPT, false>(top, ntop, topcap, a.pp, S, (unsigned long long)qv[2], fx.f, qv[0], b.cap[j],
                                      b.tmp_row + (obase - b.tmp_off0),
                                      b.tmp_val + (obase - b.tmp_off0), hist, mhist, sh, ctr, lo,
                                      span, reinterpret_cast<unsigned*>(keys), &mstar, &ch);
-        for (int i = tid; i < (T / 32) * 256; i += T) keys[i] = KEY_EMPTY;
+        for (int i = tid; i < (T / 32) * 256; i += T) keys[i] = 0;
         if (tid == 0) {
             b.kept[j] = mstar;
             b.chaos[j] = ch;
@@ -699,6 +691,16 @@ static void conf_launch(int conf, const CscView& A, const PruneParams& pp, const
     if (plan < 64) plan = 64;
     ExpandArgs a{A, pp, b, conf, plan};
     k_expand<C::T, C::HS, C::MINB><<<grid, C::T, conf_smem<C>(pp.ksel), s>>>(a);
+}
+
+// Bytes of candidate spill: a window's slots for every CTA of the largest configuration.
+size_t numeric_spill_bytes(const PruneParams& pp, int num_sms) {
+    const size_t hs = pp.table == 0 ? Conf1a::HS : Conf1b::HS;
+    static_assert(Conf1b::HS == Conf1c::HS, "one size for both wide shapes");
+    const size_t b0 = (size_t)numeric_grid(0, pp, num_sms) * Conf0::HS * 8;
+    const size_t b1 = (size_t)numeric_grid(CONF_LARGE, pp, num_sms) * hs * 8;
+    const size_t b2 = direct_spill_bytes(direct_grid(pp.ksel, num_sms));
+    return b0 > b1 ? (b0 > b2 ? b0 : b2) : (b1 > b2 ? b1 : b2);
 }
 
 int numeric_grid(int conf, const PruneParams& pp, int num_sms) {
@@ -868,11 +870,10 @@ __global__ void __launch_bounds__(PR_T, PR_MINB) k_prune(PruneArgs a) {
         double dv[1] = {0.0};
         long long qv[2] = {s_t, (long long)s_mt};
         block_sum<PR_T>(dv, 0, qv, 2, &sh->bs);
-        const double MT = ldexp((double)(unsigned long long)qv[1], -fx.f);
         int mstar = 0;
         double ch = 0.0;
         const int64_t obase = b.off[j];
-        finish_column<PR_T, 8, true>(top, ntop, topcap, a.pp, S, MT, qv[0], b.cap[j],
+        finish_column<PR_T, 8, true>(top, ntop, topcap, a.pp, S, (unsigned long long)qv[1], fx.f, qv[0], b.cap[j],
                                      b.tmp_row + (obase - b.tmp_off0),
                                      b.tmp_val + (obase - b.tmp_off0), hist, mhist, sh, b.ctr, 0,
                                      0, nullptr, &mstar, &ch);
