@@ -59,6 +59,63 @@ __device__ __forceinline__ int block_scan_excl(int x, int* total, int* wsm) {
     return res;
 }
 
+// Radix select by count over the distinct keys of A ++ B (bit 63 clear):
+// returns kappa with #{x : x >= kappa} == M exactly (1 <= M <= na + nb).  Most
+// significant digit first; stops as soon as the chosen bin holds exactly the
+// keys still needed, returning its prefix with zero low bits.  Digits of 11
+// bits: two passes for the values of a column where eight-bit digits take four
+// (the first of which sees two or three different exponents), and one shared
+// atomic per key.  bins: SEL_BINS counters, zero on entry and on return.
+constexpr int SEL_BINS = 2048;
+template <int T>
+__device__ uint64_t block_select_wide(const uint64_t* A, int na, const uint64_t* B, int nb, int M,
+                                      unsigned* bins, BlockScratch* bs, int* wsm) {
+    constexpr int PER = SEL_BINS / T;
+    const int tid = threadIdx.x, tot = na + nb;
+    uint64_t prefix = 0;
+    int need = M;
+    for (int shift = 52, bits = 11;;) {
+        const uint64_t himask = ~0ull << (shift + bits);
+        const unsigned dmask = (1u << bits) - 1u;
+        for (int i = tid; i < tot; i += T) {
+            const uint64_t x = cat_at(A, na, B, i);
+            if ((x & himask) == prefix) atomicAdd(bins + ((unsigned)(x >> shift) & dmask), 1u);
+        }
+        __syncthreads();
+        // thread t owns the bins from SEL_BINS - 1 - t PER down
+        int c[PER], sum = 0;
+#pragma unroll
+        for (int q = 0; q < PER; ++q) {
+            unsigned* bin = bins + (SEL_BINS - 1 - tid * PER - q);
+            c[q] = (int)*bin;
+            *bin = 0u;
+            sum += c[q];
+        }
+        int total;
+        int before = block_scan_excl<T>(sum, &total, wsm);
+        if (before < need && before + sum >= need) {
+#pragma unroll
+            for (int q = 0; q < PER; ++q) {
+                if (before < need && before + c[q] >= need) {
+                    bs->sel_prefix = prefix | ((uint64_t)(SEL_BINS - 1 - tid * PER - q) << shift);
+                    bs->sel_need = need - before;
+                    bs->sel_done = c[q] == need - before;
+                }
+                before += c[q];
+            }
+        }
+        __syncthreads();
+        prefix = bs->sel_prefix;
+        need = bs->sel_need;
+        const bool done = bs->sel_done != 0;
+        __syncthreads();
+        if (done || shift == 0) break;
+        bits = shift < 11 ? shift : 11;
+        shift -= bits;
+    }
+    return prefix;
+}
+
 // Stable in-place compaction of a[0..n) keeping keys >= cut; returns the
 // new length.  Each thread owns IPT consecutive elements per round; all
 // reads of a round precede its writes (the scan's barriers), and outputs
@@ -402,7 +459,7 @@ template <int T, int IPT, bool ROW_ORDERED>
 __device__ void finish_column(uint64_t* top, int ntop, int topcap, const PruneParams& pp, double S,
                               unsigned long long mt, int f, long long Tt, int64_t cap, int32_t* out_row,
                               float* out_val, unsigned* hist, unsigned long long* mhist,
-                              WinShared* sh, DevCounters* ctr, int row_lo, int row_span,
+                              unsigned* bins, WinShared* sh, DevCounters* ctr, int row_lo, int row_span,
                               unsigned* rscratch, int* mstar_out, double* chaos_out) {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     // FP64 work is one warp's, not every warp's: its instructions take 16 clocks
@@ -428,7 +485,7 @@ __device__ void finish_column(uint64_t* top, int ntop, int topcap, const PrunePa
     // finds, so neither the top-q mass nor m_rec is needed
     const bool krec_bound = q >= pp.Krec;
     if (!krec_bound && Tt > pp.K) {
-        kq = block_select_count<T>(top, ntop, top, 0, pp.K, hist, &sh->bs);
+        kq = block_select_wide<T>(top, ntop, top, 0, pp.K, bins, &sh->bs, sh->wsm);
         mq = mass_at_or_above<T>(top, ntop, kq, sh);
     }
     int mstar;
@@ -470,7 +527,7 @@ __device__ void finish_column(uint64_t* top, int ntop, int topcap, const PrunePa
         else if (mstar >= ntop)
             cut = 0ull;
         else
-            cut = block_select_count<T>(top, ntop, top, 0, mstar, hist, &sh->bs);
+            cut = block_select_wide<T>(top, ntop, top, 0, mstar, bins, &sh->bs, sh->wsm);
     }
     // the kept keys (exactly m* of them: keys are distinct) to the front
     m = mstar > 0 ? compact_stable<T, IPT>(top, ntop, cut, sh->wsm) : 0;

@@ -120,73 +120,6 @@ __device__ __forceinline__ uint64_t cat_at(const uint64_t* A, int na, const uint
     return i < na ? A[i] : B[i - na];
 }
 
-// Radix select by count over the distinct keys of A ++ B: returns kappa with
-// #{x : x >= kappa} == M exactly (1 <= M <= na + nb).  Most-significant
-// byte first; stops as soon as the chosen bucket holds exactly the keys
-// still needed, returning its prefix with zero low bits.  Histogram updates
-// are aggregated per warp over lanes with the same digit.  With SKIP0, zero
-// elements are not keys (empty slots of a table; every key is >= 1) and M
-// counts nonzero keys only.
-template <int T, bool SKIP0 = false>
-__device__ uint64_t block_select_count(const uint64_t* A, int na, const uint64_t* B, int nb, int M,
-                                       unsigned* hist, BlockScratch* bs) {
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int tot = na + nb;
-    uint64_t prefix = 0;
-    int need = M;
-    for (int shift = 56; shift >= 0; shift -= 8) {
-        const uint64_t hmask = (shift == 56) ? 0ull : (~0ull << (shift + 8));
-        for (int i = tid; i < 256; i += T) hist[i] = 0u;
-        __syncthreads();
-        for (int base = 0; base < tot; base += T) {
-            const int i = base + tid;
-            const bool valid = i < tot;
-            const uint64_t x = valid ? cat_at(A, na, B, i) : 0ull;
-            const bool in = valid && (!SKIP0 || x != 0ull) && (x & hmask) == prefix;
-            const unsigned act = __ballot_sync(FULL, in);
-            if (in) {
-                const unsigned dg = (unsigned)((x >> shift) & 255u);
-                const unsigned grp = __match_any_sync(act, dg);
-                if (__ffs(grp) - 1 == lane) atomicAdd(&hist[dg], (unsigned)__popc(grp));
-            }
-        }
-        __syncthreads();
-        if (warp == 0) {
-            // lane l owns buckets 255-8l ... 248-8l, scanned from the top
-            int c[8];
-            int lsum = 0;
-#pragma unroll
-            for (int q = 0; q < 8; ++q) {
-                c[q] = (int)hist[255 - 8 * lane - q];
-                lsum += c[q];
-            }
-            int incl = lsum;
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                int y = __shfl_up_sync(FULL, incl, o);
-                if (lane >= o) incl += y;
-            }
-            int before = incl - lsum;
-#pragma unroll
-            for (int q = 0; q < 8; ++q) {
-                if (before < need && before + c[q] >= need) {
-                    int d = 255 - 8 * lane - q;
-                    bs->sel_prefix = prefix | ((uint64_t)d << shift);
-                    bs->sel_need = need - before;
-                    bs->sel_done = (c[q] == need - before);
-                }
-                before += c[q];
-            }
-        }
-        __syncthreads();
-        prefix = bs->sel_prefix;
-        need = bs->sel_need;
-        if (bs->sel_done) break;
-    }
-    __syncthreads();
-    return prefix;
-}
-
 __device__ __forceinline__ unsigned long long fixed_of(float v, int f);
 
 // Radix select by mass over the distinct keys of A[0..na): the smallest m

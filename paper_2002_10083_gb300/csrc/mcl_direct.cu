@@ -549,7 +549,7 @@ __global__ void __launch_bounds__(DIR_T, DIR_MINB) k_expand_direct(DirectArgs a)
             }
             if (have > topcap) {  // cut back to the ksel largest
                 const int over = have - topcap;
-                tau = block_select_count<T>(top, topcap, spill, over, ksel, hist, &sh->bs);
+                tau = block_select_wide<T>(top, topcap, spill, over, ksel, lo32, &sh->bs, sh->wsm);
                 ntop = compact_stable<T, IPT>(top, topcap, tau, sh->wsm);
                 for (int i = tid; i < over; i += T) {
                     const uint64_t x = spill[i];
@@ -578,7 +578,7 @@ __global__ void __launch_bounds__(DIR_T, DIR_MINB) k_expand_direct(DirectArgs a)
         // the table is free (and zero) here: radix counters of the row sort
         finish_column<T, IPT, false>(top, ntop, topcap, a.pp, S, (unsigned long long)qv[2], fx.f, qv[0], b.cap[j],
                                      b.tmp_row + (obase - b.tmp_off0), b.tmp_val + (obase - b.tmp_off0),
-                                     hist, mhist, sh, ctr, lo, span, lo32, &mstar, &ch);
+                                     hist, mhist, hi32, sh, ctr, lo, span, lo32, &mstar, &ch);
         for (int i = tid; i < NW * 256; i += T) lo32[i] = 0u;
         if (tid == 0) {
             b.kept[j] = mstar;

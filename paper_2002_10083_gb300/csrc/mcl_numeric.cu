@@ -86,6 +86,7 @@ __global__ void __launch_bounds__(T, MINB) k_expand(ExpandArgs a) {
     constexpr int IPT = 8, NW = T / 32;
     static_assert(HS >= (T / 32) * 256, "the row sort's counters fit in the key array");
     static_assert(HS % (T * 4) == 0, "the scan takes four slots per thread");
+    static_assert(2 * HS >= SEL_BINS, "the selects' counters fit in the (empty) table");
     extern __shared__ __align__(16) unsigned char smem[];
     // sums' words and keys (row + 1, 0 = empty); idle lanes add 0 beyond the slots
     unsigned* lo32 = reinterpret_cast<unsigned*>(smem);
@@ -602,7 +603,7 @@ __global__ void __launch_bounds__(T, MINB) k_expand(ExpandArgs a) {
             if (tid == 0) es->cand = 0;
             if (have > topcap) {  // cut back to the ksel largest
                 const int over = have - topcap;
-                tau = block_select_count<T>(top, topcap, spill, over, ksel, hist, &sh->bs);
+                tau = block_select_wide<T>(top, topcap, spill, over, ksel, lo32, &sh->bs, sh->wsm);
                 ntop = compact_stable<T, IPT>(top, topcap, tau, sh->wsm);
                 for (int i = tid; i < over; i += T) {
                     const uint64_t x = spill[i];
@@ -643,8 +644,8 @@ __global__ void __launch_bounds__(T, MINB) k_expand(ExpandArgs a) {
         // the table's key array is free here: counters of the row sort
         finish_column<T, IPT, false>(top, ntop, topcap, a.pp, S, (unsigned long long)qv[2], fx.f, qv[0], b.cap[j],
                                      b.tmp_row + (obase - b.tmp_off0),
-                                     b.tmp_val + (obase - b.tmp_off0), hist, mhist, sh, ctr, lo,
-                                     span, reinterpret_cast<unsigned*>(keys), &mstar, &ch);
+                                     b.tmp_val + (obase - b.tmp_off0), hist, mhist, lo32, sh, ctr,
+                                     lo, span, reinterpret_cast<unsigned*>(keys), &mstar, &ch);
         for (int i = tid; i < (T / 32) * 256; i += T) keys[i] = 0;
         if (tid == 0) {
             b.kept[j] = mstar;
@@ -737,6 +738,7 @@ constexpr int PR_T = 256, PR_IPT = 8, PR_VC = PR_T * PR_IPT;
 struct PruneShared {
     WinShared w;
     int cnt[2][PR_IPT * PR_T / 32];  // candidates per round and warp, by chunk parity
+    unsigned bins[SEL_BINS];         // counters of the selects, zero between them
 };
 
 // The candidates and statistics of one column of m entries, in row order.
@@ -745,8 +747,7 @@ struct PruneShared {
 // of its candidates are counted (ballots per round and warp, in entry order).
 template <class Load>
 __device__ __forceinline__ void prune_candidates(int64_t m, const FixScale& fx, float theta, Load load,
-                                                 uint64_t* top, int topcap, int ksel, unsigned* hist,
-                                                 PruneShared* ps, int& ntop, long long& s_t,
+                                                 uint64_t* top, int topcap, int ksel, PruneShared* ps, int& ntop, long long& s_t,
                                                  unsigned long long& s_mt) {
     constexpr int NW = PR_T / 32;
     static_assert(PR_IPT * NW == 64, "two counts per lane");
@@ -792,7 +793,7 @@ __device__ __forceinline__ void prune_candidates(int64_t m, const FixScale& fx, 
         int at;
         int C = count(cnt, at);
         if (ntop + C > topcap) {  // C <= PR_VC = topcap - ksel, so ntop > ksel here
-            tau = block_select_count<PR_T>(top, ntop, top, 0, ksel, hist, &ps->w.bs);
+            tau = block_select_wide<PR_T>(top, ntop, top, 0, ksel, ps->bins, &ps->w.bs, ps->w.wsm);
             ntop = compact_stable<PR_T, PR_IPT>(top, ntop, tau, ps->w.wsm);
             C = count(cnt, at);
         }
@@ -838,6 +839,7 @@ __global__ void __launch_bounds__(PR_T, PR_MINB) k_prune(PruneArgs a) {
     WinShared* sh = &ps->w;
     const int tid = threadIdx.x;
     const ExpandBuffers& b = a.b;
+    for (int i = tid; i < SEL_BINS; i += PR_T) ps->bins[i] = 0u;
     for (;;) {
         if (tid == 0) sh->item = atomicAdd(&b.ctr->work_ctr, 1);
         __syncthreads();
@@ -866,7 +868,7 @@ __global__ void __launch_bounds__(PR_T, PR_MINB) k_prune(PruneArgs a) {
                     q = fx.qv(v);
                 }
             },
-            top, topcap, ksel, hist, ps, ntop, s_t, s_mt);
+            top, topcap, ksel, ps, ntop, s_t, s_mt);
         double dv[1] = {0.0};
         long long qv[2] = {s_t, (long long)s_mt};
         block_sum<PR_T>(dv, 0, qv, 2, &sh->bs);
@@ -875,7 +877,7 @@ __global__ void __launch_bounds__(PR_T, PR_MINB) k_prune(PruneArgs a) {
         const int64_t obase = b.off[j];
         finish_column<PR_T, 8, true>(top, ntop, topcap, a.pp, S, (unsigned long long)qv[1], fx.f, qv[0], b.cap[j],
                                      b.tmp_row + (obase - b.tmp_off0),
-                                     b.tmp_val + (obase - b.tmp_off0), hist, mhist, sh, b.ctr, 0,
+                                     b.tmp_val + (obase - b.tmp_off0), hist, mhist, ps->bins, sh, b.ctr, 0,
                                      0, nullptr, &mstar, &ch);
         if (tid == 0) {
             b.kept[j] = mstar;
