@@ -298,8 +298,8 @@ __global__ void __launch_bounds__(FWD_T) k_mlp_forward(const float* feats, int64
 // ---------------------------------------------------------------------------
 
 constexpr int BWD_B = 64;            // samples per CTA
-constexpr int BWD_TPS = 8;           // threads per sample (8 units each)
-constexpr int BWD_T = BWD_B * BWD_TPS;
+constexpr int BWD_TPS = 8;           // threads per pair of samples (8 units each)
+constexpr int BWD_T = BWD_B / 2 * BWD_TPS;
 
 struct BwdShared {
     MlpWeights m;
@@ -312,83 +312,127 @@ struct BwdShared {
     double red[BWD_T / 32];
 };
 
+// mlp_layer for two samples: every weight read serves both
+template <int TPS, int K, int STRIDE>
+__device__ __forceinline__ void mlp_layer2(const float* w, const float* b, const float* x0, const float* x1,
+                                           int e, float (&a0)[NH / TPS], float (&a1)[NH / TPS]) {
+#pragma unroll
+    for (int t = 0; t < NH / TPS; ++t) a0[t] = a1[t] = b[t * TPS + e];
+#pragma unroll 2
+    for (int i = 0; i < K; i += 4) {
+        const float4 u = *reinterpret_cast<const float4*>(x0 + i), v = *reinterpret_cast<const float4*>(x1 + i);
+#pragma unroll
+        for (int t = 0; t < NH / TPS; ++t) {
+            const float4 wv = *reinterpret_cast<const float4*>(w + (t * TPS + e) * STRIDE + i);
+            a0[t] = fmaf(wv.x, u.x, a0[t]);
+            a1[t] = fmaf(wv.x, v.x, a1[t]);
+            a0[t] = fmaf(wv.y, u.y, a0[t]);
+            a1[t] = fmaf(wv.y, v.y, a1[t]);
+            a0[t] = fmaf(wv.z, u.z, a0[t]);
+            a1[t] = fmaf(wv.z, v.z, a1[t]);
+            a0[t] = fmaf(wv.w, u.w, a0[t]);
+            a1[t] = fmaf(wv.w, v.w, a1[t]);
+        }
+    }
+}
+
 // Gradient of (scale * sum over samples and outputs of (y - t)^2) with
 // respect to the (BF16-valued) weights, added into grad; the loss sum
 // (unscaled) is added into *loss.
 //
-// Eight threads per sample for the two passes over the layers, then the CTA's
-// weight gradients as register tiles (8 of W2 per thread: six words read per
-// sample for 8 multiply-adds).  A thread per sample with its activations in
-// shared memory left two warps on an SM: latency-bound, 74 us at 8,192 samples.
+// Eight threads per pair of samples for the two passes over the layers (bound
+// by the shared-memory reads of the weights: one read serves both samples),
+// then the CTA's weight gradients as register tiles (16 of W2 per thread:
+// eight words read per sample for 16 multiply-adds).  A thread per sample with
+// its activations in shared memory left two warps on an SM: latency-bound,
+// 74 us at 8,192 samples; eight threads per sample took 29.
 __global__ void __launch_bounds__(BWD_T) k_mlp_backward(const float* feats, const float* targets,
                                                         int64_t n, const uint16_t* wbits,
                                                         const float* norm, float scale,
                                                         float* grad, double* loss) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     BwdShared& S = *reinterpret_cast<BwdShared*>(smem_raw);
-    const int tid = threadIdx.x, q = tid / BWD_TPS, e = tid % BWD_TPS;
+    const int tid = threadIdx.x, q = tid / BWD_TPS * 2, e = tid % BWD_TPS;
     load_weights(S.m, wbits, norm);
     __syncthreads();
     const int64_t s = (int64_t)blockIdx.x * BWD_B + q;
-    const bool v = s < n;
     constexpr int U = NH / BWD_TPS;
+    bool v[2];
 #pragma unroll
-    for (int i = 0; i < NIN; i += BWD_TPS)
-        S.Z[q][i + e] = v ? (feats[s * NIN + i + e] - S.m.mu[i + e]) * S.m.isg[i + e] : 0.0f;
+    for (int p = 0; p < 2; ++p) {
+        v[p] = s + p < n;
+#pragma unroll
+        for (int i = 0; i < NIN; i += BWD_TPS)
+            S.Z[q + p][i + e] =
+                v[p] ? (feats[(s + p) * NIN + i + e] - S.m.mu[i + e]) * S.m.isg[i + e] : 0.0f;
+    }
     __syncwarp();
-    float acc[U];
-    mlp_layer<BWD_TPS, NIN, NIN>(S.m.w1, S.m.b1, S.Z[q], e, acc);
+    float acc[2][U];
+    mlp_layer2<BWD_TPS, NIN, NIN>(S.m.w1, S.m.b1, S.Z[q], S.Z[q + 1], e, acc[0], acc[1]);
 #pragma unroll
-    for (int t = 0; t < U; ++t) S.H1[q][t * BWD_TPS + e] = v ? fmaxf(acc[t], 0.0f) : 0.0f;
+    for (int p = 0; p < 2; ++p)
+#pragma unroll
+        for (int t = 0; t < U; ++t) S.H1[q + p][t * BWD_TPS + e] = v[p] ? fmaxf(acc[p][t], 0.0f) : 0.0f;
     __syncwarp();
-    mlp_layer<BWD_TPS, NH, W2P>(S.m.w2, S.m.b2, S.H1[q], e, acc);
-    float y0 = 0.0f, y1 = 0.0f;
+    mlp_layer2<BWD_TPS, NH, W2P>(S.m.w2, S.m.b2, S.H1[q], S.H1[q + 1], e, acc[0], acc[1]);
+    double lsum = 0.0;
 #pragma unroll
-    for (int t = 0; t < U; ++t) {
-        const int o = t * BWD_TPS + e;
-        const float h2 = fmaxf(acc[t], 0.0f);
-        S.H2[q][o] = v ? h2 : 0.0f;
-        y0 = fmaf(S.m.w3[o], h2, y0);
-        y1 = fmaf(S.m.w3[NH + o], h2, y1);
-    }
+    for (int p = 0; p < 2; ++p) {
+        float y0 = 0.0f, y1 = 0.0f;
 #pragma unroll
-    for (int o = BWD_TPS / 2; o > 0; o >>= 1) {
-        y0 += __shfl_xor_sync(FULL, y0, o);
-        y1 += __shfl_xor_sync(FULL, y1, o);
-    }
-    y0 += S.m.b3[0];
-    y1 += S.m.b3[1];
-    const float e0 = v ? y0 - targets[s * 2] : 0.0f, e1 = v ? y1 - targets[s * 2 + 1] : 0.0f;
-    double lsum = e == 0 ? (double)e0 * e0 + (double)e1 * e1 : 0.0;
-    const float d0 = 2.0f * e0 * scale, d1 = 2.0f * e1 * scale;
-    if (e == 0) {
-        S.DY[q][0] = d0;
-        S.DY[q][1] = d1;
-    }
+        for (int t = 0; t < U; ++t) {
+            const int o = t * BWD_TPS + e;
+            const float h2 = fmaxf(acc[p][t], 0.0f);
+            S.H2[q + p][o] = v[p] ? h2 : 0.0f;
+            y0 = fmaf(S.m.w3[o], h2, y0);
+            y1 = fmaf(S.m.w3[NH + o], h2, y1);
+        }
 #pragma unroll
-    for (int t = 0; t < U; ++t) {
-        const int o = t * BWD_TPS + e;
-        S.D2[q][o] = acc[t] > 0.0f ? d0 * S.m.w3[o] + d1 * S.m.w3[NH + o] : 0.0f;
+        for (int o = BWD_TPS / 2; o > 0; o >>= 1) {
+            y0 += __shfl_xor_sync(FULL, y0, o);
+            y1 += __shfl_xor_sync(FULL, y1, o);
+        }
+        y0 += S.m.b3[0];
+        y1 += S.m.b3[1];
+        const float e0 = v[p] ? y0 - targets[(s + p) * 2] : 0.0f, e1 = v[p] ? y1 - targets[(s + p) * 2 + 1] : 0.0f;
+        if (e == 0) lsum += (double)e0 * e0 + (double)e1 * e1;
+        const float d0 = 2.0f * e0 * scale, d1 = 2.0f * e1 * scale;
+        if (e == 0) {
+            S.DY[q + p][0] = d0;
+            S.DY[q + p][1] = d1;
+        }
+#pragma unroll
+        for (int t = 0; t < U; ++t) {
+            const int o = t * BWD_TPS + e;
+            S.D2[q + p][o] = acc[p][t] > 0.0f ? d0 * S.m.w3[o] + d1 * S.m.w3[NH + o] : 0.0f;
+        }
     }
     __syncwarp();
     {  // D1 of units 8 e .. 8 e + 7
-        float g[U];
+        float g[2][U];
 #pragma unroll
-        for (int t = 0; t < U; ++t) g[t] = 0.0f;
+        for (int t = 0; t < U; ++t) g[0][t] = g[1][t] = 0.0f;
 #pragma unroll 4
         for (int o = 0; o < NH; ++o) {
-            const float dd = S.D2[q][o];
+            const float da = S.D2[q][o], db = S.D2[q + 1][o];
 #pragma unroll
             for (int t = 0; t < U; t += 4) {
                 const float4 wv = *reinterpret_cast<const float4*>(S.m.w2 + o * W2P + e * U + t);
-                g[t] = fmaf(dd, wv.x, g[t]);
-                g[t + 1] = fmaf(dd, wv.y, g[t + 1]);
-                g[t + 2] = fmaf(dd, wv.z, g[t + 2]);
-                g[t + 3] = fmaf(dd, wv.w, g[t + 3]);
+                g[0][t] = fmaf(da, wv.x, g[0][t]);
+                g[0][t + 1] = fmaf(da, wv.y, g[0][t + 1]);
+                g[0][t + 2] = fmaf(da, wv.z, g[0][t + 2]);
+                g[0][t + 3] = fmaf(da, wv.w, g[0][t + 3]);
+                g[1][t] = fmaf(db, wv.x, g[1][t]);
+                g[1][t + 1] = fmaf(db, wv.y, g[1][t + 1]);
+                g[1][t + 2] = fmaf(db, wv.z, g[1][t + 2]);
+                g[1][t + 3] = fmaf(db, wv.w, g[1][t + 3]);
             }
         }
 #pragma unroll
-        for (int t = 0; t < U; ++t) S.D1[q][e * U + t] = S.H1[q][e * U + t] > 0.0f ? g[t] : 0.0f;
+        for (int p = 0; p < 2; ++p)
+#pragma unroll
+            for (int t = 0; t < U; ++t)
+                S.D1[q + p][e * U + t] = S.H1[q + p][e * U + t] > 0.0f ? g[p][t] : 0.0f;
     }
     lsum = warp_sum(lsum);
     if ((tid & 31) == 0) S.red[tid >> 5] = lsum;
@@ -400,52 +444,54 @@ __global__ void __launch_bounds__(BWD_T) k_mlp_backward(const float* feats, cons
     }
     // weight gradients: sums over the CTA's samples
     {
-        const int o = tid / 16 * 2, i = tid % 16 * 4;  // W2: units o, o + 1, inputs i .. i + 3
-        float g[8] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
+        const int o = tid / 16 * 4, i = tid % 16 * 4;  // W2: units o .. o + 3, inputs i .. i + 3
+        float g[4][4] = {};
 #pragma unroll 4
         for (int b = 0; b < BWD_B; ++b) {
-            const float2 dv = *reinterpret_cast<const float2*>(&S.D2[b][o]);
+            const float4 dv = *reinterpret_cast<const float4*>(&S.D2[b][o]);
             const float4 hv = *reinterpret_cast<const float4*>(&S.H1[b][i]);
-            g[0] = fmaf(dv.x, hv.x, g[0]);
-            g[1] = fmaf(dv.x, hv.y, g[1]);
-            g[2] = fmaf(dv.x, hv.z, g[2]);
-            g[3] = fmaf(dv.x, hv.w, g[3]);
-            g[4] = fmaf(dv.y, hv.x, g[4]);
-            g[5] = fmaf(dv.y, hv.y, g[5]);
-            g[6] = fmaf(dv.y, hv.z, g[6]);
-            g[7] = fmaf(dv.y, hv.w, g[7]);
+            const float d4[4] = {dv.x, dv.y, dv.z, dv.w}, h4[4] = {hv.x, hv.y, hv.z, hv.w};
+#pragma unroll
+            for (int r = 0; r < 4; ++r)
+#pragma unroll
+                for (int c = 0; c < 4; ++c) g[r][c] = fmaf(d4[r], h4[c], g[r][c]);
         }
 #pragma unroll
-        for (int t = 0; t < 8; ++t) atomicAdd(grad + OFF_W2 + (o + t / 4) * NH + i + t % 4, g[t]);
+        for (int r = 0; r < 4; ++r)
+#pragma unroll
+            for (int c = 0; c < 4; ++c) atomicAdd(grad + OFF_W2 + (o + r) * NH + i + c, g[r][c]);
     }
     {
-        const int o = tid / 8, i = tid % 8 * 2;  // W1: unit o, inputs i, i + 1
-        float g0 = 0.0f, g1 = 0.0f;
+        const int o = tid / 4, i = tid % 4 * 4;  // W1: unit o, inputs i .. i + 3
+        float g[4] = {};
 #pragma unroll 4
         for (int b = 0; b < BWD_B; ++b) {
             const float dd = S.D1[b][o];
-            const float2 zv = *reinterpret_cast<const float2*>(&S.Z[b][i]);
-            g0 = fmaf(dd, zv.x, g0);
-            g1 = fmaf(dd, zv.y, g1);
+            const float4 zv = *reinterpret_cast<const float4*>(&S.Z[b][i]);
+            g[0] = fmaf(dd, zv.x, g[0]);
+            g[1] = fmaf(dd, zv.y, g[1]);
+            g[2] = fmaf(dd, zv.z, g[2]);
+            g[3] = fmaf(dd, zv.w, g[3]);
         }
-        atomicAdd(grad + OFF_W1 + o * NIN + i, g0);
-        atomicAdd(grad + OFF_W1 + o * NIN + i + 1, g1);
+#pragma unroll
+        for (int c = 0; c < 4; ++c) atomicAdd(grad + OFF_W1 + o * NIN + i + c, g[c]);
     }
-    if (tid < 2 * NH + NOUT * NH + NOUT) {  // b1, b2, W3, b3
+    static_assert(BWD_T == NH / 4 * (NH / 4) && BWD_T == NH * NIN / 4, "one tile per thread");
+    for (int k = tid; k < 2 * NH + NOUT * NH + NOUT; k += BWD_T) {  // b1, b2, W3, b3
         float g = 0.0f;
         int p;
-        if (tid < NH) {
-            p = OFF_B1 + tid;
-            for (int b = 0; b < BWD_B; ++b) g += S.D1[b][tid];
-        } else if (tid < 2 * NH) {
-            p = OFF_B2 + tid - NH;
-            for (int b = 0; b < BWD_B; ++b) g += S.D2[b][tid - NH];
-        } else if (tid < 2 * NH + NOUT * NH) {
-            const int o = (tid - 2 * NH) / NH, i = tid % NH;
+        if (k < NH) {
+            p = OFF_B1 + k;
+            for (int b = 0; b < BWD_B; ++b) g += S.D1[b][k];
+        } else if (k < 2 * NH) {
+            p = OFF_B2 + k - NH;
+            for (int b = 0; b < BWD_B; ++b) g += S.D2[b][k - NH];
+        } else if (k < 2 * NH + NOUT * NH) {
+            const int o = (k - 2 * NH) / NH, i = k % NH;
             p = OFF_W3 + o * NH + i;
             for (int b = 0; b < BWD_B; ++b) g = fmaf(S.DY[b][o], S.H2[b][i], g);
         } else {
-            const int o = tid - 2 * NH - NOUT * NH;
+            const int o = k - 2 * NH - NOUT * NH;
             p = OFF_B3 + o;
             for (int b = 0; b < BWD_B; ++b) g += S.DY[b][o];
         }
