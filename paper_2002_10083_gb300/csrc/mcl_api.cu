@@ -728,7 +728,7 @@ mcl_status mcl_expand_split(mcl_ctx* c, const mcl_csc* A, const mcl_params* prm,
     int64_t stride = (int64_t)c->hctr->max_deg;
     if (stride < MCL_SPLIT_MAX_PARTS) stride = MCL_SPLIT_MAX_PARTS;
     stride = (stride + 31) & ~31ll;
-    const int grid_cap = 4 * c->num_sms;
+    const int grid_cap = split_grid_cap(n, c->num_sms);
     const size_t n1 = (size_t)n + 1;
     if (!ensure(c, c->split_cnt, n1 * 8, s) ||
         !ensure(c, c->split_scratch, (size_t)grid_cap * 6 * stride * 8, s))

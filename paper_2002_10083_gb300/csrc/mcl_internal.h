@@ -190,6 +190,7 @@ struct RankArgs {
     unsigned long long* val_out;  // fill mode
     DevCounters* ctr;
 };
+int split_grid_cap(int64_t n, int num_sms);  // CTAs that the scratch serves at most
 void launch_bsum(const CscView& A, const double* colsum, double* bsum, cudaStream_t s);
 void launch_split_count(const RankArgs& a, bool stage, int num_sms, cudaStream_t s);
 void launch_split_fill(const RankArgs& a, bool stage, int num_sms, cudaStream_t s);

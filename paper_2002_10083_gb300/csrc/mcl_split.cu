@@ -57,26 +57,27 @@ void launch_bsum(const CscView& A, const double* colsum, double* bsum, cudaStrea
     count_launches(1);
 }
 
-constexpr int RA_T = 512;
 constexpr int RA_UNIT = 128;   // entries a warp takes at once
-constexpr int RA_BATCH = 512;  // sources whose units are listed at once
-// Shapes by the rows of the output: bitmap words (32 rows each) and sums.  Up
-// to 131k rows are one window and two CTAs share an SM.
-template <int WORDS_, int CAP_, int MINB_>
+// Shapes by the rows of the output: threads, bitmap words (32 rows each), sums,
+// CTAs per SM.  A column's steps are short and separated by barriers, so small
+// outputs take many small CTAs.
+template <int T_, int WORDS_, int CAP_, int MINB_>
 struct RankShape {
-    static constexpr int WORDS = WORDS_, CAP = CAP_, MINB = MINB_;
+    static constexpr int T = T_, WORDS = WORDS_, CAP = CAP_, MINB = MINB_;
 };
-using RankSmall = RankShape<4096, 8192, 2>;
-using RankLarge = RankShape<16384, 8192, 1>;
+using RankTiny = RankShape<256, 1024, 4096, 5>;
+using RankSmall = RankShape<512, 4096, 8192, 2>;
+using RankLarge = RankShape<512, 16384, 8192, 1>;
 // More passes than this over a window's sources: add in global memory instead.
-constexpr int RA_PASSES = 4;
+constexpr int RA_PASSES = 8;
 
+template <int T>
 struct RankShared {
     BlockScratch bs;
     int wsm[34];
     int item;
     int lo, hi;               // row span of the column's sources
-    int upre[RA_BATCH + 1];   // first unit of each source of a batch
+    int upre[T + 1];          // first unit of each source of a batch of T
 };
 
 // Sources of one output column, per CTA in global scratch (stride entries):
@@ -92,6 +93,7 @@ struct RankScratch {
 };
 
 // Exclusive block scan of x; the total to all threads.  Ends with a barrier.
+template <int T>
 __device__ __forceinline__ int ra_scan(int x, int* total, int* wsm) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     int incl = x;
@@ -103,14 +105,14 @@ __device__ __forceinline__ int ra_scan(int x, int* total, int* wsm) {
     if (lane == 31) wsm[warp] = incl;
     __syncthreads();
     if (warp == 0) {
-        const int w0 = lane < RA_T / 32 ? wsm[lane] : 0;
+        const int w0 = lane < T / 32 ? wsm[lane] : 0;
         int wi = w0;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
             const int y = __shfl_up_sync(FULL, wi, o);
             if (lane >= o) wi += y;
         }
-        if (lane < RA_T / 32) wsm[lane] = wi - w0;
+        if (lane < T / 32) wsm[lane] = wi - w0;
         if (lane == 31) wsm[32] = wi;
     }
     __syncthreads();
@@ -124,14 +126,15 @@ __device__ __forceinline__ int ra_scan(int x, int* total, int* wsm) {
 // otherwise the columns j of the partial products.  FILL: write the output
 // (else count it).
 template <bool STAGE, bool FILL, class SH>
-__global__ void __launch_bounds__(RA_T, SH::MINB) k_rank_acc(RankArgs a) {
+__global__ void __launch_bounds__(SH::T, SH::MINB) k_rank_acc(RankArgs a) {
     extern __shared__ __align__(16) unsigned char smem[];
+    constexpr int RA_T = SH::T;
     constexpr int WORDS = SH::WORDS, CAP = SH::CAP, WB = WORDS * 32;
     uint32_t* bm = reinterpret_cast<uint32_t*>(smem);
     int32_t* wpre = reinterpret_cast<int32_t*>(bm + WORDS);  // from here FILL only, up to sh
     unsigned* lo32 = reinterpret_cast<unsigned*>(wpre + WORDS);
     unsigned* hi32 = lo32 + CAP;
-    RankShared* sh = reinterpret_cast<RankShared*>(FILL ? reinterpret_cast<unsigned char*>(hi32 + CAP)
+    RankShared<RA_T>* sh = reinterpret_cast<RankShared<RA_T>*>(FILL ? reinterpret_cast<unsigned char*>(hi32 + CAP)
                                                         : reinterpret_cast<unsigned char*>(bm + WORDS));
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     constexpr int NWP = RA_T / 32;
@@ -243,15 +246,13 @@ __global__ void __launch_bounds__(RA_T, SH::MINB) k_rank_acc(RankArgs a) {
             __syncthreads();
             // f(s, p0, end) for every unit [p0, p0 + RA_UNIT) of the sources' entries
             auto each_unit = [&](auto f) {
-                for (int b0 = 0; b0 < ns; b0 += RA_BATCH) {
-                    const int m = min(RA_BATCH, ns - b0);
-                    if (RA_T >= RA_BATCH) {
-                        const int u = tid < m ? (rs.nxt[b0 + tid] - rs.cur[b0 + tid] + RA_UNIT - 1) / RA_UNIT : 0;
-                        int tot;
-                        const int at = ra_scan(u, &tot, sh->wsm);
-                        if (tid < m) sh->upre[tid] = at;
-                        if (tid == 0) sh->upre[m] = tot;
-                    }
+                for (int b0 = 0; b0 < ns; b0 += RA_T) {
+                    const int m = min(RA_T, ns - b0);
+                    const int u = tid < m ? (rs.nxt[b0 + tid] - rs.cur[b0 + tid] + RA_UNIT - 1) / RA_UNIT : 0;
+                    int tot;
+                    const int at = ra_scan<RA_T>(u, &tot, sh->wsm);
+                    if (tid < m) sh->upre[tid] = at;
+                    if (tid == 0) sh->upre[m] = tot;
                     __syncthreads();
                     const int units = sh->upre[m];
                     int s = 0;
@@ -285,7 +286,7 @@ __global__ void __launch_bounds__(RA_T, SH::MINB) k_rank_acc(RankArgs a) {
                 for (int w0 = 0; w0 < nwords; w0 += RA_T) {
                     const int w = w0 + tid;
                     int tot;
-                    const int at = ra_scan(w < nwords ? __popc(bm[w]) : 0, &tot, sh->wsm);
+                    const int at = ra_scan<RA_T>(w < nwords ? __popc(bm[w]) : 0, &tot, sh->wsm);
                     if (w < nwords) wpre[w] = wtot + at;
                     wtot += tot;
                 }
@@ -364,17 +365,17 @@ __global__ void __launch_bounds__(RA_T, SH::MINB) k_rank_acc(RankArgs a) {
 
 template <bool STAGE, bool FILL, class SH>
 static void rank_launch(const RankArgs& a, int num_sms, cudaStream_t s) {
-    const size_t smem = (size_t)SH::WORDS * 4 * (FILL ? 2 : 1) + (FILL ? (size_t)SH::CAP * 8 : 0) + sizeof(RankShared);
+    const size_t smem = (size_t)SH::WORDS * 4 * (FILL ? 2 : 1) + (FILL ? (size_t)SH::CAP * 8 : 0) + sizeof(RankShared<SH::T>);
     auto kern = k_rank_acc<STAGE, FILL, SH>;
     cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     int occ = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, RA_T, smem);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, SH::T, smem);
     if (occ < 1) occ = 1;
     int grid = occ * num_sms;
     if (grid > a.grid_cap) grid = a.grid_cap;
     if ((int64_t)grid > a.n) grid = a.n > 0 ? (int)a.n : 1;
     cudaMemsetAsync(&a.ctr->work_ctr, 0, sizeof(int), s);
-    kern<<<grid, RA_T, smem, s>>>(a);
+    kern<<<grid, SH::T, smem, s>>>(a);
     count_launches(1);
 }
 
@@ -388,10 +389,16 @@ static void rank_any(const RankArgs& a, bool stage, bool fill, int num_sms, cuda
 
 static void rank_shape(const RankArgs& a, bool stage, bool fill, int num_sms, cudaStream_t s) {
     if (a.n == 0) return;
-    if (a.n <= RankSmall::WORDS * 32)
+    if (a.n <= RankTiny::WORDS * 32)
+        rank_any<RankTiny>(a, stage, fill, num_sms, s);
+    else if (a.n <= RankSmall::WORDS * 32)
         rank_any<RankSmall>(a, stage, fill, num_sms, s);
     else
         rank_any<RankLarge>(a, stage, fill, num_sms, s);
+}
+
+int split_grid_cap(int64_t n, int num_sms) {
+    return num_sms * (n <= RankTiny::WORDS * 32 ? RankTiny::MINB : 4);
 }
 
 void launch_split_count(const RankArgs& a, bool stage, int num_sms, cudaStream_t s) {

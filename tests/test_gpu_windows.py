@@ -80,9 +80,9 @@ def test_direct_windows_equal_hashed_ones(ctx, n, d, K, theta, zeros, budget):
     assert torch.equal(out.val.view(torch.int32), ref.val.view(torch.int32))
 
 
-# several passes of sums per window, 64-bit global atomics (more than four passes), the large
-# bitmap, several bitmap windows; merges of 2 to 4 and a last merge of leftovers
-@pytest.mark.parametrize("n,d,ns", [(12000, 130, 4), (45000, 250, 2), (140000, 20, 3), (600000, 5, 2), (33, 5, 7)])
+# several passes of sums per window, 64-bit global atomics (more than eight passes: 80k entries),
+# the edges of the bitmaps, several bitmap windows; merges of 2 to 4 and a last merge of leftovers
+@pytest.mark.parametrize("n,d,ns", [(12000, 130, 4), (32768, 300, 2), (32769, 20, 2), (45000, 250, 2), (100000, 400, 2), (140000, 20, 3), (600000, 5, 2), (33, 5, 7)])
 def test_split_shapes_equal_one_pass(ctx, n, d, ns):
     from paper_2002_10083_gb300 import mcl
     A = _random(n, d, seed=n, zeros=n < 20000)
