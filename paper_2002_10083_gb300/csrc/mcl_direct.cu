@@ -27,9 +27,9 @@
 //
 // Bound by the instructions of the insert (78% of issue slots when it took
 // about 95 per product; 8% of DRAM peak).  Iteration 2 of the 40k-vertex
-// power-law graph (4.4e10 products): 240 ms with mcl_numeric.cu, 99 ms here;
-// iteration 2 of 16 planted partitions of up to 50k vertices (4.8e10): 401 ms
-// and 130 ms.
+// power-law graph (4.4e10 products): 240 ms with the hashed windows that
+// mcl_numeric.cu then had, 95 ms here; iteration 2 of 16 planted partitions of
+// up to 50k vertices (4.8e10): 401 ms and 121 ms.
 #include <cfloat>
 #include <climits>
 #include <cstdint>

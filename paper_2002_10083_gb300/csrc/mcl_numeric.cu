@@ -34,6 +34,16 @@
 // published by one thread, a block scan for the candidates' positions and
 // separate passes for extraction, emission and clearing there were ten.)
 //
+// Bound by instruction issue and the latency of the probes: 55% of issue
+// slots busy at 32 warps per SM (64 registers), DRAM at 6%; about 2.3 clocks
+// of an SM per hashed product.  First iteration of the 1M-vertex power-law
+// graph, columns that are not dense in their span: 448 ms before the two
+// barriers, the FP64-free column end and the wide selects, 394 ms with them.
+// Not faster: the four probe chains of a lane advanced together (583 ms the
+// iteration against 524), windows of 5,120 slots in 512-thread CTAs (696
+// against 606), windows planned for 896 or 1,280 entries (501 and 494 against
+// 492).
+//
 // Windows come from per-window product buckets (a counting pass and a
 // scatter of (row, FP32 product) into window order); a column that is one
 // small window from its sources, product by product; without bucket space
