@@ -542,16 +542,17 @@ __global__ void __launch_bounds__(T, MINB) k_expand(ExpandArgs a) {
             }
             __syncthreads();
             if (es->full) {  // split: a quarter of the rows at once from here on
+                __syncthreads();  // every thread has read the flag
                 for (int i = tid; i < HS; i += T) {
                     lo32[i] = 0u;
                     hi32[i] = 0u;
                     keys[i] = 0;
                 }
-                __syncthreads();
                 if (tid == 0) {
-                    es->full = 0;
+                    es->full = 0;  // before the barrier: the redone window may set it again
                     atomicAdd(&ctr->splits, 1ull);
                 }
+                __syncthreads();
                 pw = max(1, (r1 - r0) / 4);
                 r1 = r0 + pw;
                 continue;

@@ -171,3 +171,38 @@ def test_small_plan_sizes(ctx, n):
     assert ch == ch_ref and torch.equal(out.colptr, ref.colptr) and torch.equal(out.rowidx, ref.rowidx)
     assert torch.equal(out.val.view(torch.int32), ref.val.view(torch.int32))
     assert all(st[k] == ctx.stats()[k] for k in ("flops", "nnz_b", "nnz_out", "estimator_misses"))
+
+
+@pytest.fixture(scope="module")
+def sparse_spans(ctx):
+    """Columns of about 27,000 products in spans of 160,000 rows: too sparse for a sum per row,
+    17 windows or more in every table of the large configuration.  With the exact iteration."""
+    from paper_2002_10083_gb300 import mcl
+    A = _random(160_000, 140, seed=17)
+    flops, _ = ctx.symbolic(A)
+    assert int(flops.max()) * 4 < 0.95 * A.n
+    prm = mcl.Params(threshold=1e-5, select_k=300, recover_pct=0.9, inflation=2.0)
+    return A, prm, ctx.expand(A, prm), ctx.stats()["nnz_b"]
+
+
+# estimates that are right, short, and so short that a window's redone quarter overflows too
+@pytest.mark.parametrize("scale", [1000, 100, 10])
+@pytest.mark.parametrize("table,plan", [(0, 0), (0, 300), (1, 0), (1, 3000), (2, 0), (2, 1024)])
+def test_table_shapes_and_overflowing_windows(ctx, sparse_spans, table, plan, scale):
+    from paper_2002_10083_gb300 import mcl
+    A, prm, (ref, ch_ref), nnz_b = sparse_spans
+    opts = {mcl.OPT_CONF_MASK: (2, 3), mcl.OPT_TABLE: (table, 0), mcl.OPT_PLAN: (plan, 0),
+            mcl.OPT_EST_SCALE: (scale, 1000)}
+    try:
+        for o, (v, _) in opts.items():
+            ctx.set_option(o, v)
+        for _ in range(5):
+            out, ch = ctx.expand(A, prm)
+            st = ctx.stats()
+            assert st["nnz_b"] == nnz_b and ch == ch_ref
+            assert scale == 1000 or st["range_splits"] > A.n * (0.5 if scale == 100 else 1.5)
+            assert torch.equal(out.colptr, ref.colptr) and torch.equal(out.rowidx, ref.rowidx)
+            assert torch.equal(out.val.view(torch.int32), ref.val.view(torch.int32))
+    finally:
+        for o, (_, v) in opts.items():
+            ctx.set_option(o, v)
