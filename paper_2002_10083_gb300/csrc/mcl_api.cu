@@ -265,6 +265,12 @@ ExpandBuffers with_buckets(mcl_ctx* c, const ExpandBuffers& b, int q, int g, siz
     return bq;
 }
 
+// Whether columns of configuration q may be many windows without product
+// buckets (the small configuration alone, or columns of up to max_flops products).
+bool walks_sources(const mcl_ctx* c, const ExpandBuffers& bq, int q, int64_t max_flops) {
+    return q == 0 ? !conf_on(c, CONF_LARGE) : bq.bucket_cap < max_flops;
+}
+
 }  // namespace
 
 // Learned estimate: features -> MLP -> b.est (needs colstats done).
@@ -509,8 +515,11 @@ static mcl_status expand_impl(mcl_ctx* c, const mcl_csc* A, const mcl_params* pr
             // the host has a small plan's column counts; none binned: no launch
             int cols = small ? c->hctr->bin_off[(q + 1) * NZ] - c->hctr->bin_off[q * NZ] : g;
             if (q == CONF_DIRECT && c->hctr->max_span <= DIRECT_MIN_SPAN) cols = 0;
-            if (cols > 0)
-                launch_numeric(q, Av, pp, with_buckets(c, bb, q, g, bkt_bytes), cols < g ? cols : g, s);
+            if (cols > 0) {
+                const ExpandBuffers bq = with_buckets(c, bb, q, g, bkt_bytes);
+                launch_numeric(q, Av, pp, bq, cols < g ? cols : g,
+                               walks_sources(c, bq, q, (int64_t)c->hctr->max_flops), s);
+            }
             ++used;
         }
         return check_launch(c, "numeric");
@@ -1224,7 +1233,8 @@ static void static_iteration(mcl_ctx* c, const mcl_params* prm, const PruneParam
     for (int q = NCONF - 1; q >= 0; --q) {
         if (!conf_on(c, q) || (q == CONF_DIRECT && max_comp <= DIRECT_MIN_SPAN)) continue;
         const int g = numeric_grid(q, pp, c->num_sms);
-        launch_numeric(q, Av, pp, with_buckets(c, b, q, g, c->bucket_row.p ? c->bucket_row.bytes : 0), g, s);
+        const ExpandBuffers bq = with_buckets(c, b, q, g, c->bucket_row.p ? c->bucket_row.bytes : 0);
+        launch_numeric(q, Av, pp, bq, g, walks_sources(c, bq, q, (int64_t)pp.Krec * pp.Krec), s);
     }
     if (small) {
         launch_result_small(Av, b, out.colptr, nullptr, s);

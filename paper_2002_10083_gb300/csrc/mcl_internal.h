@@ -136,8 +136,9 @@ int direct_grid(int ksel, int num_sms);
 size_t direct_spill_bytes(int grid);
 void launch_direct(const CscView& A, const PruneParams& pp, const ExpandBuffers& b, int grid,
                    cudaStream_t s);
+// walk: columns of many windows may have no product buckets
 void launch_numeric(int conf, const CscView& A, const PruneParams& pp, const ExpandBuffers& b,
-                    int grid, cudaStream_t s);
+                    int grid, bool walk, cudaStream_t s);
 void launch_compact(const CscView& A, const ExpandBuffers& b, const int64_t* colptr_out,
                     int32_t* row_out, float* val_out, cudaStream_t s);
 void launch_finalize_stats(int32_t n, const ExpandBuffers& b, cudaStream_t s);

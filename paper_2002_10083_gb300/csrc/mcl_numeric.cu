@@ -47,7 +47,7 @@
 // Windows come from per-window product buckets (a counting pass and a
 // scatter of (row, FP32 product) into window order); a column that is one
 // small window from its sources, product by product; without bucket space
-// from per-source cursors over the sorted rows.  A hashed window whose
+// from per-source cursors over the sorted rows (a warp or a lane per source).  A hashed window whose
 // probe runs exceed PMAX slots is split by rows and redone (counted as a
 // split), and the rest of the column starts at the width that fitted;
 // results never depend on the size estimate.  Finally the prune rule picks
@@ -63,6 +63,14 @@
 namespace mcl {
 
 constexpr int PMAX = 64;          // probe run that marks a hashed window as overflowed
+// Products per source and window below which the walk over the sources gives
+// each lane a source, and 4 of its products a round, instead of each warp one and
+// 128.  Power-law graphs through the small configuration alone, 20k, 200k and
+// 600k vertices: 26, 420 and 1,007 ms without lanes; 16.1, 131 and 340 ms with
+// the line at 12; 11.6, 134 and 347 at 16; 10.6, 138 and 356 at 20.  Only for
+// launches where columns can be many windows without buckets (WALK): its
+// registers cost the others 1% (1M vertices: 505 -> 511 ms).
+constexpr int LANE_MAX = 16;
 constexpr int FLAT_SOURCES = 256; // a column of so few sources and products in one window:
 constexpr int FLAT_PRODUCTS = 65536;  // every lane finds its own products' sources
 
@@ -90,7 +98,7 @@ struct ExpandLayout {
     }
 };
 
-template <int T, int HS, int MINB>
+template <int T, int HS, int MINB, bool WALK>
 __global__ void __launch_bounds__(T, MINB) k_expand(ExpandArgs a) {
     const int PLAN = a.plan;  // distinct rows a window is planned for
     constexpr int IPT = 8, NW = T / 32;
@@ -445,6 +453,8 @@ __global__ void __launch_bounds__(T, MINB) k_expand(ExpandArgs a) {
         int32_t* cur = meta.cur;
         int32_t* nxt = meta.nxt;
         const int batch = max(1, min(32, d / (4 * NW)));  // sources a warp takes at once
+        const bool lanes = WALK && !bucket &&
+                           (float)flops_j * (float)width < (float)LANE_MAX * (float)d * (float)span;
         int w = 0, pw = width;
         int we = bucket ? (int)min((int64_t)lo + width, (int64_t)hiE) : hiE;
         int r0 = lo, r1 = (int)min((int64_t)r0 + pw, (int64_t)we);
@@ -505,14 +515,18 @@ __global__ void __launch_bounds__(T, MINB) k_expand(ExpandArgs a) {
                     add4(h, v, wr, r0, hash);
                 }
             } else {
+                // a warp per source and 128 of its products a round; with few products per
+                // source and window a lane per source and four
                 int* next = &es->next[it & 1];
+                const int take = lanes ? 32 : batch;
+                const int step = lanes ? 1 : 32;
                 for (;;) {
                     int k0 = 0;
-                    if (lane == 0) k0 = atomicAdd(next, batch);
+                    if (lane == 0) k0 = atomicAdd(next, take);
                     k0 = __shfl_sync(FULL, k0, 0);
                     if (k0 >= d) break;
-                    const int nb = min(batch, d - k0);
-                    for (int s = k0; s < k0 + nb; ++s) {
+                    const int k1 = min(k0 + take, d);
+                    for (int s = lanes ? k0 + lane : k0; s < k1; s += lanes ? 32 : 1) {
                         const int len = meta.len[s];
                         const int64_t ks = meta.ks[s];
                         const float akj = meta.akj[s];
@@ -522,7 +536,7 @@ __global__ void __launch_bounds__(T, MINB) k_expand(ExpandArgs a) {
                             float v[4];
 #pragma unroll
                             for (int c = 0; c < 4; ++c) {
-                                const int p = pos + 32 * c + lane;
+                                const int p = pos + step * c + (lanes ? 0 : lane);
                                 h[c] = (unsigned)((p < len ? __ldg(A.rowidx + ks + p) : INT_MAX) - r0);
                                 v[c] = p < len ? __ldg(A.val + ks + p) : 0.0f;
                             }
@@ -530,13 +544,13 @@ __global__ void __launch_bounds__(T, MINB) k_expand(ExpandArgs a) {
 #pragma unroll
                             for (int c = 0; c < 4; ++c) {
                                 v[c] = __fmul_rn(v[c], akj);
-                                nin += __popc(__ballot_sync(FULL, h[c] < wr));
+                                nin += lanes ? (int)(h[c] < wr) : __popc(__ballot_sync(FULL, h[c] < wr));
                             }
                             add4(h, v, wr, r0, hash);
                             pos += nin;
-                            if (nin < 128) break;
+                            if (nin < 4 * step) break;
                         }
-                        if (lane == 0) nxt[s] = pos;
+                        if (lanes || lane == 0) nxt[s] = pos;
                     }
                 }
             }
@@ -687,7 +701,7 @@ static size_t conf_smem(int ksel) { return ExpandLayout<C::T, C::HS>::bytes(ksel
 template <class C>
 static int conf_grid(int ksel, int num_sms) {
     const size_t smem = conf_smem<C>(ksel);
-    auto kern = k_expand<C::T, C::HS, C::MINB>;
+    auto kern = k_expand<C::T, C::HS, C::MINB, false>;
     cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     int occ = 0;
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, C::T, smem);
@@ -697,12 +711,15 @@ static int conf_grid(int ksel, int num_sms) {
 
 template <class C>
 static void conf_launch(int conf, const CscView& A, const PruneParams& pp, const ExpandBuffers& b,
-                        int grid, cudaStream_t s) {
+                        int grid, bool walk, cudaStream_t s) {
     int plan = conf == 0 ? C::HS / 2 : (pp.plan > 0 ? pp.plan : C::HS / 2);
     if (plan > (3 * C::HS) / 4) plan = (3 * C::HS) / 4;
     if (plan < 64) plan = 64;
     ExpandArgs a{A, pp, b, conf, plan};
-    k_expand<C::T, C::HS, C::MINB><<<grid, C::T, conf_smem<C>(pp.ksel), s>>>(a);
+    const size_t smem = conf_smem<C>(pp.ksel);
+    auto kern = walk ? k_expand<C::T, C::HS, C::MINB, true> : k_expand<C::T, C::HS, C::MINB, false>;
+    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    kern<<<grid, C::T, smem, s>>>(a);
 }
 
 // Bytes of candidate spill: a window's slots for every CTA of the largest configuration.
@@ -724,17 +741,17 @@ int numeric_grid(int conf, const PruneParams& pp, int num_sms) {
 }
 
 void launch_numeric(int conf, const CscView& A, const PruneParams& pp, const ExpandBuffers& b,
-                    int grid, cudaStream_t s) {
+                    int grid, bool walk, cudaStream_t s) {
     if (conf == CONF_DIRECT)
         launch_direct(A, pp, b, grid, s);
     else if (conf == 0)
-        conf_launch<Conf0>(conf, A, pp, b, grid, s);
+        conf_launch<Conf0>(conf, A, pp, b, grid, walk, s);
     else if (pp.table == 1)
-        conf_launch<Conf1b>(conf, A, pp, b, grid, s);
+        conf_launch<Conf1b>(conf, A, pp, b, grid, walk, s);
     else if (pp.table == 2)
-        conf_launch<Conf1c>(conf, A, pp, b, grid, s);
+        conf_launch<Conf1c>(conf, A, pp, b, grid, walk, s);
     else
-        conf_launch<Conf1a>(conf, A, pp, b, grid, s);
+        conf_launch<Conf1a>(conf, A, pp, b, grid, walk, s);
     count_launches(1);
 }
 

@@ -206,3 +206,27 @@ def test_table_shapes_and_overflowing_windows(ctx, sparse_spans, table, plan, sc
     finally:
         for o, (_, v) in opts.items():
             ctx.set_option(o, v)
+
+
+# columns of many windows without product buckets: no bucket space, space for some columns only
+# (8 MB: about 1,700 products each), the small configuration alone; estimates right and short
+@pytest.mark.parametrize("budget,mask,scale", [(0, 3, 1000), (0, 3, 50), (8 << 20, 3, 1000), (8 << 20, 2, 30),
+                                               (32 << 30, 1, 1000), (0, 1, 20)])
+@pytest.mark.parametrize("n,d", [(300, 3), (9000, 2), (40000, 30), (60000, 41), (90000, 130)])
+def test_walked_sources_equal_buckets(ctx, n, d, budget, mask, scale):
+    from paper_2002_10083_gb300 import mcl
+    A = _random(n, d, seed=n + 3 * d, zeros=d == 41)
+    prm = mcl.Params(threshold=1e-4, select_k=150, recover_pct=0.9, inflation=2.0)
+    ref, ch_ref = ctx.expand(A, prm)
+    nnz_b = ctx.stats()["nnz_b"]
+    opts = {mcl.OPT_BUCKET_BUDGET: (budget, 32 << 30), mcl.OPT_CONF_MASK: (mask, 3), mcl.OPT_EST_SCALE: (scale, 1000)}
+    try:
+        for o, (v, _) in opts.items():
+            ctx.set_option(o, v)
+        out, ch = ctx.expand(A, prm)
+        assert ctx.stats()["nnz_b"] == nnz_b
+    finally:
+        for o, (_, v) in opts.items():
+            ctx.set_option(o, v)
+    assert ch == ch_ref and torch.equal(out.colptr, ref.colptr) and torch.equal(out.rowidx, ref.rowidx)
+    assert torch.equal(out.val.view(torch.int32), ref.val.view(torch.int32))
