@@ -19,6 +19,7 @@
 #include <cfloat>
 #include <climits>
 #include <cstdint>
+#include <type_traits>
 
 #include "mcl_device.cuh"
 #include "mcl_internal.h"
@@ -282,10 +283,20 @@ template void launch_exclusive_scan<int32_t>(const int32_t*, int64_t, int64_t*, 
 // and clears it.  The sources are cut into units of 128 rows that the warps
 // take in turn, all four loads of a lane first: a warp per source left most
 // warps idle behind the longest one, with one load in flight each.  300k
-// vertices, 1.1e10 products: 30.1 -> 10.1 ms, 0.27 clocks of an SM per product
+// vertices, 1.1e10 products: 30.1 -> 10.2 ms, 0.27 clocks of an SM per product
 // (a shared atomic's rate at random words is 0.09, its instructions 0.12).
 constexpr int SYM_WORDS = 16384;  // 64 KB bitmap -> 524,288 rows per window
 constexpr int SYM_UNIT = 128;
+// Listed products per row of the window from which a bit is read before it is
+// set: most are set already, and the lanes that share a word do not wait for each
+// other.  20 components of 2,000 vertices, 60% dense: 124 ms without the read,
+// 41.7 with it (77 with a warp per source); 8k vertices of 1,100 entries: 4.6 ms
+// with the line at 64, 3.7 at 16.
+constexpr int SYM_TEST = 16;
+// Graphs of so few vertices have one short bitmap: CTAs of 256 threads, twice as
+// many, beat 512 where columns are short (16k vertices, 50 and 300 entries a
+// column: 0.58 and 1.20 ms, with 512 threads 0.58 and 1.38, with 128 0.72 and 1.15).
+constexpr int SYM_SMALL_N = 16384;
 constexpr int SYM_BATCH = 512;    // sources whose units are listed at once
 
 struct SymShared {
@@ -328,6 +339,11 @@ __global__ void __launch_bounds__(T) k_symbolic(CscView A, ExpandBuffers b, int6
             continue;
         }
         long long cnt = 0;
+        // a thread lists the same sources in every window, if they are one batch (the small
+        // CTAs have one window)
+        const bool once = T == 512 && d <= SYM_BATCH;
+        int64_t ks[PER];
+        int len[PER], next[PER];
         for (int r0 = lo; r0 < hiE;) {
             const int r1 = (int)min((int64_t)r0 + WB, (int64_t)hiE);
             for (int b0 = 0; b0 < d; b0 += SYM_BATCH) {
@@ -338,22 +354,27 @@ __global__ void __launch_bounds__(T) k_symbolic(CscView A, ExpandBuffers b, int6
                     const int i = tid * PER + q;
                     u[q] = 0;
                     if (i < m) {
-                        const int k = __ldg(A.rowidx + cb + b0 + i);
-                        const int64_t ks = __ldg(A.colptr + k);
-                        const int len = (int)(__ldg(A.colptr + k + 1) - ks);
-                        int c0 = 0, c1 = len;
+                        if (!once || r0 == lo) {
+                            const int k = __ldg(A.rowidx + cb + b0 + i);
+                            ks[q] = __ldg(A.colptr + k);
+                            len[q] = (int)(__ldg(A.colptr + k + 1) - ks[q]);
+                        }
+                        int c0 = 0, c1 = len[q];
                         if (windows) {  // the source's rows in [r0, r1): [c0, c1)
-                            c0 = r0 == lo ? 0 : cur[b0 + i];
+                            c0 = r0 == lo ? 0 : once ? next[q] : cur[b0 + i];
                             if (r1 < hiE) {
                                 int x = c0;
                                 while (x < c1) {
                                     const int mid = (x + c1) >> 1;
-                                    if (__ldg(A.rowidx + ks + mid) < r1) x = mid + 1; else c1 = mid;
+                                    if (__ldg(A.rowidx + ks[q] + mid) < r1) x = mid + 1; else c1 = mid;
                                 }
                             }
-                            cur[b0 + i] = c1;
+                            if (once)
+                                next[q] = c1;
+                            else
+                                cur[b0 + i] = c1;
                         }
-                        sh->first[i] = ks + c0;
+                        sh->first[i] = ks[q] + c0;
                         sh->cnt[i] = c1 - c0;
                         u[q] = (c1 - c0 + SYM_UNIT - 1) / SYM_UNIT;
                     }
@@ -381,20 +402,31 @@ __global__ void __launch_bounds__(T) k_symbolic(CscView A, ExpandBuffers b, int6
                 }
                 if (tid == T - 1) sh->upre[SYM_BATCH] = units;
                 __syncthreads();
-                int s = 0;
-                for (int un = warp; un < units; un += NW) {
-                    while (sh->upre[s + 1] <= un) ++s;  // ends: upre[SYM_BATCH] = units > un
-                    const int p0 = (un - sh->upre[s]) * SYM_UNIT;
-                    const int rem = sh->cnt[s] - p0 - lane;
-                    const int32_t* rows = A.rowidx + sh->first[s] + p0 + lane;
-                    int off[SYM_UNIT / 32];
+                auto mark = [&](auto read_first) {
+                    int s = 0;
+                    for (int un = warp; un < units; un += NW) {
+                        while (sh->upre[s + 1] <= un) ++s;  // ends: upre[SYM_BATCH] = units > un
+                        const int p0 = (un - sh->upre[s]) * SYM_UNIT;
+                        const int rem = sh->cnt[s] - p0 - lane;
+                        const int32_t* rows = A.rowidx + sh->first[s] + p0 + lane;
+                        int off[SYM_UNIT / 32];
 #pragma unroll
-                    for (int c = 0; c < SYM_UNIT / 32; ++c)
-                        off[c] = 32 * c < rem ? __ldg(rows + 32 * c) - r0 : -1;
+                        for (int c = 0; c < SYM_UNIT / 32; ++c)
+                            off[c] = 32 * c < rem ? __ldg(rows + 32 * c) - r0 : -1;
 #pragma unroll
-                    for (int c = 0; c < SYM_UNIT / 32; ++c)
-                        if (off[c] >= 0) atomicOr(bm + (off[c] >> 5), 1u << (off[c] & 31));
-                }
+                        for (int c = 0; c < SYM_UNIT / 32; ++c) {
+                            uint32_t* w = bm + (off[c] >> 5);
+                            const uint32_t bit = 1u << (off[c] & 31);
+                            if (off[c] >= 0 &&
+                                !(decltype(read_first)::value && (*reinterpret_cast<volatile uint32_t*>(w) & bit)))
+                                atomicOr(w, bit);
+                        }
+                    }
+                };
+                if ((int64_t)units * SYM_UNIT >= (int64_t)SYM_TEST * (r1 - r0))
+                    mark(std::true_type{});
+                else
+                    mark(std::false_type{});
                 __syncthreads();
             }
             const int n4 = (r1 - r0 + 127) >> 7;  // the bitmap's words in fours
@@ -417,35 +449,41 @@ __global__ void __launch_bounds__(T) k_symbolic(CscView A, ExpandBuffers b, int6
 
 static size_t symbolic_smem(int words) { return (size_t)words * 4 + sizeof(SymShared); }
 
-// The dynamic shared-memory limit is a per-device attribute of the kernel:
-// it is set on the current device before every launch.
+// CTAs of the grid: as many as stay resident, from the limits on threads and
+// shared memory alone (more would only find the work taken; asking the runtime
+// took 3 us a call, of 66 for 500 vertices).
 template <int T>
-static int symbolic_occupancy(int words, int num_sms) {
-    cudaFuncSetAttribute(k_symbolic<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)symbolic_smem(words));
-    int occ = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_symbolic<T>, T, symbolic_smem(words));
-    return (occ < 1 ? 1 : occ) * num_sms;
+static int symbolic_ctas(int words, int num_sms) {
+    const int fit = (int)((size_t)228 * 1024 / (symbolic_smem(words) + 1024));
+    const int per_sm = fit < 2048 / T ? fit : 2048 / T;
+    return (per_sm < 1 ? 1 : per_sm) * num_sms;
 }
 
 // CTAs that the cursor scratch has to serve (several windows: the full bitmap)
-int symbolic_grid(int num_sms) { return symbolic_occupancy<512>(SYM_WORDS, num_sms); }
+int symbolic_grid(int num_sms) { return symbolic_ctas<512>(SYM_WORDS, num_sms); }
+
+template <int T>
+static void symbolic_launch(const CscView& A, const ExpandBuffers& b, int64_t* nnz_out, int words, int num_sms,
+                            int grid_cap, cudaStream_t s) {
+    const size_t smem = symbolic_smem(words);
+    if (smem > 48 * 1024)  // a per-device attribute: set on the current device before every launch
+        cudaFuncSetAttribute(k_symbolic<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    int grid = symbolic_ctas<T>(words, num_sms);
+    if (A.n > SYM_WORDS * 32 && grid > grid_cap) grid = grid_cap;
+    if ((int64_t)grid > A.n) grid = A.n;
+    k_symbolic<T><<<grid, T, smem, s>>>(A, b, nnz_out, words);
+}
 
 void launch_symbolic(const CscView& A, const ExpandBuffers& b, int64_t* nnz_out, int num_sms,
                      int grid_cap, cudaStream_t s, bool fresh) {
     if (A.n == 0) return;
     int words = (int)(((int64_t)A.n + 127) / 128 * 4);
     if (words > SYM_WORDS) words = SYM_WORDS;
-    // a short bitmap: more columns at once beat more warps on one
-    const bool small = A.n <= SYM_WORDS;
-    int grid = small ? symbolic_occupancy<128>(words, num_sms) : symbolic_occupancy<512>(words, num_sms);
-    if (A.n > SYM_WORDS * 32 && grid > grid_cap) grid = grid_cap;
-    if ((int64_t)grid > A.n) grid = A.n;
     if (!fresh) cudaMemsetAsync(&b.ctr->work_ctr, 0, sizeof(int), s);
-    if (small)
-        k_symbolic<128><<<grid, 128, symbolic_smem(words), s>>>(A, b, nnz_out, words);
+    if (A.n <= SYM_SMALL_N)
+        symbolic_launch<256>(A, b, nnz_out, words, num_sms, grid_cap, s);
     else
-        k_symbolic<512><<<grid, 512, symbolic_smem(words), s>>>(A, b, nnz_out, words);
+        symbolic_launch<512>(A, b, nnz_out, words, num_sms, grid_cap, s);
     count_launches(1);
 }
 

@@ -230,3 +230,10 @@ def test_walked_sources_equal_buckets(ctx, n, d, budget, mask, scale):
             ctx.set_option(o, v)
     assert ch == ch_ref and torch.equal(out.colptr, ref.colptr) and torch.equal(out.rowidx, ref.rowidx)
     assert torch.equal(out.val.view(torch.int32), ref.val.view(torch.int32))
+
+
+# columns on both sides of the rule that reads a bit before it is set (16 products per row of the
+# window, counted in units of 128), several windows of batches on both sides of it, and graphs on both sides of the small CTAs' line
+@pytest.mark.parametrize("n,d", [(1500, 12), (1500, 150), (1500, 900), (16384, 30), (16385, 30), (17000, 700), (530000, 3)])
+def test_symbolic_dense_columns(ctx, n, d):
+    test_symbolic_shapes(ctx, n, d)
