@@ -28,7 +28,7 @@ struct DevCounters {
     int max_deg;
     int max_span;
     unsigned err;                    // bit flags (ERR_*)
-    int pad;
+    int cc_left;                     // components: a first link was left to the last step
     int bin_cnt[NBUCKET];
     int bin_off[NBUCKET + 1];
     int bin_fill[NBUCKET];

@@ -237,3 +237,35 @@ def test_walked_sources_equal_buckets(ctx, n, d, budget, mask, scale):
 @pytest.mark.parametrize("n,d", [(1500, 12), (1500, 150), (1500, 900), (16384, 30), (16385, 30), (17000, 700), (530000, 3)])
 def test_symbolic_dense_columns(ctx, n, d):
     test_symbolic_shapes(ctx, n, d)
+
+
+def _graph(n, col, row):
+    from paper_2002_10083_gb300 import mcl
+    key = torch.unique(col * n + row)
+    col, row = key // n, key % n
+    colptr = torch.zeros(n + 1, dtype=torch.int64)
+    colptr[1:] = torch.cumsum(torch.bincount(col, minlength=n), 0)
+    return mcl.DeviceCSC(n, colptr.cuda(), row.int().cuda(), torch.ones(key.numel(), device="cuda"))
+
+
+# long paths in both directions and in random order, bands, trees, rows shared by all columns, empty
+# columns; sizes on both sides of the rules that link every entry at once
+@pytest.mark.parametrize("n", [1, 7, 8192, 8193, 70000, 1200000])
+@pytest.mark.parametrize("kind", ["up", "down", "perm", "band", "tree", "pairs", "one row", "one column", "blocks"])
+def test_components_of_long_and_shallow_graphs(ctx, n, kind):
+    import scipy.sparse as sp
+    from scipy.sparse.csgraph import connected_components
+    v, g = torch.arange(n), torch.Generator().manual_seed(n)
+    perm = torch.randperm(n, generator=g)
+    col, row = {"up": (v, (v + 1) % n), "down": (v, (v - 1) % n), "perm": (perm, perm.roll(1)),
+                "band": (v.repeat(5), torch.cat([(v + o).clamp(0, n - 1) for o in range(-2, 3)])),
+                "tree": (v, (torch.rand(n, generator=g) * v).long()), "pairs": (v, (v ^ 1).clamp(max=n - 1)),
+                "one row": (v[::3], v[::3] * 0 + n // 2), "one column": (v[::3] * 0 + n // 2, v[::3]),
+                "blocks": (v.repeat(4), torch.cat([v // 97 * 97 + (v * m) % 97 for m in (0, 5, 11, 13)]).clamp(max=n - 1))}[kind]
+    A = _graph(n, col, row)
+    label = ctx.components(A).cpu().numpy()
+    S = sp.csc_matrix((np.ones(A.nnz), A.rowidx.cpu().numpy(), A.colptr.cpu().numpy()), shape=(n, n))
+    k, ref = connected_components(S, directed=False)
+    first = np.full(k, n, np.int64)
+    np.minimum.at(first, ref, np.arange(n))
+    assert (label == first[ref]).all()
