@@ -21,8 +21,7 @@ struct WinShared {
     double red;    // result of a mass
     double sum4[2][4];  // partial sums of the warps
     float max4[4];
-    double inv;         // 1 / sum, and as two FP32 numbers
-    float inv_hi, inv_lo;
+    Quotient quo;       // by the sum
     double chaos;
     int flag;
 };
@@ -560,8 +559,7 @@ __device__ void finish_column(uint64_t* top, int ntop, int topcap, const PrunePa
     // U = sum u and the sum of u^2 over the kept u = v^r, in an order that does not depend on
     // the block size: thread t of the first SUM_T takes i = t, t + SUM_T, ..., a warp's lanes
     // are added by a fixed butterfly and the warps' sums in turn (warps beyond m add 0).
-    // a = u / U is written as u (hi + lo), 1 / U as two FP32 numbers: one rounding of a product
-    // exact to 2^-48.
+    // a = u (1 / U) in FP64, rounded to FP32.
     const float rr = pp.r;
     if (!pp.inflate) {
         for (int i = tid; i < m; i += T) {
@@ -602,12 +600,10 @@ __device__ void finish_column(uint64_t* top, int ntop, int topcap, const PrunePa
         const double U = ((sh->sum4[0][0] + sh->sum4[0][1]) + sh->sum4[0][2]) + sh->sum4[0][3];
         const double U2 = ((sh->sum4[1][0] + sh->sum4[1][1]) + sh->sum4[1][2]) + sh->sum4[1][3];
         const float mu = fmaxf(fmaxf(sh->max4[0], sh->max4[1]), fmaxf(sh->max4[2], sh->max4[3]));
-        const double inv = U > 0.0 ? 1.0 / U : 0.0;
-        const float hi = (float)inv;
-        sh->inv = inv;
-        sh->inv_hi = hi;
-        sh->inv_lo = (float)(inv - (double)hi);
-        sh->flag = U > 1e-25 && U < 1e25;
+        Quotient quo;
+        quo.init(U);
+        sh->quo = quo;
+        const double inv = quo.inv;
         // max a - sum a^2; the largest u gives the largest a
         const double ch = (double)mu * inv - (U2 * inv) * inv;
         sh->chaos = ch < 0.0 ? 0.0 : ch;
@@ -615,21 +611,14 @@ __device__ void finish_column(uint64_t* top, int ntop, int topcap, const PrunePa
         *chaos_out = sh->chaos;
     }
     __syncthreads();
-    if (sh->flag) {
-        const float hi = sh->inv_hi, lo = sh->inv_lo;
-        for (int i = tid; i < m; i += T) {
-            const uint64_t x = top[i];
-            const float u = inflate_value(key_val(x), rr);
-            out_row[i] = key_row(x);
-            out_val[i] = fmaf(u, hi, __fmul_rn(u, lo));
-        }
-    } else {
-        const double inv = sh->inv;
-        for (int i = tid; i < m; i += T) {
-            const uint64_t x = top[i];
-            out_row[i] = key_row(x);
-            out_val[i] = (float)((double)inflate_value(key_val(x), rr) * inv);
-        }
+    const Quotient quo = sh->quo;
+    for (int i = tid; i < m; i += T) {
+        const uint64_t x = top[i];
+        const float u = inflate_value(key_val(x), rr);
+        float a;
+        if (!quo.plain() || !quo.quick(u, &a)) a = (float)((double)u * quo.inv);
+        out_row[i] = key_row(x);
+        out_val[i] = a;
     }
     __syncthreads();
 }

@@ -381,6 +381,32 @@ __device__ __forceinline__ unsigned long long fixed_of(float v, int f) {
     return fx.qv(v);
 }
 
+// The quotients u / s of a column as FP64 gives them, rounded to FP32, mostly
+// without FP64 instructions (2 lanes per clock and SM).  1 / s is hi plus a rest
+// that lies between lo[0] and lo[1], 2^-46 hi to each side.  That covers the
+// roundings of the rest's product (2^-48), of the rest (2^-49), of its ends
+// (2^-49) and of the FP64 quotient (2^-52): where both ends round to the same
+// number it is the quotient.  About one entry in 2^21, and those too small for
+// the rest's product to be a normal number, take FP64.
+struct Quotient {
+    double inv;
+    float hi, lo[2];
+    __device__ __forceinline__ void init(double s) {
+        inv = s > 0.0 ? 1.0 / s : 0.0;
+        hi = (float)inv;
+        const float rest = (float)(inv - (double)hi);
+        lo[0] = __fsub_rn(rest, __fmul_rn(hi, 0x1p-46f));
+        lo[1] = __fadd_rn(rest, __fmul_rn(hi, 0x1p-46f));
+    }
+    // whether hi and the rest stay in FP32's range
+    __device__ __forceinline__ bool plain() const { return hi > 1e-25f && hi < 1e25f; }
+    // true: *a is u / s
+    __device__ __forceinline__ bool quick(float u, float* a) const {
+        *a = fmaf(u, hi, __fmul_rn(u, lo[0]));
+        return *a > 1e-30f && *a == fmaf(u, hi, __fmul_rn(u, lo[1]));
+    }
+};
+
 // Inflation (Alg. 1, Hadamard power r) of one FP32 value.
 __device__ __forceinline__ float inflate_value(float v, float r) {
     if (r == 2.0f) return v * v;

@@ -912,11 +912,10 @@ void launch_finalize_stats(int32_t n, const ExpandBuffers& b, cudaStream_t s) {
     count_launches(1);
 }
 
-// Warp per column: v <- v^r / sum v^r (FP32 power, FP64 sum).  The quotient is
-// u (hi + lo) with 1 / sum as two FP32 numbers, one rounding of a product that
-// is exact to 2^-48: an FP64 division per entry ran at the FP64 pipe's 2 lanes
-// per clock and SM (351 us for 13.5M entries; 8 bytes of traffic each take 32).
-// Sums whose reciprocal or whose terms leave FP32's range divide in FP64.
+// Warp per column: v <- v^r / sum v^r (FP32 power, FP64 sum and quotient).  An
+// FP64 division per entry ran at the FP64 pipe's 2 lanes per clock and SM (351 us
+// for 13.5M entries; 8 bytes of traffic each take 32): Quotient leaves it to the
+// few entries that need it.
 __global__ void k_inflate_normalize(int32_t n, const int64_t* colptr, float* val, float r) {
     const int lane = threadIdx.x & 31;
     const int64_t gw = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -927,13 +926,15 @@ __global__ void k_inflate_normalize(int32_t n, const int64_t* colptr, float* val
 #pragma unroll 4
         for (int64_t p = cb + lane; p < ce; p += 32) s += float_to_double(inflate_value(val[p], r));
         s = warp_sum(s);
-        if (s > 1e-25 && s < 1e25) {
-            const double inv = 1.0 / s;
-            const float hi = (float)inv, lo = (float)(inv - (double)hi);
+        Quotient quo;
+        quo.init(s);
+        if (quo.plain()) {
 #pragma unroll 4
             for (int64_t p = cb + lane; p < ce; p += 32) {
                 const float u = inflate_value(val[p], r);
-                val[p] = fmaf(u, hi, __fmul_rn(u, lo));
+                float a;
+                if (!quo.quick(u, &a)) a = (float)((double)u / s);
+                val[p] = a;
             }
         } else {
             for (int64_t p = cb + lane; p < ce; p += 32) {

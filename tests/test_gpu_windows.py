@@ -269,3 +269,47 @@ def test_components_of_long_and_shallow_graphs(ctx, n, kind):
     first = np.full(k, n, np.int64)
     np.minimum.at(first, ref, np.arange(n))
     assert (label == first[ref]).all()
+
+
+def _near_ties():
+    """FP32 numbers (u, w) with u / (u + w) within 2^-45 of the middle of two FP32 numbers: for odd
+    s < 2^24 and small odd d, u = (s t - d) / 2^25 with t = d / s mod 2^25, so u / s = (t - d / s) / 2^25."""
+    rng = np.random.default_rng(11)
+    out = []
+    for s in rng.integers(1 << 22, 1 << 23, 4000) * 2 + 1:
+        for d in (-3, -1, 1, 3):
+            t = d * pow(int(s), -1, 1 << 25) % (1 << 25)
+            if t >= 1 << 24 and t & 1:
+                u = (int(s) * t - d) >> 25
+                out.append((u, int(s) - u))
+    return np.array(out, np.float64)
+
+
+def test_normalised_values_are_fp64_quotients(ctx):
+    """v / sum in FP64, rounded once to FP32, where that is hardest: near the middle of two FP32
+    numbers (sums of whole numbers are exact in any order)."""
+    from paper_2002_10083_gb300 import mcl
+    uw = _near_ties()
+    m = len(uw)
+    assert m > 1000
+    want = torch.from_numpy((uw / uw.sum(1, keepdims=True)).astype(np.float32).ravel())
+    val = torch.from_numpy(uw.astype(np.float32).ravel()).cuda()
+    M = mcl.DeviceCSC(m, torch.arange(m + 1).cuda() * 2, torch.tensor([0, 1]).int().repeat(m).cuda(), val.clone())
+    ctx.inflate_normalize(M, 1.0)
+    assert torch.equal(M.val.cpu().view(torch.int32), want.view(torch.int32))
+    # columns 2 .. m + 1 hold the pairs; column m + 2 + i of A A is column 2 + i
+    n = 2 * m + 2
+    colptr = torch.cat([torch.arange(3), 2 + 2 * torch.arange(1, m + 1), 2 + 2 * m + torch.arange(1, m + 1)])
+    row = torch.cat([torch.tensor([0, 1]), torch.tensor([0, 1]).repeat(m), 2 + torch.arange(m)])
+    one = torch.ones(1, device="cuda")
+    A = mcl.DeviceCSC(n, colptr.cuda(), row.int().cuda(), torch.cat([one.repeat(2), val, one.repeat(m)]))
+    out, _ = ctx.expand(A, mcl.Params(threshold=0.0, select_k=8, recover_pct=0.9, inflation=1.0))
+    assert int(out.colptr[n]) == 2 + 4 * m
+    assert torch.equal(out.val[2 + 2 * m:].cpu().view(torch.int32), want.view(torch.int32))
+    # results and sums at the ends of FP32's range
+    for scale in (1e-37, 1e-32, 1e-20, 1e20, 1e30):
+        v = torch.tensor([1.0, 3.0, 7e-7, 1e-12, 3e-25]) * scale
+        M = mcl.DeviceCSC(5, torch.tensor([0, 5, 5, 5, 5, 5]).cuda(), torch.arange(5).int().cuda(), v.cuda())
+        ctx.inflate_normalize(M, 1.0)
+        d = v.double()
+        assert torch.equal(M.val.cpu(), (d / d.sum()).float())
