@@ -71,8 +71,9 @@ constexpr int CC_FIRST = 2;
 // 1.5 times as long on shallow trees; 64: 0.67 instead of 0.45 on a band of five.
 constexpr int CC_FIRST_WALK = 16;
 // Few entries, or few per column (a converged matrix), are linked at once: two
-// launches less (20,000 columns of one entry: 51 us against 60).
-constexpr int64_t CC_FEW = 8192, CC_FEW_SPARSE = 65536;
+// launches less (300 columns of 30 entries: 52 us against 60; 1,000 of 16: 77
+// against 70; 20,000 of one: 51 against 60).
+constexpr int64_t CC_FEW = 12288, CC_FEW_SPARSE = 65536;
 
 // thread per column: link its first CC_FIRST entries and its last
 __global__ void k_cc_first(CscView A, int* parent, DevCounters* ctr) {
