@@ -104,7 +104,8 @@ typedef struct {
     int64_t range_splits;     /* row windows cut because their entries exceeded the capacity */
     double chaos;             /* max_j chaos_j */
     float ms_colstats, ms_estimate, ms_bin, ms_numeric, ms_compact, ms_chaos, ms_total;
-    int32_t bins_used;
+    int32_t bins_used;        /* configurations that MCL_OPT_CONF_MASK allows, summed over the
+                                 column batches */
     int32_t iterations;
     int32_t phases;           /* column batches of the last mcl_expand */
     int32_t graph_replays;    /* iterations of the last batched mcl_run replayed as CUDA graphs */

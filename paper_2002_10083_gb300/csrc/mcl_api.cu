@@ -520,8 +520,8 @@ static mcl_status expand_impl(mcl_ctx* c, const mcl_csc* A, const mcl_params* pr
                 launch_numeric(q, Av, pp, bq, cols < g ? cols : g,
                                walks_sources(c, bq, q, (int64_t)c->hctr->max_flops), s);
             }
-            ++used;
         }
+        used += (c->conf_mask & 1) + ((c->conf_mask >> 1) & 1);
         return check_launch(c, "numeric");
     };
     int64_t* colptr_out = nullptr;

@@ -313,3 +313,16 @@ def test_normalised_values_are_fp64_quotients(ctx):
         ctx.inflate_normalize(M, 1.0)
         d = v.double()
         assert torch.equal(M.val.cpu(), (d / d.sum()).float())
+
+
+def test_bins_used_counts_the_mask(ctx):
+    from paper_2002_10083_gb300 import mcl
+    prm = mcl.Params(threshold=1e-4, select_k=50, recover_pct=0.9, inflation=2.0)
+    try:
+        for A in (_random(500, 5, seed=1), _random(9000, 60, seed=2)):
+            for mask, bins in ((1, 1), (2, 1), (3, 2)):
+                ctx.set_option(mcl.OPT_CONF_MASK, mask)
+                ctx.expand(A, prm)
+                assert ctx.stats()["bins_used"] == bins
+    finally:
+        ctx.set_option(mcl.OPT_CONF_MASK, 3)
