@@ -14,7 +14,6 @@
 namespace mcl {
 
 constexpr unsigned FULL = 0xffffffffu;
-constexpr uint64_t EMPTY_SLOT = 0x00000000FFFFFFFFull;  // key -1, value +0.0f
 
 __device__ __forceinline__ uint64_t make_key(float v, int row) {
     return ((uint64_t)__float_as_uint(v) << 32) | (uint32_t)(0x7FFFFFFF - row);
@@ -60,11 +59,8 @@ struct BlockScratch {
     uint64_t sel_prefix;
     int sel_need;
     int sel_done;
-    double sel_target;
     int sel_found;
     int sel_above;
-    int cnt;
-    int pad;
 };
 
 // Sums of up to four doubles and four integers over the block (two barriers).
@@ -97,22 +93,6 @@ __device__ __forceinline__ void block_sum(double* dv, int nd, long long* qv, int
     __syncthreads();
     for (int a = 0; a < nd; ++a) dv[a] = bs->d[a][32];
     for (int a = 0; a < nq; ++a) qv[a] = bs->q[a][32];
-}
-
-template <int T>
-__device__ __forceinline__ double block_max_d(double x, BlockScratch* bs) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    constexpr int NW = T / 32;
-    x = warp_max(x);
-    if (lane == 0) bs->d[3][warp] = x;
-    __syncthreads();
-    if (warp == 0) {
-        double y = lane < NW ? bs->d[3][lane] : -1.0e300;
-        y = warp_max(y);
-        if (lane == 0) bs->d[3][32] = y;
-    }
-    __syncthreads();
-    return bs->d[3][32];
 }
 
 // Element i of the concatenation A[0..na) ++ B[0..nb).
@@ -234,7 +214,6 @@ __device__ int block_select_mass(const uint64_t* A, int na, double target, uint6
             } else if (lane == __ffs(hm) - 1) {
                 int d = 255 - 8 * lane - hitq;
                 bs->sel_prefix = prefix | ((uint64_t)d << shift);
-                bs->sel_target = (double)(need - hb);
                 bs->sel_above = above + hbc;
                 bs->sel_need = c[hitq];
                 bs->sel_found = 1;
@@ -412,12 +391,6 @@ __device__ __forceinline__ float inflate_value(float v, float r) {
     if (r == 2.0f) return v * v;
     if (r == 1.0f) return v;
     return powf(v, r);
-}
-
-__host__ __device__ __forceinline__ int next_pow2(int x) {
-    int p = 1;
-    while (p < x) p <<= 1;
-    return p;
 }
 
 }  // namespace mcl

@@ -18,7 +18,7 @@ constexpr int NBUCKET = NCONF * NZ;
 // device-side counters (one small block of memory per context)
 struct DevCounters {
     unsigned long long misses;       // columns whose nnz exceeded the estimate
-    unsigned long long splits;       // range overflows resolved by halving
+    unsigned long long splits;       // windows that overflowed and were cut
     unsigned long long flops;        // sum of flops_j
     unsigned long long nnz_b;        // sum of nnz(B_*j)
     unsigned long long chaos_bits;   // max chaos_j as ordered bits (>= 0)
