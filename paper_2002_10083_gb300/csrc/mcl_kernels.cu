@@ -338,6 +338,11 @@ __global__ void __launch_bounds__(T) k_symbolic(CscView A, ExpandBuffers b, int6
             __syncthreads();
             continue;
         }
+        if (d == 1) {  // the rows of one source
+            if (tid == 0) nnz_out[j] = b.flops[j];
+            __syncthreads();
+            continue;
+        }
         long long cnt = 0;
         // a thread lists the same sources in every window, if they are one batch (the small
         // CTAs have one window)

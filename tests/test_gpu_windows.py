@@ -326,3 +326,17 @@ def test_bins_used_counts_the_mask(ctx):
                 assert ctx.stats()["bins_used"] == bins
     finally:
         ctx.set_option(mcl.OPT_CONF_MASK, 3)
+
+
+# columns of no entry, of one, and of more side by side
+@pytest.mark.parametrize("n", [40, 20000, 600000])
+def test_symbolic_columns_of_one_entry(ctx, n):
+    v, g = torch.arange(n), torch.Generator().manual_seed(n)
+    A = _graph(n, torch.cat([v[v % 5 > 0], v[v % 3 > 0]]),
+               torch.randint(n, (int((v % 5 > 0).sum() + (v % 3 > 0).sum()),), generator=g))
+    import scipy.sparse as sp
+    P = sp.csc_matrix((np.ones(A.nnz), A.rowidx.cpu().numpy(), A.colptr.cpu().numpy()), shape=(n, n))
+    B = P @ P
+    flops, nnz = ctx.symbolic(A)
+    assert (nnz.cpu().numpy() == np.diff(B.indptr)).all()
+    assert (flops.cpu().numpy() == np.asarray(B.sum(axis=0)).ravel()).all()
