@@ -461,8 +461,10 @@ __device__ void finish_column(uint64_t* top, int ntop, int topcap, const PrunePa
                               unsigned* bins, WinShared* sh, DevCounters* ctr, int row_lo, int row_span,
                               unsigned* rscratch, int* mstar_out, double* chaos_out) {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    // FP64 work is one warp's, not every warp's: its instructions take 16 clocks
-    // of the SM each, and a column of a few entries took 23k clocks in here
+    // FP64 sums, quotients and the test of the mass at or above theta are one
+    // warp's, not every warp's: their instructions take 16 clocks of the SM each,
+    // and a column of a few entries took 23k clocks in here (the recovery's
+    // targets, where that test fails, are computed by every warp)
     const int q = (int)(Tt < (long long)pp.K ? Tt : (long long)pp.K);
     bool theta_cut = false;  // the entries >= theta are at most K and carry the mass to recover
     if (q < pp.Krec && Tt <= pp.K) {

@@ -4,7 +4,10 @@
 // Two CTAs share an SM, each with a table of 10,240 rows, so that one's scans
 // and selects overlap the other's inserts (one CTA with 24,576 rows: the same
 // on 40k-row columns, 5-30% slower on shorter or sparser ones, whose time goes
-// into the phases between barriers).
+// into the phases between barriers).  The candidate buffer grows with K: above
+// about 1,200 one CTA fits an SM (iteration 2 of a 30k-vertex power-law graph
+// with K = 1,100, 1,500 and 4,096: 28.9, 40.1 and 41.5 ms; 72.7, 82.9 and 112 ms
+// with hashed windows).
 //
 //   insert:  the products of the window's rows, from per-source cursors over
 //            the sorted rows of A (one or more windows: a source is visited
