@@ -288,11 +288,22 @@ __global__ void __launch_bounds__(SH::T, SH::MINB) k_rank_acc(RankArgs a) {
             } else {
                 // ---- positions: exclusive prefix counts of the bitmap words ----
                 int wtot = 0;
-                for (int w0 = 0; w0 < nwords; w0 += RA_T) {
-                    const int w = w0 + tid;
-                    int tot;
-                    const int at = ra_scan<RA_T>(w < nwords ? __popc(bm[w]) : 0, &tot, sh->wsm);
-                    if (w < nwords) wpre[w] = wtot + at;
+                // Four words per thread and scan: with one, the 32 scans of a wide bitmap were most
+                // of a sparse column (1M vertices of 8 entries, 2 stages: 696 ms, now 444).
+                for (int w0 = 0; w0 < nwords; w0 += RA_T * 4) {
+                    const int w = w0 + tid * 4;
+                    int c[4], sum = 0, tot;
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) {
+                        c[q] = w + q < nwords ? __popc(bm[w + q]) : 0;
+                        sum += c[q];
+                    }
+                    int at = wtot + ra_scan<RA_T>(sum, &tot, sh->wsm);
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) {
+                        if (w + q < nwords) wpre[w + q] = at;
+                        at += c[q];
+                    }
                     wtot += tot;
                 }
                 __syncthreads();

@@ -340,3 +340,9 @@ def test_symbolic_columns_of_one_entry(ctx, n):
     flops, nnz = ctx.symbolic(A)
     assert (nnz.cpu().numpy() == np.diff(B.indptr)).all()
     assert (flops.cpu().numpy() == np.asarray(B.sum(axis=0)).ravel()).all()
+
+
+# sparse columns over bitmaps whose words are not a multiple of four, or of four per thread
+@pytest.mark.parametrize("n,d,ns", [(33, 3, 2), (97, 4, 3), (32767, 4, 2), (65600, 4, 2), (131073, 5, 3), (524289, 3, 2), (1000003, 3, 2)])
+def test_split_of_sparse_columns(ctx, n, d, ns):
+    test_split_shapes_equal_one_pass(ctx, n, d, ns)
