@@ -16,17 +16,17 @@
 // the columns of the partial products being merged) in windows of rows; a
 // shared bitmap marks the rows present (count mode: their number) and a prefix
 // count of the bitmap gives each row its position in the output column.  Fill
-// mode adds the values at their positions in a shared array of 64-bit sums
-// (several passes over the sources where the window has more entries than the
-// array) and writes the window's entries out in order, so the output comes out
-// sorted and its sums do not depend on the order of the additions.
+// mode adds the values at their positions in a shared array of 64-bit sums (or
+// in the output itself, where the window has more entries than the array) and
+// writes the window's entries out in order, so the output comes out sorted and
+// its sums do not depend on the order of the additions.
 //
 // The sources are cut into units of 128 entries that the warps take in turn:
 // a merge has 2 to 5 sources and a stage of a sparse column a handful, which
 // would leave most warps idle with a source per warp.  20k-vertex power-law
 // graph (3.8e8 products) in 8 stages: 96 ms with a source per warp and every
 // product a global atomic, 17 ms with units and shared sums, 15 ms with the
-// small CTAs.
+// small CTAs, 11.1 ms without passes over the sources for parts of a window.
 #include <climits>
 #include <cstdint>
 
@@ -64,7 +64,9 @@ constexpr int RA_UNIT = 128;   // entries a warp takes at once
 // Shapes by the rows of the output: threads, bitmap words (32 rows each), sums,
 // CTAs per SM.  A column's steps are short and separated by barriers, so small
 // outputs take many small CTAs (16.4 -> 15.2 ms against RankSmall at 20k rows);
-// a wider bitmap leaves room for fewer.
+// a wider bitmap leaves room for fewer.  With a source per warp and every product
+// a global atomic, power-law graphs in 4 stages: 60k rows 170 ms (RankSmall: 26.9),
+// 400k rows 1,793 ms (RankLarge: 401).
 template <int T_, int WORDS_, int CAP_, int MINB_>
 struct RankShape {
     static constexpr int T = T_, WORDS = WORDS_, CAP = CAP_, MINB = MINB_;
@@ -72,9 +74,10 @@ struct RankShape {
 using RankTiny = RankShape<256, 1024, 4096, 5>;
 using RankSmall = RankShape<512, 4096, 8192, 2>;
 using RankLarge = RankShape<512, 16384, 8192, 1>;
-// More passes than this over a window's sources: add in global memory instead
-// (RankTiny never does: eight passes hold all of its 32k rows).
-constexpr int RA_PASSES = 8;
+// A window with more entries than the array of sums holds adds in global memory
+// (the L2).  Walking its sources again for every arrayful was no better anywhere:
+// 100k vertices of 400 entries, 2 stages: 557 ms with up to eight passes, 390 with
+// two, 389 with one; 12k of 130, 4 stages: 6.6 and 5.9 ms; 140k of 100: 120 and 116.
 
 template <int T>
 struct RankShared {
@@ -339,27 +342,20 @@ __global__ void __launch_bounds__(SH::T, SH::MINB) k_rank_acc(RankArgs a) {
                             }
                     });
                 };
-                const int npass = (wtot + CAP - 1) / CAP;
-                if (npass <= RA_PASSES) {
-                    for (int e0 = 0; e0 < wtot; e0 += CAP) {
-                        products([&](int rank, unsigned long long q) {
-                            const unsigned e = (unsigned)(rank - e0);
-                            if (e < (unsigned)CAP) {
-                                const unsigned ql = (unsigned)q;
-                                const unsigned old = atomicAdd(lo32 + e, ql);
-                                const unsigned qh = (unsigned)(q >> 32) + (old + ql < old ? 1u : 0u);
-                                if (qh) atomicAdd(hi32 + e, qh);
-                            }
-                        });
-                        const int m = min(CAP, wtot - e0);
-                        for (int e = tid; e < m; e += RA_T) {
-                            a.val_out[obase + e0 + e] = ((unsigned long long)hi32[e] << 32) | lo32[e];
-                            lo32[e] = 0u;
-                            hi32[e] = 0u;
-                        }
-                        __syncthreads();
+                if (wtot <= CAP) {
+                    products([&](int rank, unsigned long long q) {
+                        const unsigned ql = (unsigned)q;
+                        const unsigned old = atomicAdd(lo32 + rank, ql);
+                        const unsigned qh = (unsigned)(q >> 32) + (old + ql < old ? 1u : 0u);
+                        if (qh) atomicAdd(hi32 + rank, qh);
+                    });
+                    for (int e = tid; e < wtot; e += RA_T) {
+                        a.val_out[obase + e] = ((unsigned long long)hi32[e] << 32) | lo32[e];
+                        lo32[e] = 0u;
+                        hi32[e] = 0u;
                     }
-                } else {  // more entries than a few passes hold: 64-bit atomics in global memory
+                    __syncthreads();
+                } else {  // 64-bit atomics in global memory
                     for (int e = tid; e < wtot; e += RA_T) a.val_out[obase + e] = 0ull;
                     __syncthreads();
                     products([&](int rank, unsigned long long q) { atomicAdd(a.val_out + obase + rank, q); });
