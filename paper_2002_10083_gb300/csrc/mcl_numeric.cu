@@ -71,8 +71,13 @@ constexpr int PMAX = 64;          // probe run that marks a hashed window as ove
 // launches where columns can be many windows without buckets (WALK): its
 // registers cost the others 1% (1M vertices: 505 -> 511 ms).
 constexpr int LANE_MAX = 16;
-constexpr int FLAT_SOURCES = 256; // a column of so few sources and products in one window:
-constexpr int FLAT_PRODUCTS = 65536;  // every lane finds its own products' sources
+// A column of so few sources and products in one window: every lane finds its own
+// products' sources, with a search each, instead of a warp walking one source at a
+// time.  300k vertices of 8 entries: 9.6 ms with the walk, 8.6 with the search;
+// 1,000 of 250 (62,500 products a column): 0.42 ms with the walk, 0.63 with the
+// search.  With the line at 65,536, 16,384, 8,192, 4,096 and 2,048 iteration 2 of
+// the 2,000-vertex planted partition takes 0.43, 0.43, 0.39, 0.37 and 0.37 ms.
+constexpr int FLAT_SOURCES = 256, FLAT_PRODUCTS = 4096;
 
 struct ExpandShared {
     WinShared w;

@@ -346,3 +346,16 @@ def test_symbolic_columns_of_one_entry(ctx, n):
 @pytest.mark.parametrize("n,d,ns", [(33, 3, 2), (97, 4, 3), (32767, 4, 2), (65600, 4, 2), (131073, 5, 3), (524289, 3, 2), (1000003, 3, 2)])
 def test_split_of_sparse_columns(ctx, n, d, ns):
     test_split_shapes_equal_one_pass(ctx, n, d, ns)
+
+
+# columns of one window on both sides of the rules by which lanes search their products' sources (256
+# sources, 4,096 products), against the split form, whose kernel has no such rule
+@pytest.mark.parametrize("n,d", [(900, 64), (500, 66), (700, 252), (1500, 258), (3000, 40)])
+def test_searched_and_walked_products(ctx, n, d):
+    from paper_2002_10083_gb300 import mcl
+    A = _random(n, d, seed=n + d, zeros=True)
+    prm = mcl.Params(threshold=1e-4, select_k=120, recover_pct=0.9, inflation=2.0)
+    out, ch = ctx.expand(A, prm)
+    ref, ch_ref, _ = ctx.expand_split(A, prm, 2)
+    assert ch == ch_ref and torch.equal(out.colptr, ref.colptr) and torch.equal(out.rowidx, ref.rowidx)
+    assert torch.equal(out.val.view(torch.int32), ref.val.view(torch.int32))
